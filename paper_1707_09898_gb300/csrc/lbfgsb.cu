@@ -16,6 +16,7 @@
 #include <cstdint>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/topomag.h"
@@ -26,7 +27,12 @@ namespace {
 constexpr int MAXM = 16;  // 2m <= 32: one lane per column of W in the breakpoint scan
 constexpr int NT = 256;
 constexpr int WPB = NT / 32;
-constexpr int TILE = 2048;  // elements per block in compaction and radix sort (8 per thread)
+// Elements per block of the breakpoint pass and of its compaction (2 per thread): the pass
+// reads 2m columns per element, so its time is load latency times rounds per thread; at
+// 59,319 variables 2048 per block left 29 blocks on 152 SMs and took 24 us, 512 take 13 us.
+constexpr int TILE = 512;
+// Elements per block of a radix pass (4 per thread). 2048 at 59,319 keys: 29 blocks.
+constexpr int RTILE = 1024;
 constexpr double EPSMCH = 2.220446049250313e-16;
 constexpr double BIG = 1e10;
 
@@ -62,21 +68,13 @@ __device__ void block_sums(double (&v)[K], int nv, double* part) {
   }
 }
 
-__global__ void k_finish(const double* part, int nblk, int nv, double* out) {
-  for (int k = threadIdx.x; k < nv; k += blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nblk; b++) s += part[(long long)b * nv + k];
-    out[k] = s;
-  }
-}
-
 // min of (value, index) pairs: smaller value, then smaller index
 struct VI {
   double v;
   long long i;
 };
 __device__ __forceinline__ VI vimin(VI a, VI b) { return (b.v < a.v || (b.v == a.v && b.i < a.i)) ? b : a; }
-__device__ void block_min(VI x, VI* part) {
+__device__ void block_min_to(VI x, VI* out) {
   __shared__ VI sh[WPB];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int o = 16; o; o >>= 1) {
@@ -90,15 +88,36 @@ __device__ void block_min(VI x, VI* part) {
   if (threadIdx.x == 0) {
     VI r = sh[0];
     for (int i = 1; i < WPB; i++) r = vimin(r, sh[i]);
-    part[blockIdx.x] = r;
-  }
-}
-__global__ void k_finish_min(const VI* part, int nblk, VI* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    VI r = part[0];
-    for (int b = 1; b < nblk; b++) r = vimin(r, part[b]);
     *out = r;
   }
+}
+__device__ void block_min(VI x, VI* part) { block_min_to(x, part + blockIdx.x); }
+// Sums of nblk partials of nv values and, in the last block, the min of nblk_m pairs. The
+// results go straight to pinned host memory (no copy behind the kernel). A block takes
+// FV values; 32 threads per value add every 32nd partial and a fixed tree adds the 32, so
+// the order is the same on every run. (One thread per value over all partials was a chain
+// of dependent adds behind cache misses, 12 us for 240 partials, and the min in one thread
+// 20 us; both together now take 4.)
+constexpr int FV = NT / 32;
+__global__ void k_finish(const double* part, int nblk, int nv, double* out, const VI* mpart, int nblk_m, VI* mout) {
+  __shared__ double sh[32][FV];
+  if (mpart && blockIdx.x == gridDim.x - 1) {
+    VI r = mpart[0];
+    for (int b = threadIdx.x; b < nblk_m; b += NT) r = vimin(r, mpart[b]);
+    block_min_to(r, mout);
+    return;
+  }
+  const int v = threadIdx.x % FV, row = threadIdx.x / FV, k = blockIdx.x * FV + v;
+  double s = 0.0;
+  if (k < nv)
+    for (int b = row; b < nblk; b += 32) s += part[(long long)b * nv + k];
+  sh[row][v] = s;
+  __syncthreads();
+  for (int o = 16; o; o >>= 1) {
+    if (row < o) sh[row][v] += sh[row + o][v];
+    __syncthreads();
+  }
+  if (row == 0 && k < nv) out[k] = sh[0][v];
 }
 
 // ---- start: x = P(x0) --------------------------------------------------------
@@ -193,32 +212,62 @@ __global__ void k_bp(const double* __restrict__ x, const double* __restrict__ g,
   }
 }
 
-// exclusive scan of a (small) int array in one block; total in out[len]
-__global__ void k_scan_ex(int* a, long long len) {
-  __shared__ long long sh[1024];
-  const int T = blockDim.x;
-  const long long chunk = (len + T - 1) / T;
-  const long long b0 = threadIdx.x * chunk, b1 = min(len, b0 + chunk);
-  long long s = 0;
-  for (long long i = b0; i < b1; i++) s += a[i];
-  sh[threadIdx.x] = s;
+// exclusive prefix of x over the block's threads, and the block's total
+template <typename T>
+__device__ __forceinline__ T block_prefix(T x, T* shw, T& total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  T inc = x;
+  for (int o = 1; o < 32; o <<= 1) {
+    const T y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) shw[w] = inc;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    long long run = 0;
-    for (int k = 0; k < T; k++) {
-      const long long v = sh[k];
-      sh[k] = run;
-      run += v;
-    }
-    a[len] = (int)run;
+  T off = T(0);
+  total = T(0);
+  for (int k = 0; k < (int)blockDim.x / 32; k++) {
+    if (k < w) off += shw[k];
+    total += shw[k];
   }
   __syncthreads();
-  long long run = sh[threadIdx.x];
+  return off + (inc - x);
+}
+
+// exclusive scan of a (small) int array in one block; total in a[len] and *host_total
+__global__ void k_scan_ex(int* a, long long len, int* host_total) {
+  __shared__ int sh[32];
+  const long long chunk = (len + blockDim.x - 1) / blockDim.x;
+  const long long b0 = threadIdx.x * chunk, b1 = min(len, b0 + chunk);
+  int s = 0, total;
+  for (long long i = b0; i < b1; i++) s += a[i];
+  int run = block_prefix(s, sh, total);
   for (long long i = b0; i < b1; i++) {
     const int v = a[i];
-    a[i] = (int)run;
+    a[i] = run;
     run += v;
   }
+  if (threadIdx.x == 0) {
+    a[len] = total;
+    *host_total = total;
+  }
+}
+
+// Exclusive scan of every row of hist[256][ntile] (block d: digit d), its total in tot[d];
+// the scatter adds the prefix over digits itself. One block over the whole table took
+// 11.5 us at 29 tiles, this 2.6 at 58.
+__global__ void k_rs_scan(int* hist, int ntile, int* tot) {
+  __shared__ int sh[NT / 32];
+  int* row = hist + (long long)blockIdx.x * ntile;
+  int run = 0;
+  for (int t0 = 0; t0 < ntile; t0 += NT) {
+    const int t = t0 + threadIdx.x;
+    int total;
+    const int v = t < ntile ? row[t] : 0;
+    const int pre = block_prefix(v, sh, total);
+    if (t < ntile) row[t] = run + pre;
+    run += total;
+  }
+  if (threadIdx.x == 0) tot[blockIdx.x] = run;
 }
 
 // block-stable position of flagged elements, 256 per round
@@ -261,8 +310,9 @@ __global__ void k_rs_hist(const unsigned long long* key, int K, int shift, int* 
   __shared__ int h[256];
   h[threadIdx.x] = 0;
   __syncthreads();
-  const long long base = (long long)blockIdx.x * TILE;
-  for (int r = 0; r < TILE / NT; r++) {
+  const long long base = (long long)blockIdx.x * RTILE;
+#pragma unroll
+  for (int r = 0; r < RTILE / NT; r++) {
     const long long e = base + r * NT + threadIdx.x;
     if (e < K) atomicAdd(&h[(key[e] >> shift) & 255], 1);
   }
@@ -270,86 +320,147 @@ __global__ void k_rs_hist(const unsigned long long* key, int K, int shift, int* 
   hist[threadIdx.x * ntile + blockIdx.x] = h[threadIdx.x];
 }
 
+// Warp w holds the tile's elements [w EPW, (w + 1) EPW), EPW = RTILE / WPB, so one pass over
+// the warps' digit counts orders the whole tile (a count and two barriers per 256 elements
+// before).
 __global__ void k_rs_scatter(const unsigned long long* key, const int* val, int K, int shift, const int* off,
-                             int ntile, unsigned long long* key2, int* val2) {
+                             const int* tot, int ntile, unsigned long long* key2, int* val2) {
+  constexpr int EPW = RTILE / WPB, ROUNDS = EPW / 32;
   __shared__ int wc[WPB][256];
-  __shared__ int run[256];
+  __shared__ int sh[WPB];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  run[threadIdx.x] = off[threadIdx.x * ntile + blockIdx.x];
-  const long long base = (long long)blockIdx.x * TILE;
-  for (int r = 0; r < TILE / NT; r++) {
-    for (int k = 0; k < WPB; k++) wc[k][threadIdx.x] = 0;
-    __syncthreads();
-    const long long e = base + r * NT + threadIdx.x;
-    const bool ok = e < K;
-    const unsigned long long kk = ok ? key[e] : 0ull;
-    const int dg = ok ? (int)((kk >> shift) & 255) : 256 + lane;  // invalid: unique per lane, never matched
+  const long long base = (long long)blockIdx.x * RTILE + w * EPW;
+  unsigned long long kk[ROUNDS];
+  int vv[ROUNDS], rank[ROUNDS];
+#pragma unroll
+  for (int r = 0; r < ROUNDS; r++) {
+    const long long e = base + r * 32 + lane;
+    kk[r] = e < K ? key[e] : 0ull;
+    vv[r] = e < K ? val[e] : 0;
+  }
+  const int first = off[threadIdx.x * ntile + blockIdx.x];
+  int grand;
+  const int digit0 = block_prefix(tot[threadIdx.x], sh, grand);
+  for (int k = 0; k < WPB; k++) wc[k][threadIdx.x] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < ROUNDS; r++) {  // rank of each element among its warp's equal digits
+    const bool ok = base + r * 32 + lane < K;
+    const int dg = ok ? (int)((kk[r] >> shift) & 255) : 256 + lane;  // invalid: unique per lane, never matched
     const unsigned mm = __match_any_sync(0xffffffffu, dg);
-    const int rank = __popc(mm & ((1u << lane) - 1u));
-    if (ok && rank == 0) wc[w][dg] = __popc(mm);
-    __syncthreads();
-    // exclusive prefix over warps per digit
-    int acc = 0;
-    for (int k = 0; k < WPB; k++) {
-      const int v = wc[k][threadIdx.x];
-      wc[k][threadIdx.x] = acc;
-      acc += v;
+    const int before = __popc(mm & ((1u << lane) - 1u));
+    rank[r] = ok ? wc[w][dg] + before : 0;
+    __syncwarp();
+    if (ok && before == 0) wc[w][dg] += __popc(mm);
+    __syncwarp();
+  }
+  __syncthreads();
+  int acc = digit0 + first;  // thread d: where digit d of this tile starts, warp by warp
+  for (int k = 0; k < WPB; k++) {
+    const int v = wc[k][threadIdx.x];
+    wc[k][threadIdx.x] = acc;
+    acc += v;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < ROUNDS; r++) {
+    if (base + r * 32 + lane < K) {
+      const int pos = wc[w][(int)((kk[r] >> shift) & 255)] + rank[r];
+      key2[pos] = kk[r];
+      val2[pos] = vv[r];
     }
-    __syncthreads();
-    if (ok) {
-      const int pos = run[dg] + wc[w][dg] + rank;
-      key2[pos] = kk;
-      val2[pos] = val[e];
-    }
-    __syncthreads();
-    run[threadIdx.x] += acc;
-    __syncthreads();
   }
 }
 
 // ---- prefix sums over sorted breakpoints ------------------------------------------
 // For sorted breakpoint e (b = val[e], t_e, d_b, w_b): u = d_b w_b, v = t_e d_b w_b, s = d_b^2.
-// Pass 1: sums per warp chunk. Layout of a partial: [u(0..col2) | v(0..col2) | s].
-__global__ void k_gcp_sum(const unsigned long long* key, const int* val, int K, int chunk, const double* d,
-                          const double* S, const double* Y, long long n, Cols c, double theta, double* part) {
+// Pass 1: sums per warp chunk, part[component][warp] with the components
+// [u(0..col2) | v(0..col2) | s]. The chunk's breakpoints are read 32 at a time, one per
+// lane, so that the gathers of W of several breakpoints are in flight together. Float64
+// arithmetic bounds it (two lanes a cycle on an SM), so a breakpoint costs a column two
+// multiply-adds and no more (59,319 breakpoints, 20 columns: 21 us with seven operations,
+// 12 us so): t d_b and d_b^2 are formed once per lane, theta at the end.
+__global__ void k_gcp_sum(const unsigned long long* key, const int* val, int K, int chunk, int nw, const double* d,
+                          const double* S, const double* Y, long long n, Cols c, double theta, double* part,
+                          int* jstar) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *jstar = 0x7fffffff;
   const int lane = threadIdx.x & 31;
   const int wg = (blockIdx.x * NT + threadIdx.x) >> 5;
   const int col2 = 2 * c.col;
   const long long e0 = (long long)wg * chunk, e1 = min((long long)K, e0 + chunk);
   if (e0 >= e1) return;  // warps past the last chunk
+  const double* col = lane < c.col ? Y + (long long)c.slot[lane] * n
+                      : lane < col2 ? S + (long long)c.slot[lane - c.col] * n : nullptr;
+  const double cs = lane < c.col ? 1.0 : theta;
   double u = 0.0, v = 0.0, s = 0.0;
-  for (long long e = e0; e < e1; e++) {
-    const int b = val[e];
-    const double te = __longlong_as_double((long long)key[e]);
-    const double db = d[b];
-    const double w = lane < col2 ? wcol(S, Y, n, c, theta, lane, b) : 0.0;
-    u += db * w;
-    v += te * db * w;
-    s += db * db;
+  for (long long eb = e0; eb < e1; eb += 32) {
+    const int m = (int)min((long long)32, e1 - eb);
+    const int bl = lane < m ? val[eb + lane] : 0;
+    double tl = lane < m ? __longlong_as_double((long long)key[eb + lane]) : 0.0;
+    const double dl = lane < m ? d[bl] : 0.0;
+    tl *= dl;
+    s += dl * dl;
+#pragma unroll 8
+    for (int q = 0; q < m; q++) {
+      const int b = __shfl_sync(0xffffffffu, bl, q);
+      const double tdb = __shfl_sync(0xffffffffu, tl, q), db = __shfl_sync(0xffffffffu, dl, q);
+      if (col) {
+        const double w = col[b];
+        u += db * w;
+        v += tdb * w;
+      }
+    }
   }
-  const int nv = 2 * col2 + 1;
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane < col2) {
-    part[(long long)wg * nv + lane] = u;
-    part[(long long)wg * nv + col2 + lane] = v;
+    part[(long long)lane * nw + wg] = cs * u;
+    part[(long long)(col2 + lane) * nw + wg] = cs * v;
   }
-  if (lane == 0) part[(long long)wg * nv + 2 * col2] = s;
+  if (lane == 0) part[(long long)(2 * col2) * nw + wg] = s;
 }
 
-// Pass 2: exclusive prefix over warps of every component (fixed order)
-__global__ void k_gcp_scan(double* part, int nw, int nv) {
-  for (int k = threadIdx.x; k < nv; k += blockDim.x) {
-    double run = 0.0;
-    for (int w = 0; w < nw; w++) {
-      const double x = part[(long long)w * nv + k];
-      part[(long long)w * nv + k] = run;
-      run += x;
-    }
+// Pass 2: exclusive prefix over warps, one block per component: each thread adds its run of
+// consecutive values, the block scans the run sums, each thread walks its run again (one
+// thread over all 4,600 warps, load and store in turn, took 0.70 ms, this 7 us).
+__global__ void k_gcp_scan(double* part, int nw) {
+  __shared__ double sh[NT / 32];
+  double* row = part + (long long)blockIdx.x * nw;
+  const int chunk = (nw + NT - 1) / NT;
+  const int w0 = min(nw, (int)threadIdx.x * chunk), w1 = min(nw, w0 + chunk);
+  double s = 0.0, total;
+  for (int w = w0; w < w1; w++) s += row[w];
+  // the inclusive scan minus the value would round: shift the inclusive scan by one thread
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  double inc = s;
+  for (int o = 1; o < 32; o <<= 1) {
+    const double y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  double run = __shfl_up_sync(0xffffffffu, inc, 1);
+  if (lane == 0) run = 0.0;
+  if (lane == 31) sh[wp] = inc;
+  __syncthreads();
+  total = 0.0;
+  for (int k = 0; k < wp; k++) total += sh[k];
+  run += total;
+  for (int w = w0; w < w1; w++) {
+    const double x = row[w];
+    row[w] = run;
+    run += x;
   }
 }
 
 struct GcpScal {
   double theta, D2, f2org;
-  int K;
+  int K, nw;
+};
+// p0 = W^T d and the middle matrix M (2 col x 2 col, row-major), passed by value
+struct GcpSmall {
+  double p0[2 * MAXM];
+  double M[4 * MAXM * MAXM];
+};
+struct Vec2m {
+  double v[2 * MAXM];
 };
 // Pass 3: walk each chunk with running prefixes Q (sum d_b w_b), R (sum t d_b w_b), S2;
 // after breakpoint j (1-based): P_j = p0 - Q_j, c_j = t_j P_{j-1} + R_{j-1},
@@ -358,88 +469,99 @@ struct GcpScal {
 // cand[warp] = {j, dtm, t_j, P_j (col2), c_j (col2)}.
 __global__ void k_gcp_search(const unsigned long long* key, const int* val, int chunk, const double* d,
                              const double* S, const double* Y, long long n, Cols c, GcpScal q, const double* part,
-                             const double* p0, const double* Mmat, int* jstar, double* cand) {
-  __shared__ double Ms[2 * MAXM][2 * MAXM];
+                             const __grid_constant__ GcpSmall sm, int* jstar, double* cand) {
+  __shared__ double Ms[2 * MAXM][2 * MAXM + 1];  // padded: lanes read a column
   const int col2 = 2 * c.col;
-  for (int k = threadIdx.x; k < col2 * col2; k += NT) Ms[k / col2][k % col2] = Mmat[k];
+  for (int k = threadIdx.x; k < col2 * col2; k += NT) Ms[k / col2][k % col2] = sm.M[k];
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int wg = (blockIdx.x * NT + threadIdx.x) >> 5;
-  const int nv = 2 * col2 + 1;
   const long long e0 = (long long)wg * chunk, e1 = min((long long)q.K, e0 + chunk);
   if (e0 >= e1) return;
-  double Q = lane < col2 ? part[(long long)wg * nv + lane] : 0.0;
-  double R = lane < col2 ? part[(long long)wg * nv + col2 + lane] : 0.0;
-  double S2 = part[(long long)wg * nv + 2 * col2];
-  const double p0l = lane < col2 ? p0[lane] : 0.0;
-  for (long long e = e0; e < e1; e++) {
-    if ((e & 63) == 0) {  // an earlier segment already holds the Cauchy point (warp-uniform test)
+  double Q = lane < col2 ? part[(long long)lane * q.nw + wg] : 0.0;
+  double R = lane < col2 ? part[(long long)(col2 + lane) * q.nw + wg] : 0.0;
+  double S2 = part[(long long)(2 * col2) * q.nw + wg];
+  const double p0l = lane < col2 ? sm.p0[lane] : 0.0;
+  const double* col = lane < c.col ? Y + (long long)c.slot[lane] * n
+                      : lane < col2 ? S + (long long)c.slot[lane - c.col] * n : nullptr;
+  const double cs = lane < c.col ? 1.0 : q.theta;
+  for (long long eb = e0; eb < e1; eb += 32) {
+    {  // an earlier segment already holds the Cauchy point (warp-uniform test)
       int js = 0;
       if (lane == 0) js = *((volatile int*)jstar);
       js = __shfl_sync(0xffffffffu, js, 0);
-      if (js <= e) return;
+      if (js <= eb) return;
     }
-    const int b = val[e];
-    const double te = __longlong_as_double((long long)key[e]);
-    const double db = d[b];
-    const double w = lane < col2 ? wcol(S, Y, n, c, q.theta, lane, b) : 0.0;
-    const double Cj = te * (p0l - Q) + R;  // c_j from P_{j-1}, R_{j-1}
-    Q += db * w;
-    R += te * db * w;
-    S2 += db * db;
-    const double Pj = p0l - Q;
-    const double Dj = q.D2 - S2;
-    double mp = 0.0;
-    for (int a = 0; a < col2; a++) {
-      const double pa = __shfl_sync(0xffffffffu, Pj, a);
-      if (lane < col2) mp += Ms[lane][a] * pa;
-    }
-    double cmp = Cj * mp, pmp = Pj * mp;
-    for (int o = 16; o; o >>= 1) {
-      cmp += __shfl_xor_sync(0xffffffffu, cmp, o);
-      pmp += __shfl_xor_sync(0xffffffffu, pmp, o);
-    }
-    const long long j = e + 1;
-    double f1 = -Dj + q.theta * te * Dj - cmp;
-    double f2 = fmax(EPSMCH * q.f2org, q.theta * Dj - pmp);
-    double dtm;
-    bool stop;
-    if (j == q.K) {
-      dtm = 0.0;  // every breakpoint passed: all moving variables at their bounds
-      stop = true;
-    } else {
-      dtm = -f1 / f2;
-      const double tn = __longlong_as_double((long long)key[e + 1]);
-      stop = dtm < tn - te;
-    }
-    if (stop) {
-      double* o = cand + (long long)wg * (3 + 2 * 2 * MAXM);
-      if (lane == 0) {
-        o[0] = (double)j;
-        o[1] = dtm;
-        o[2] = te;
-        atomicMin(jstar, (int)j);
+    const int m = (int)min((long long)32, e1 - eb);
+    const int bl = lane < m ? val[eb + lane] : 0;
+    const double tl = lane < m ? __longlong_as_double((long long)key[eb + lane]) : 0.0;
+    const double dl = lane < m ? d[bl] : 0.0;
+    const int b0 = __shfl_sync(0xffffffffu, bl, 0);
+    double wn = col ? cs * col[b0] : 0.0;
+    for (int r = 0; r < m; r++) {
+      const long long e = eb + r;
+      const double te = __shfl_sync(0xffffffffu, tl, r), db = __shfl_sync(0xffffffffu, dl, r);
+      const double w = wn;
+      const int bn = __shfl_sync(0xffffffffu, bl, r + 1 < m ? r + 1 : r);
+      wn = col ? cs * col[bn] : 0.0;  // the next breakpoint's, in flight meanwhile
+      const double Cj = te * (p0l - Q) + R;  // c_j from P_{j-1}, R_{j-1}
+      const double dw = db * w;
+      Q += dw;
+      R += te * dw;
+      S2 += db * db;
+      const double Pj = p0l - Q;
+      const double Dj = q.D2 - S2;
+      double mp = 0.0;
+      for (int a = 0; a < col2; a++) {
+        const double pa = __shfl_sync(0xffffffffu, Pj, a);
+        if (lane < col2) mp += Ms[lane][a] * pa;
       }
-      if (lane < col2) {
-        o[3 + lane] = Pj;
-        o[3 + col2 + lane] = Cj;
+      double cmp = Cj * mp, pmp = Pj * mp;
+      for (int o = 16; o; o >>= 1) {
+        cmp += __shfl_xor_sync(0xffffffffu, cmp, o);
+        pmp += __shfl_xor_sync(0xffffffffu, pmp, o);
       }
-      return;
+      const long long j = e + 1;
+      double f1 = -Dj + q.theta * te * Dj - cmp;
+      double f2 = fmax(EPSMCH * q.f2org, q.theta * Dj - pmp);
+      double dtm;
+      bool stop;
+      if (j == q.K) {
+        dtm = 0.0;  // every breakpoint passed: all moving variables at their bounds
+        stop = true;
+      } else {
+        dtm = -f1 / f2;
+        const double tn = __longlong_as_double((long long)key[e + 1]);
+        stop = dtm < tn - te;
+      }
+      if (stop) {
+        double* o = cand + (long long)wg * (3 + 2 * 2 * MAXM);
+        if (lane == 0) {
+          o[0] = (double)j;
+          o[1] = dtm;
+          o[2] = te;
+          atomicMin(jstar, (int)j);
+        }
+        if (lane < col2) {
+          o[3 + lane] = Pj;
+          o[3 + col2 + lane] = Cj;
+        }
+        return;
+      }
     }
   }
 }
 
-// the winning warp's candidate {j, dtm, t_j, P_j, c_j} into out (one thread)
+// the winning warp's candidate {j, dtm, t_j, P_j, c_j} into out (pinned host memory)
 __global__ void k_pick_cand(const int* jstar, int chunk, const double* cand, double* out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const int js = *jstar;
   constexpr int cl = 3 + 2 * 2 * MAXM;
   if (js < 1 || js == 0x7fffffff) {
-    out[0] = -1.0;
+    if (threadIdx.x == 0) out[0] = -1.0;
     return;
   }
   const double* c = cand + (long long)((js - 1) / chunk) * cl;
-  for (int i = 0; i < cl; i++) out[i] = c[i];
+  for (int i = threadIdx.x; i < cl; i += blockDim.x) out[i] = c[i];
 }
 
 // xcp = x + tsum d; free = moving or zero-gradient; then the first jst sorted
@@ -462,16 +584,13 @@ __global__ void k_xcp_fix(const int* val, int jst, const double* d, double lo, d
 // ---- subspace minimisation -----------------------------------------------------------
 // r = -theta (xcp - x) - g + W (M c) on free variables (the negative reduced gradient)
 __global__ void k_rgrad(const double* x, const double* g, const double* xcp, const int8_t* fr, long long n,
-                        const double* S, const double* Y, Cols c, double theta, const double* Mc, double* r) {
-  __shared__ double mc[2 * MAXM];
+                        const double* S, const double* Y, Cols c, double theta, const Vec2m mc, double* r) {
   const int col2 = 2 * c.col;
-  if (threadIdx.x < col2) mc[threadIdx.x] = Mc[threadIdx.x];
-  __syncthreads();
   for (long long i = blockIdx.x * (long long)NT + threadIdx.x; i < n; i += (long long)gridDim.x * NT) {
     double ri = 0.0;
     if (fr[i]) {
       ri = -theta * (xcp[i] - x[i]) - g[i];
-      for (int a = 0; a < col2; a++) ri += wcol(S, Y, n, c, theta, a, i) * mc[a];
+      for (int a = 0; a < col2; a++) ri += wcol(S, Y, n, c, theta, a, i) * mc.v[a];
     }
     r[i] = ri;
   }
@@ -545,17 +664,14 @@ __global__ void k_gram(const int8_t* fr, const double* r, long long n, const dou
 // sums: [0] (xbar - x) . g, [1] number of free variables that landed on a bound
 __global__ void k_newton(const double* x, const double* g, const double* xcp, const int8_t* fr, long long n,
                          double lo, double hi, const double* S, const double* Y, Cols c, double theta,
-                         const double* vv, double* r, double* xbar, double* part) {
-  __shared__ double v[2 * MAXM];
+                         const Vec2m v, double* r, double* xbar, double* part) {
   const int col2 = 2 * c.col;
-  if (threadIdx.x < col2) v[threadIdx.x] = vv[threadIdx.x];
-  __syncthreads();
   double s[2] = {0.0, 0.0};
   for (long long i = blockIdx.x * (long long)NT + threadIdx.x; i < n; i += (long long)gridDim.x * NT) {
     double xb = xcp[i];
     if (fr[i]) {
       double wv = 0.0;
-      for (int a = 0; a < col2; a++) wv += wcol(S, Y, n, c, theta, a, i) * v[a];
+      for (int a = 0; a < col2; a++) wv += wcol(S, Y, n, c, theta, a, i) * v.v[a];
       const double du = r[i] / theta + wv / (theta * theta);
       r[i] = du;
       xb = fmin(hi, fmax(lo, xb + du));
@@ -869,13 +985,14 @@ struct tm_lbfgsb {
   double lo = 0, hi = 1, factr = 1e7, pgtol = 1e-5;
   std::string err;
   // device state
+  void* arena = nullptr;  // holds every array below
   double *x = nullptr, *g = nullptr, *xt = nullptr, *gt = nullptr, *d = nullptr, *xcp = nullptr, *xbar = nullptr,
          *r = nullptr, *t = nullptr, *S = nullptr, *Y = nullptr;
   int8_t *st = nullptr, *fr = nullptr;
   unsigned long long *key = nullptr, *key2 = nullptr;
-  int *val = nullptr, *val2 = nullptr, *cnt = nullptr, *hist = nullptr, *jstar = nullptr;
-  double *part = nullptr, *red = nullptr, *small = nullptr, *cand = nullptr;
-  VI *mpart = nullptr, *mred = nullptr;
+  int *val = nullptr, *val2 = nullptr, *cnt = nullptr, *hist = nullptr, *tot = nullptr, *jstar = nullptr;
+  double *part = nullptr, *cand = nullptr;
+  VI* mpart = nullptr;
   size_t part_doubles = 0;
   double* hbuf = nullptr;  // pinned
   // host state
@@ -910,32 +1027,23 @@ Cols cols_of(const tm_lbfgsb* o) {
   return c;
 }
 
-// sums in o->part (nblk partials of nv) -> host hbuf[0..nv)
-int fetch_sums(tm_lbfgsb* o, int nblk, int nv, cudaStream_t s) {
-  k_finish<<<1, 256, 0, s>>>(o->part, nblk, nv, o->red);
-  LCKL();
-  LCK(cudaMemcpyAsync(o->hbuf, o->red, nv * sizeof(double), cudaMemcpyDeviceToHost, s));
-  LCK(cudaStreamSynchronize(s));
-  return TM_OK;
-}
-// sums (nblk_s partials of nv) to hbuf[0..nv) and the min of nblk_m partials to *out, one sync
+// Pinned host memory the kernels write to: results in hbuf[0 .. 999], then the count of
+// breakpoints and the pair of a min reduction.
+constexpr int kHbufCount = 1000, kHbufMin = 1002;
+
+// sums in o->part (nblk partials of nv, if nv > 0) to hbuf[0..nv) and the min of nblk_m pairs
+// of o->mpart (if nblk_m > 0) to *out, one launch and one wait
 int fetch_both(tm_lbfgsb* o, int nblk_s, int nv, int nblk_m, VI* out, cudaStream_t s) {
-  k_finish<<<1, 256, 0, s>>>(o->part, nblk_s, nv, o->red);
+  VI* hm = reinterpret_cast<VI*>(o->hbuf + kHbufMin);
+  k_finish<<<(nv + FV - 1) / FV + (nblk_m > 0 ? 1 : 0), NT, 0, s>>>(o->part, nblk_s, nv, o->hbuf,
+                                                                    nblk_m > 0 ? o->mpart : nullptr, nblk_m, hm);
   LCKL();
-  k_finish_min<<<1, 32, 0, s>>>(o->mpart, nblk_m, o->mred);
-  LCKL();
-  LCK(cudaMemcpyAsync(o->hbuf, o->red, nv * sizeof(double), cudaMemcpyDeviceToHost, s));
-  LCK(cudaMemcpyAsync(out, o->mred, sizeof(VI), cudaMemcpyDeviceToHost, s));
   LCK(cudaStreamSynchronize(s));
+  if (nblk_m > 0) *out = *hm;
   return TM_OK;
 }
-int fetch_min(tm_lbfgsb* o, int nblk, VI* out, cudaStream_t s) {
-  k_finish_min<<<1, 32, 0, s>>>(o->mpart, nblk, o->mred);
-  LCKL();
-  LCK(cudaMemcpyAsync(out, o->mred, sizeof(VI), cudaMemcpyDeviceToHost, s));
-  LCK(cudaStreamSynchronize(s));
-  return TM_OK;
-}
+int fetch_sums(tm_lbfgsb* o, int nblk, int nv, cudaStream_t s) { return fetch_both(o, nblk, nv, 0, nullptr, s); }
+int fetch_min(tm_lbfgsb* o, int nblk, VI* out, cudaStream_t s) { return fetch_both(o, 0, 0, nblk, out, s); }
 
 // the inverse middle matrix [[-D, L^T], [L, theta S^T S]] (2col x 2col, row-major)
 std::vector<double> middle_inv(const tm_lbfgsb* o) {
@@ -965,10 +1073,9 @@ int direction(tm_lbfgsb* o, cudaStream_t s) {
   k_bp<<<ntile, NT, 0, s>>>(o->x, o->g, n, o->lo, o->hi, o->S, o->Y, c, theta, o->d, o->t, o->st, o->part, o->cnt,
                             o->mpart);
   LCKL();
-  k_scan_ex<<<1, 1024, 0, s>>>(o->cnt, ntile);
+  int* Kh = reinterpret_cast<int*>(o->hbuf + kHbufCount);
+  k_scan_ex<<<1, 1024, 0, s>>>(o->cnt, ntile, Kh);
   LCKL();
-  int* Kh = reinterpret_cast<int*>(o->hbuf + 1000);  // pinned slot for the count
-  LCK(cudaMemcpyAsync(Kh, o->cnt + ntile, sizeof(int), cudaMemcpyDeviceToHost, s));
   VI tmin;
   if (int e = fetch_both(o, ntile, col2 + 1, ntile, &tmin, s)) return e;
   std::vector<double> p0(o->hbuf, o->hbuf + col2);
@@ -1001,15 +1108,15 @@ int direction(tm_lbfgsb* o, cudaStream_t s) {
       k_bp_compact<<<ntile, NT, 0, s>>>(o->t, o->st, n, o->cnt, o->key, o->val);
       LCKL();
       // sort by t (stable, so equal t keep index order)
-      const int kt = (K + TILE - 1) / TILE;
+      const int kt = (K + RTILE - 1) / RTILE;
       unsigned long long *k1 = o->key, *k2 = o->key2;
       int *v1 = o->val, *v2 = o->val2;
       for (int sh = 0; sh < 64; sh += 8) {
         k_rs_hist<<<kt, NT, 0, s>>>(k1, K, sh, o->hist, kt);
         LCKL();
-        k_scan_ex<<<1, 1024, 0, s>>>(o->hist, 256LL * kt);
+        k_rs_scan<<<256, NT, 0, s>>>(o->hist, kt, o->tot);
         LCKL();
-        k_rs_scatter<<<kt, NT, 0, s>>>(k1, v1, K, sh, o->hist, kt, k2, v2);
+        k_rs_scatter<<<kt, NT, 0, s>>>(k1, v1, K, sh, o->hist, o->tot, kt, k2, v2);
         LCKL();
         std::swap(k1, k2);
         std::swap(v1, v2);
@@ -1025,25 +1132,19 @@ int direction(tm_lbfgsb* o, cudaStream_t s) {
       const int chunk = (K + nw - 1) / nw;
       const int nwu = (K + chunk - 1) / chunk;
       const int blocks = (nwu + WPB - 1) / WPB;
-      k_gcp_sum<<<blocks, NT, 0, s>>>(o->key, o->val, K, chunk, o->d, o->S, o->Y, n, c, theta, o->part);
+      k_gcp_sum<<<blocks, NT, 0, s>>>(o->key, o->val, K, chunk, nwu, o->d, o->S, o->Y, n, c, theta, o->part, o->jstar);
       LCKL();
-      k_gcp_scan<<<1, 128, 0, s>>>(o->part, nwu, 2 * col2 + 1);
+      k_gcp_scan<<<2 * col2 + 1, NT, 0, s>>>(o->part, nwu);
       LCKL();
-      // small: p0 (col2), M (col2^2)
-      std::vector<double> hs(col2 + col2 * col2);
-      std::copy(p0.begin(), p0.end(), hs.begin());
-      std::copy(M.begin(), M.end(), hs.begin() + col2);
-      if (!hs.empty()) LCK(cudaMemcpyAsync(o->small, hs.data(), hs.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-      const int big = 0x7fffffff;
-      LCK(cudaMemcpyAsync(o->jstar, &big, sizeof(int), cudaMemcpyHostToDevice, s));
-      GcpScal q{theta, D2, f2org, K};
-      k_gcp_search<<<blocks, NT, 0, s>>>(o->key, o->val, chunk, o->d, o->S, o->Y, n, c, q, o->part, o->small,
-                                        o->small + col2, o->jstar, o->cand);
+      GcpSmall sm;
+      std::copy(p0.begin(), p0.end(), sm.p0);
+      std::copy(M.begin(), M.end(), sm.M);
+      GcpScal q{theta, D2, f2org, K, nwu};
+      k_gcp_search<<<blocks, NT, 0, s>>>(o->key, o->val, chunk, o->d, o->S, o->Y, n, c, q, o->part, sm, o->jstar,
+                                        o->cand);
       LCKL();
-      const int cl = 3 + 2 * 2 * MAXM;
-      k_pick_cand<<<1, 32, 0, s>>>(o->jstar, chunk, o->cand, o->red);
+      k_pick_cand<<<1, 64, 0, s>>>(o->jstar, chunk, o->cand, o->hbuf);
       LCKL();
-      LCK(cudaMemcpyAsync(o->hbuf, o->red, cl * sizeof(double), cudaMemcpyDeviceToHost, s));
       LCK(cudaStreamSynchronize(s));
       const int js = (int)o->hbuf[0];
       if (js < 1 || js > K) return fail(o, TM_ERR_STATE, "Cauchy point search found no segment");
@@ -1066,11 +1167,10 @@ int direction(tm_lbfgsb* o, cudaStream_t s) {
     o->nfree = -1;
     return TM_OK;
   }
-  std::vector<double> Mc(col2, 0.0);
+  Vec2m Mc{};
   for (int a = 0; a < col2; a++)
-    for (int b = 0; b < col2; b++) Mc[a] += M[a * col2 + b] * cvec[b];
-  LCK(cudaMemcpyAsync(o->small, Mc.data(), col2 * sizeof(double), cudaMemcpyHostToDevice, s));
-  k_rgrad<<<gb, NT, 0, s>>>(o->x, o->g, o->xcp, o->fr, n, o->S, o->Y, c, theta, o->small, o->r);
+    for (int b = 0; b < col2; b++) Mc.v[a] += M[a * col2 + b] * cvec[b];
+  k_rgrad<<<gb, NT, 0, s>>>(o->x, o->g, o->xcp, o->fr, n, o->S, o->Y, c, theta, Mc, o->r);
   LCKL();
   const int np = col2 * (col2 + 1) / 2, ntot = np + col2 + 1;
   const int gg = std::max(1, std::min((int)((n + GT - 1) / GT), 2 * o->nsm));
@@ -1095,9 +1195,10 @@ int direction(tm_lbfgsb* o, cudaStream_t s) {
     }
   for (int a = 0; a < col2; a++) rhs[a] = h[np + a] * (a < o->col ? 1.0 : theta);
   if (!solve_inplace(A, rhs, col2, 1)) return fail(o, TM_ERR_STATE, "singular reduced system");
-  LCK(cudaMemcpyAsync(o->small, rhs.data(), col2 * sizeof(double), cudaMemcpyHostToDevice, s));
-  k_newton<<<gb, NT, 0, s>>>(o->x, o->g, o->xcp, o->fr, n, o->lo, o->hi, o->S, o->Y, c, theta, o->small, o->r,
-                             o->xbar, o->part);
+  Vec2m rv{};
+  std::copy(rhs.begin(), rhs.end(), rv.v);
+  k_newton<<<gb, NT, 0, s>>>(o->x, o->g, o->xcp, o->fr, n, o->lo, o->hi, o->S, o->Y, c, theta, rv, o->r, o->xbar,
+                             o->part);
   LCKL();
   if (int e = fetch_sums(o, gb, 2, s)) return e;
   const double ddp = o->hbuf[0], hit = o->hbuf[1];
@@ -1186,9 +1287,10 @@ int tm_lbfgsb_create(tm_lbfgsb** out, int device, long long n, int m, double low
   const long long nwmax = (long long)WPB * 4 * o->nsm;
   o->part_doubles = (size_t)std::max({ntile * (2 * MAXM + 1), nwmax * (4 * MAXM + 1), 4LL * o->nsm * 600,
                                       (long long)grid_for(n, o->nsm) * (2 * MAXM + 1)});
-  auto A = [&](void** p, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMalloc(p, bytes);
-  };
+  // one allocation for all arrays: an optimiser is created for every run, and 25 allocations
+  // and as many frees took longer than two iterations at 59,319 variables
+  std::vector<std::pair<void**, size_t>> want;
+  auto A = [&](void** p, size_t bytes) { want.emplace_back(p, (bytes + 255) / 256 * 256); };
   const size_t nd = (size_t)n * sizeof(double);
   A((void**)&o->x, nd);
   A((void**)&o->g, nd);
@@ -1208,15 +1310,23 @@ int tm_lbfgsb_create(tm_lbfgsb** out, int device, long long n, int m, double low
   A((void**)&o->val, n * sizeof(int));
   A((void**)&o->val2, n * sizeof(int));
   A((void**)&o->cnt, (ntile + 1) * sizeof(int));
-  A((void**)&o->hist, (256 * ntile + 1) * sizeof(int));
+  A((void**)&o->hist, 256 * ((n + RTILE - 1) / RTILE) * sizeof(int));
+  A((void**)&o->tot, 256 * sizeof(int));
   A((void**)&o->jstar, sizeof(int));
   A((void**)&o->part, o->part_doubles * sizeof(double));
-  A((void**)&o->red, 1024 * sizeof(double));
-  A((void**)&o->small, (2 * MAXM + 4 * MAXM * MAXM) * sizeof(double));
   A((void**)&o->cand, nwmax * (3 + 4 * MAXM) * sizeof(double));
   A((void**)&o->mpart, std::max(8LL * o->nsm, ntile) * sizeof(VI));  // also one per k_bp tile
-  A((void**)&o->mred, sizeof(VI));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&o->hbuf, 1024 * sizeof(double));
+  size_t bytes = 0;
+  for (const auto& w : want) bytes += w.second;
+  if (e == cudaSuccess) e = cudaMalloc(&o->arena, bytes);
+  if (e == cudaSuccess) {
+    char* at = static_cast<char*>(o->arena);
+    for (const auto& w : want) {
+      *w.first = at;
+      at += w.second;
+    }
+    e = cudaMallocHost((void**)&o->hbuf, 1024 * sizeof(double));
+  }
   if (e != cudaSuccess) {
     tm_lbfgsb_destroy(o);
     return e == cudaErrorMemoryAllocation ? TM_ERR_NOMEM : TM_ERR_CUDA;
@@ -1228,11 +1338,7 @@ int tm_lbfgsb_create(tm_lbfgsb** out, int device, long long n, int m, double low
 void tm_lbfgsb_destroy(tm_lbfgsb* o) {
   if (!o) return;
   cudaSetDevice(o->device);
-  void* ps[] = {o->x,   o->g,    o->xt,   o->gt,  o->d,    o->xcp,   o->xbar, o->r,     o->t,
-                o->S,   o->Y,    o->st,   o->fr,  o->key,  o->key2,  o->val,  o->val2,  o->cnt,
-                o->hist, o->jstar, o->part, o->red, o->small, o->cand, o->mpart, o->mred};
-  for (void* p : ps)
-    if (p) cudaFree(p);
+  cudaFree(o->arena);
   if (o->hbuf) cudaFreeHost(o->hbuf);
   delete o;
 }
