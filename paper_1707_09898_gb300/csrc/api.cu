@@ -361,18 +361,24 @@ int conv_yz(tm_ctx* ctx, const ConvSpec& cs, int zin, int zout, cudaStream_t s) 
   z.nin = cs.nin;
   z.nout = cs.nout;
   for (int i = 0; i < cs.nin; i++) z.in_slot[i] = cs.bin[i];
+  z.need = 0;
   for (int o = 0; o < cs.nout; o++) {
     z.out_slot[o] = cs.bout[o];
-    z.need[o] = 0;
     for (int i = 0; i < cs.nin; i++) {
-      coef6(z.coef[o][i], cs.v[o], cs.u[i]);
-      for (int c = 0; c < 6; c++)
-        if (z.coef[o][i][c] != 0.0f) z.need[o] |= 1 << c;
+      float c6[6];
+      coef6(c6, cs.v[o], cs.u[i]);
+      for (int c = 0; c < 6; c++) {
+        if (c6[c] != 0.0f) z.need |= 1 << c;
+        if (i == 0) z.coef[o][c] = c6[c];
+      }
     }
+    for (int c = 0; c < 3; c++) z.v[o][c] = (float)cs.v[o][c];
   }
+  for (int i = 0; i < cs.nin; i++)
+    for (int c = 0; c < 3; c++) z.u[i][c] = (float)cs.u[i][c];
   z.T = ctx->T;
-  z.Tz = (long long)(Ly / 2 + 1) * P;
-  z.Tc = (long long)(Lz / 2 + 1) * z.Tz;
+  z.Tz = (int)((Ly / 2 + 1) * P);
+  z.Tc = (Lz / 2 + 1) * z.Tz;  // at most 289 * 289 * 304
   z.zcol = ctx->zcol;
   z.ext = cs.ext;
   z.in_ext = cs.in_ext;
@@ -798,7 +804,6 @@ int tm_set_grid_lengths(tm_ctx* ctx, const int n_out[3], int nzd, const double c
   const int Lx = ctx->L[0], Ly = ctx->L[1], Lz = ctx->L[2];
   ctx->P = ((Lx / 2 + 1) + TB - 1) / TB * TB;
   const long long P = ctx->P;
-  if (zpass_smem(Lz) > 227 * 1024) return fail(ctx, TM_ERR_SIZE, "Lz = %d too large for the z pass", Lz);
 
   CK(cudaMalloc(&ctx->A, (long long)kSlotsA * ctx->nz * ctx->ny * P * sizeof(float2)));
   CK(cudaMalloc(&ctx->B, (long long)kSlotsB * ctx->nz * Ly * P * sizeof(float2)));

@@ -125,21 +125,22 @@ struct YArgs {
 };
 
 // z pass, in place on B[slot][z][Ly][P]: forward z transform of nin input slots,
-// out_o(k) = sum_i s_oi(k) in_i(k) with s_oi = sum_c coef[o][i][c] N^_c(k) over the six
-// unique tensor components (xx, yy, zz, xy, xz, yz), inverse z transform into out_slot[o].
-// nin == 1: one block per (tile, column, output). nin > 1: a cluster of nin blocks per
-// (tile, column); block r transforms input r and computes output r (r < nout).
+// out_o(k) = sum_i (v_o^T N^(k) u_i) in_i(k) over the six unique tensor components
+// (xx, yy, zz, xy, xz, yz), inverse z transform into out_slot[o]. With several inputs every
+// u_i is a unit vector, and with several outputs too the three components go in and out.
 struct ZArgs {
   float2* buf;
   long long cstride, zstride;  // between slots, between z planes
   int n_in, n_out, Ly, P;      // input / output z planes
   int nin, nout;
   int in_slot[3], out_slot[3];
-  float coef[3][3][6];
-  int need[3];                 // per output: bit c set if tensor component c is used
+  float u[3][3], v[3][3];      // per input, per output
+  int axis[3], oaxis[3];       // launch_zn: index of the unit vector u_i, v_o, or -1
+  float coef[3][6];            // one input: v_o^T N u_0 over the components
+  int need;                    // bit c set if tensor component c is used
   const float* T;              // [6][Lz/2+1][Ly/2+1][P]
-  long long Tc;                // elements per tensor component
-  long long Tz;                // (Ly/2+1) * P
+  int Tc;                      // elements per tensor component
+  int Tz;                      // (Ly/2+1) * P
   const int2* zcol;            // launch order of columns: (ky position, ky)
   const int* ext;              // device [zlo, zhi) of the target planes
   int in_ext, out_ext;         // input / output planes restricted to ext (else 0..n_in / 0..n_out)
@@ -230,12 +231,14 @@ int launch_xinv(int L, const XInvArgs& a, cudaStream_t s);
 int launch_yfwd(int L, const YArgs& a, int ncomp, cudaStream_t s);
 int launch_yinv(int L, const YArgs& a, int ncomp, cudaStream_t s);
 int launch_zpass(int L, const ZArgs& a, cudaStream_t s);
+int launch_zn(int L, const ZArgs& a, cudaStream_t s);  // any length, any u and v
+int launch_zn_mid(int L, const ZArgs& a, cudaStream_t s);   // its lengths 128 to 256
+int launch_zn_long(int L, const ZArgs& a, cudaStream_t s);  // and 288 to 576
 int xinv_rows_per_block();
 // Objective on few target rows, compact warp-per-row-pair transforms (k_xobj.cu);
 // needs a.Jcount / a.Jout (J summed by the last block) and a.adj_out.
 int launch_xobj(int L, const XInvArgs& a, cudaStream_t s);
 int xobj_rows_per_block();
-size_t zpass_smem(int L);
 
 // Tensor setup (float64) -- tensor.cu
 int tensor_setup(int nx, int ny, int nz, const double d[3], int Lx, int Ly, int Lz, int P, float* T_out,

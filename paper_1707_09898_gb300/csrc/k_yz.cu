@@ -6,21 +6,15 @@
 // positions and keep the first n_out rows (the crop).
 // z pass: forward z transform, the product with the tensor N^(k) (real, stored
 // once for kx, ky, kz in [0, L/2] and unfolded by parity), inverse z transform,
-// fused per column so the spectra never leave shared memory. The product is
+// fused per column so the spectra never leave the block. The product is
 // written as out_o = sum_i s_oi in_i with s_oi = v_o^T N^ u_i: u_i, v_o are unit
 // vectors for plain components, or M0 when the magnetization (forward input) or
 // the chain rule (adjoint output) is contracted with a constant M0 -- exact by
 // linearity of the convolution, and it removes two of the three transforms.
-// One input: one block per (column tile, output). Several inputs: a cluster of
-// one block per input; the blocks exchange spectra through distributed shared
-// memory.
-#include <cooperative_groups.h>
-
+// k_z1m below takes one input at L = 512, k_zn.cuh everything else.
 #include "fft.cuh"
 #include "internal.h"
 #include "unet_tc.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace tmk {
 
@@ -162,7 +156,7 @@ struct TensorCol {
   }
 };
 
-__device__ __forceinline__ TensorCol make_tcol(const ZArgs& a, int o, int i, int kyf, float sy, long long kx0) {
+__device__ __forceinline__ TensorCol make_tcol(const ZArgs& a, int o, int kyf, float sy, long long kx0) {
   TensorCol t;
   t.T = a.T + kyf * (long long)a.P + kx0;
   t.Tc = a.Tc;
@@ -170,13 +164,11 @@ __device__ __forceinline__ TensorCol make_tcol(const ZArgs& a, int o, int i, int
   t.sy = sy;
   t.need = 0;
 #pragma unroll
-  for (int c = 0; c < 6; c++) {  // (o, i) selected by compile-time indexes: no local copy of a.coef
+  for (int c = 0; c < 6; c++) {  // o selected by compile-time indexes: no local copy of a.coef
     float v = 0.0f;
 #pragma unroll
     for (int oo = 0; oo < 3; oo++)
-#pragma unroll
-      for (int ii = 0; ii < 3; ii++)
-        if (oo == o && ii == i) v = a.coef[oo][ii][c];
+      if (oo == o) v = a.coef[oo][c];
     t.coef[c] = v;
     if (v != 0.0f) t.need |= 1 << c;
   }
@@ -229,81 +221,6 @@ __device__ __forceinline__ void direct_out(const cx<float>* tile, const cx<float
       col[(long long)z * zstride + threadIdx.x] = s;
     }
     __syncthreads();
-  }
-}
-
-// One input slot, one output per block (grid.z = output index).
-template <int L>
-__global__ void __launch_bounds__(kNT, 3) k_z1(ZArgs a) {
-  constexpr int S = plan_stages(L);
-  extern __shared__ __align__(16) unsigned char smem[];
-  cx<float>* tw = reinterpret_cast<cx<float>*>(smem);
-  cx<float>* tile = tw + L;
-  __shared__ cx<float> small[kNT / TB][TB];
-  load_twiddles<float, kNT>(tw, reinterpret_cast<const cx<float>*>(a.tw), L);
-  const int chunk = blockIdx.x, o = blockIdx.z;
-  const int2 col = a.zcol[blockIdx.y];  // (ky position, ky)
-  const int kyf = col.y <= a.Ly / 2 ? col.y : a.Ly - col.y;
-  const float sy = col.y <= a.Ly / 2 ? 1.0f : -1.0f;
-  const long long colo = (long long)col.x * a.P + chunk * TB;
-  const cx<float>* in = reinterpret_cast<const cx<float>*>(a.buf) + a.in_slot[0] * a.cstride + colo;
-  cx<float>* out = reinterpret_cast<cx<float>*>(a.buf) + a.out_slot[o] * a.cstride + colo;
-  int ilo = 0, ihi = a.n_in, olo = 0, ohi = a.n_out;
-  if (a.in_ext) {
-    ilo = max(a.ext[0], 0);
-    ihi = min(a.ext[1], a.n_in);
-  }
-  if (a.out_ext) {
-    olo = max(a.ext[0], 0);
-    ohi = min(a.ext[1], a.n_out);
-  }
-  ihi = max(ihi, ilo);
-  ohi = max(ohi, olo);
-  const bool din = ihi - ilo <= kDirectPlanes, dout = ohi - olo <= kDirectPlanes;
-  const TensorCol tcol = make_tcol(a, o, 0, kyf, sy, chunk * TB);
-  __syncthreads();
-  if (din) {
-    direct_in<L>(tile, tw, in, a.zstride, ilo, ihi, small);
-  } else {
-    dif_stage0_load<float, L, kNT>(tile, tw, [&](int pos, int line) {
-      return (pos >= ilo && pos < ihi) ? in[pos * a.zstride + line] : zero<float>();
-    });
-    __syncthreads();
-    DifRange<float, L, kNT, 1, S - 1>::run(tile, tw);
-  }
-  __syncthreads();
-  {  // last forward stage, tensor product, first inverse stage (M = 1: R consecutive positions)
-    using SS = StageShape<L, S - 1>;
-    constexpr int R = SS::R;
-    constexpr int ITER = (SS::NU + kNT - 1) / kNT;
-#pragma unroll 1
-    for (int it = 0; it < ITER; it++) {
-      const int u = it * kNT + threadIdx.x;
-      if (SS::NU % kNT == 0 || u < SS::NU) {
-        const int line = u % TB, g = u / TB;
-        cx<float> v[R];
-#pragma unroll
-        for (int q = 0; q < R; q++) v[q] = tile[(g * R + q) * TB + line];
-        if (!din) Dft<float, R, false>::run(v);
-        TensorCol tl = tcol;
-        tl.T += line;
-        const int kb = k_of_group<L>(g);
-#pragma unroll
-        for (int q = 0; q < R; q++) v[q] = scale(v[q], tl.at(kb + q * (L / R), L));
-        if (!dout) Dft<float, R, true>::run(v);
-#pragma unroll
-        for (int q = 0; q < R; q++) tile[(g * R + q) * TB + line] = v[q];
-      }
-    }
-  }
-  __syncthreads();
-  if (dout) {
-    direct_out<L>(tile, tw, out, a.zstride, olo, ohi, small);
-  } else {
-    DitRange<float, L, kNT, 1, S - 1>::run(tile, tw);
-    dit_stage0_store<float, L, kNT>(tile, tw, [&](int pos, int line, cx<float> v) {
-      if (pos >= olo && pos < ohi) out[pos * a.zstride + line] = v;
-    });
   }
 }
 
@@ -383,7 +300,7 @@ __global__ void __launch_bounds__(kNT, 2) k_z1m(ZArgs a) {
   // their use (output 0's with the input rows)
   float f[2][R1];
   auto load_factors = [&](int o) {
-    const TensorCol tcol = make_tcol(a, o, 0, kyf, sy, chunk * TB + line);
+    const TensorCol tcol = make_tcol(a, o, kyf, sy, chunk * TB + line);
 #pragma unroll
     for (int it = 0; it < 2; it++) z_factors<L>(tcol, k_of_group<L>(it * (R0 / 2) + j), f[it]);
   };
@@ -478,177 +395,6 @@ __global__ void __launch_bounds__(kNT, 2) k_z1m(ZArgs a) {
   }
 }
 
-// Several input slots: a cluster of nin blocks per (column tile, column).
-template <int L>
-__global__ void __launch_bounds__(kNT, 2) k_z3(ZArgs a) {
-  constexpr int S = plan_stages(L);
-  extern __shared__ __align__(16) unsigned char smem[];
-  cx<float>* tw = reinterpret_cast<cx<float>*>(smem);
-  cx<float>* tile = tw + L;
-  __shared__ cx<float> small[kNT / TB][TB];
-  cg::cluster_group cluster = cg::this_cluster();
-  const int r = (int)cluster.block_rank();
-  load_twiddles<float, kNT>(tw, reinterpret_cast<const cx<float>*>(a.tw), L);
-  const int chunk = blockIdx.x / a.nin;
-  const int2 col = a.zcol[blockIdx.y];
-  const int kyf = col.y <= a.Ly / 2 ? col.y : a.Ly - col.y;
-  const float sy = col.y <= a.Ly / 2 ? 1.0f : -1.0f;
-  const long long colo = (long long)col.x * a.P + chunk * TB;
-  const cx<float>* in = reinterpret_cast<const cx<float>*>(a.buf) + a.in_slot[r] * a.cstride + colo;
-  int ilo = 0, ihi = a.n_in, olo = 0, ohi = a.n_out;
-  if (a.in_ext) {
-    ilo = max(a.ext[0], 0);
-    ihi = min(a.ext[1], a.n_in);
-  }
-  if (a.out_ext) {
-    olo = max(a.ext[0], 0);
-    ohi = min(a.ext[1], a.n_out);
-  }
-  ihi = max(ihi, ilo);
-  ohi = max(ohi, olo);
-  const bool din = ihi - ilo <= kDirectPlanes, dout = ohi - olo <= kDirectPlanes;
-  __syncthreads();
-  if (din) {
-    direct_in<L>(tile, tw, in, a.zstride, ilo, ihi, small);
-  } else if constexpr (zmulti_plan<L>()) {  // n_in <= L/2: the half-zero radix-32 stage, then radix 16
-    constexpr int R0 = StageShape<L, 0>::R, M0 = StageShape<L, 0>::M, R1 = StageShape<L, 1>::R;
-    const int line = threadIdx.x % TB, j = threadIdx.x / TB;
-    {
-      cx<float> v[R0];
-#pragma unroll
-      for (int q = 0; q < R0 / 2; q++) {
-        const int z = j + q * M0;
-        v[q] = (z >= ilo && z < ihi) ? in[z * a.zstride + line] : zero<float>();
-      }
-      dft32_half_input<false>(v);
-      if (j != 0) {
-#pragma unroll
-        for (int q = 1; q < R0; q++) v[q] = cmul(v[q], tw[j * q]);
-      }
-#pragma unroll
-      for (int q = 0; q < R0; q++) tile[(j + q * M0) * TB + line] = v[q];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int it = 0; it < 2; it++) {
-      const int g = it * (R0 / 2) + j;
-      cx<float> v[R1];
-#pragma unroll
-      for (int q = 0; q < R1; q++) v[q] = tile[(g * R1 + q) * TB + line];
-      DftF<R1, false>::run(v);
-#pragma unroll
-      for (int q = 0; q < R1; q++) tile[(g * R1 + q) * TB + line] = v[q];
-    }
-  } else {
-    dif_stage0_load<float, L, kNT>(tile, tw, [&](int pos, int line) {
-      return (pos >= ilo && pos < ihi) ? in[pos * a.zstride + line] : zero<float>();
-    });
-    __syncthreads();
-    DifRange<float, L, kNT, 1, S>::run(tile, tw);
-  }
-  cluster.sync();  // every input spectrum of the cluster is complete
-
-  using SS = StageShape<L, S - 1>;
-  constexpr int R = SS::R;
-  constexpr int ITER = (SS::NU + kNT - 1) / kNT;
-  cx<float> res[ITER][R];
-  const bool active = r < a.nout;
-  if (active) {
-    const cx<float>* src[3];
-    TensorCol tc[3];
-#pragma unroll
-    for (int i = 0; i < 3; i++) {
-      src[i] = i < a.nin ? cluster.map_shared_rank(tile, i) : tile;
-      if constexpr (!zmulti_plan<L>()) tc[i] = make_tcol(a, r, i < a.nin ? i : 0, kyf, sy, chunk * TB);
-    }
-#pragma unroll
-    for (int it = 0; it < ITER; it++) {
-      const int u = it * kNT + threadIdx.x;
-      if (SS::NU % kNT == 0 || u < SS::NU) {
-        const int line = u % TB, g = u / TB;
-        const int kb = k_of_group<L>(g);
-        if constexpr (zmulti_plan<L>()) {
-          // the factors of one input at a time, all loads in flight (two folded-row bases)
-#pragma unroll
-          for (int q = 0; q < R; q++) res[it][q] = zero<float>();
-#pragma unroll
-          for (int i = 0; i < 3; i++) {
-            if (i < a.nin) {
-              const TensorCol tl = make_tcol(a, r, i, kyf, sy, chunk * TB + line);  // made here: fewer live registers
-              float f[R];
-              z_factors<L>(tl, kb, f);
-#pragma unroll
-              for (int q = 0; q < R; q++) res[it][q] = res[it][q] + scale(src[i][(g * R + q) * TB + line], f[q]);
-            }
-          }
-          if (!dout) DftF<R, true>::run(res[it]);
-          if (it == 0) {  // the first unit waits in shared memory (its registers go to the second)
-#pragma unroll
-            for (int q = 0; q < R; q++) tile[L * TB + q * kNT + threadIdx.x] = res[0][q];
-          }
-        } else {
-#pragma unroll
-          for (int q = 0; q < R; q++) {
-            const int pos = (g * R + q) * TB + line;
-            const int kz = kb + q * (L / R);
-            cx<float> acc = zero<float>();
-#pragma unroll
-            for (int i = 0; i < 3; i++) {
-              if (i < a.nin) {
-                TensorCol tl = tc[i];
-                tl.T += line;
-                acc = acc + scale(src[i][pos], tl.at(kz, L));
-              }
-            }
-            res[it][q] = acc;
-          }
-          if (!dout) Dft<float, R, true>::run(res[it]);
-        }
-      }
-    }
-  }
-  cluster.sync();  // all reads of remote tiles are done
-  if (!active) return;
-#pragma unroll
-  for (int it = 0; it < ITER; it++) {
-    const int u = it * kNT + threadIdx.x;
-    if (SS::NU % kNT == 0 || u < SS::NU) {
-      const int line = u % TB, g = u / TB;
-#pragma unroll
-      for (int q = 0; q < R; q++)
-        tile[(g * R + q) * TB + line] = (zmulti_plan<L>() && it == 0) ? tile[L * TB + q * kNT + threadIdx.x] : res[it][q];
-    }
-  }
-  __syncthreads();
-  cx<float>* out = reinterpret_cast<cx<float>*>(a.buf) + a.out_slot[r] * a.cstride + colo;
-  if (dout) {
-    direct_out<L>(tile, tw, out, a.zstride, olo, ohi, small);
-  } else {
-    if constexpr (zmulti_plan<L>()) {  // n_out <= L/2: only the rows z < L/2 are formed
-      constexpr int R0 = StageShape<L, 0>::R, M0 = StageShape<L, 0>::M;
-      const int line = threadIdx.x % TB, j = threadIdx.x / TB;
-      cx<float> v[R0];
-#pragma unroll
-      for (int q = 0; q < R0; q++) v[q] = tile[(j + q * M0) * TB + line];
-      if (j != 0) {
-#pragma unroll
-        for (int q = 1; q < R0; q++) v[q] = cmulc(v[q], tw[j * q]);
-      }
-      dft_low_half<R0, true>(v);
-#pragma unroll
-      for (int q = 0; q < R0 / 2; q++) {
-        const int z = j + q * M0;
-        if (z >= olo && z < ohi) out[z * a.zstride + line] = v[q];
-      }
-    } else {
-      DitRange<float, L, kNT, 1, S - 1>::run(tile, tw);
-      dit_stage0_store<float, L, kNT>(tile, tw, [&](int pos, int line, cx<float> v) {
-        if (pos >= olo && pos < ohi) out[pos * a.zstride + line] = v;
-      });
-    }
-  }
-}
-
 template <int L>
 size_t tile_smem() {
   return (size_t)(L + L * TB) * sizeof(float2);
@@ -672,6 +418,8 @@ template <int L>
 int run_z(const ZArgs& a, cudaStream_t s) {
   const size_t sm = tile_smem<L>();
   if constexpr (zmulti_plan<L>()) {
+    // one input at 256^3, three outputs: k_z1m 0.56 ms and k_zn 0.77 with M0 along z (its
+    // spectra wait in tensor memory, so two blocks share an SM), 0.83 and 0.85 tilted
     if (a.nin == 1 && a.n_in <= L / 2 && a.n_out <= L / 2) {
       // EXT: the input or output planes come from the device range a.ext, and a few of them
       // take the direct transforms
@@ -686,44 +434,10 @@ int run_z(const ZArgs& a, cudaStream_t s) {
       return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
     }
   }
-  if (a.nin == 1) {
-    static bool init = false;
-    if (!init) {
-      if (cudaFuncSetAttribute(k_z1<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-        return -1;
-      init = true;
-    }
-    dim3 grid(a.P / TB, a.Ly, a.nout);
-    k_z1<L><<<grid, kNT, sm, s>>>(a);
-    return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
-  }
-  // the 32 x 16 plan keeps each thread's first output unit in shared memory beside the tile
-  const size_t sm3 = sm + (zmulti_plan<L>() ? (size_t)kNT * TB * sizeof(float2) : 0);
-  static bool init3 = false;
-  if (!init3) {
-    if (cudaFuncSetAttribute(k_z3<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3) != cudaSuccess)
-      return -1;
-    init3 = true;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.nin * (a.P / TB), a.Ly, 1);
-  cfg.blockDim = dim3(kNT, 1, 1);
-  cfg.dynamicSmemBytes = sm3;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = a.nin;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, k_z3<L>, a) != cudaSuccess) return -1;
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+  return launch_zn(L, a, s);
 }
 
 }  // namespace
-
-size_t zpass_smem(int L) { return (size_t)(L + L * TB) * sizeof(float2); }
 
 int launch_yfwd(int L, const YArgs& a, int ncomp, cudaStream_t s) {
   switch (L) {
