@@ -322,6 +322,23 @@ struct ConvSpec {
   int in_ext, out_ext;
 };
 
+// float copies of the vectors; returns the mask of the tensor components they use
+int product_vectors(const ConvSpec& cs, float u[3][3], float v[3][3]) {
+  int need = 0;
+  for (int o = 0; o < cs.nout; o++)
+    for (int i = 0; i < cs.nin; i++) {
+      float c6[6];
+      coef6(c6, cs.v[o], cs.u[i]);
+      for (int c = 0; c < 6; c++)
+        if (c6[c] != 0.0f) need |= 1 << c;
+    }
+  for (int c = 0; c < 3; c++) {
+    for (int i = 0; i < cs.nin; i++) u[i][c] = (float)cs.u[i][c];
+    for (int o = 0; o < cs.nout; o++) v[o][c] = (float)cs.v[o][c];
+  }
+  return need;
+}
+
 int conv_yz(tm_ctx* ctx, const ConvSpec& cs, int zin, int zout, cudaStream_t s) {
   const int Lx = ctx->L[0], Ly = ctx->L[1], Lz = ctx->L[2];
   const long long P = ctx->P;
@@ -361,21 +378,11 @@ int conv_yz(tm_ctx* ctx, const ConvSpec& cs, int zin, int zout, cudaStream_t s) 
   z.nin = cs.nin;
   z.nout = cs.nout;
   for (int i = 0; i < cs.nin; i++) z.in_slot[i] = cs.bin[i];
-  z.need = 0;
   for (int o = 0; o < cs.nout; o++) {
     z.out_slot[o] = cs.bout[o];
-    for (int i = 0; i < cs.nin; i++) {
-      float c6[6];
-      coef6(c6, cs.v[o], cs.u[i]);
-      for (int c = 0; c < 6; c++) {
-        if (c6[c] != 0.0f) z.need |= 1 << c;
-        if (i == 0) z.coef[o][c] = c6[c];
-      }
-    }
-    for (int c = 0; c < 3; c++) z.v[o][c] = (float)cs.v[o][c];
+    coef6(z.coef[o], cs.v[o], cs.u[0]);
   }
-  for (int i = 0; i < cs.nin; i++)
-    for (int c = 0; c < 3; c++) z.u[i][c] = (float)cs.u[i][c];
+  z.need = product_vectors(cs, z.u, z.v);
   z.T = ctx->T;
   z.Tz = (int)((Ly / 2 + 1) * P);
   z.Tc = (Lz / 2 + 1) * z.Tz;  // at most 289 * 289 * 304
@@ -457,18 +464,12 @@ int zdirect(tm_ctx* ctx, const ConvSpec& cs, int zi0, int nzi, int zo0, int nzo,
   z.nin = cs.nin;
   z.nout = cs.nout;
   for (int i = 0; i < cs.nin; i++) z.in_slot[i] = cs.bin[i];
-  for (int o = 0; o < cs.nout; o++) {
-    z.out_slot[o] = cs.bout[o];
-    for (int i = 0; i < cs.nin; i++) {
-      coef6(z.coef[o][i], cs.v[o], cs.u[i]);
-      z.need[o][i] = 0;
-      for (int c = 0; c < 6; c++)
-        if (z.coef[o][i][c] != 0.0f) z.need[o][i] |= 1 << c;
-    }
-  }
+  for (int o = 0; o < cs.nout; o++) z.out_slot[o] = cs.bout[o];
+  z.need = product_vectors(cs, z.u, z.v);
   z.Tz = ctx->Tz;
   z.Tdz = (long long)(Ly / 2 + 1) * P;
   z.Tc = (long long)ctx->nz * z.Tdz;
+  z.ndz = ctx->nz;
   z.zcol = ctx->zcol;
   z.zin0 = zi0;
   z.nzin = nzi;

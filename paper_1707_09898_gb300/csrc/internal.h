@@ -148,19 +148,22 @@ struct ZArgs {
 };
 constexpr int kDirectPlanes = 4;  // at most this many planes: direct DFT instead of the z FFT
 
-// Direct z convolution (few planes on one side), in place on B[slot][z][Ly][P].
+// Direct z convolution (few planes on one side), in place on B[slot][z][Ly][P]:
+// out_o(z) = sum_z' sum_i (v_o^T N~(z - z') u_i) in_i(z').
 constexpr int kDirectPlanesMax = 8;
 struct ZDirArgs {
   float2* buf;
   long long cstride, zstride;
   int P, Ly;
   int nin, nout, in_slot[3], out_slot[3];
-  float coef[3][3][6];
-  int need[3][3];
+  float u[3][3], v[3][3];
+  int need;               // bit c set if tensor component c is used
   const float* Tz;        // [6][nz][Ly/2+1][P], x/y transformed, z offset
   long long Tc, Tdz;      // per component, per offset
+  int ndz;                // offsets held (nz)
   const int2* zcol;
   int zin0, nzin, zout0, nzout;
+  int pdl;                // launch with programmatic dependent launch
 };
 int launch_zdir(const ZDirArgs& a, cudaStream_t s);
 

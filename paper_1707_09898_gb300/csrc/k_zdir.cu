@@ -10,6 +10,17 @@
 // instead of a forward and an inverse z FFT. The result is the same
 // convolution (no approximation). Columns are read with consecutive threads on
 // consecutive kx.
+//
+// Bytes bound it on large grids (inputs, outputs and the tensor rows each once), latency on
+// small ones. A block takes 32 kx of the columns ky and Ly - ky, which read the same tensor
+// rows, and splits z over its eight warps. Each z needs one new tensor row whatever the
+// number of planes: the offset of plane p at z + 1 is that of plane p - 1 at z, so the rows
+// move through registers. The tensor enters as t = N~ w with the vector of the side that has
+// one component (M0, or a unit vector), and its row is formed once for every plane, input
+// and output. Before, eight columns per block with no split along z and each factor from its
+// own masked loads: 26 us on the 39 x 39 x 41 grid with two planes (24 blocks), now 4; at 256^3, both
+// directions, one plane with three components 857 -> 247 us, varying M0 500 -> 453; four
+// planes 1540 -> 314 (one component), varying M0 7703 -> 778.
 #include "fft.cuh"
 #include "internal.h"
 
@@ -17,273 +28,206 @@ namespace tmk {
 
 namespace {
 
-// s = a - i b for one (o, i) pair at offset dz: a from the real components
-// (xx, yy, zz, xy), b from the imaginary ones (xz, yz: stored r with N~ = -i r).
-struct ZTensor {
-  const float* T;  // Tz + kyf * P + kx
-  long long Tc, Tdz;
-  float sy;
-  __device__ __forceinline__ void at(int dz, const float* coef, int need, float& a, float& b) const {
-    const int adz = dz < 0 ? -dz : dz;
-    const float sz = dz < 0 ? -1.0f : 1.0f;
-    const float* t = T + adz * Tdz;
-    a = 0.0f;
-    b = 0.0f;
-    if (need & 1) a += coef[0] * t[0];
-    if (need & 2) a += coef[1] * t[Tc];
-    if (need & 4) a += coef[2] * t[2 * Tc];
-    if (need & 8) a += coef[3] * sy * t[3 * Tc];
-    if (need & 16) b += coef[4] * sz * t[4 * Tc];
-    if (need & 32) b += coef[5] * sy * sz * t[5 * Tc];
-  }
+// One tensor row at one offset: the six components, signs of the odd ones (xz, yz in z; xy,
+// yz in y) and the factor -i of xz and yz included by the functions below.
+struct Row {
+  float n[6];
 };
 
-__device__ __forceinline__ cx<float> apply_s(cx<float> v, float a, float b) {
-  // (a - i b) v
-  return mk(a * v.x + b * v.y, a * v.y - b * v.x);
+// t = N~ w = re - i im for w on the column with y sign sy
+struct Vec {
+  float re[3], im[3];
+};
+__device__ __forceinline__ Vec apply_w(const Row& r, const float w[3], float sy) {
+  const float xy = sy * r.n[3], yz = sy * r.n[5];
+  Vec t;
+  t.re[0] = r.n[0] * w[0] + xy * w[1];
+  t.re[1] = xy * w[0] + r.n[1] * w[1];
+  t.re[2] = r.n[2] * w[2];
+  t.im[0] = r.n[4] * w[2];
+  t.im[1] = yz * w[2];
+  t.im[2] = r.n[4] * w[0] + yz * w[1];
+  return t;
+}
+// acc += (o . t) x
+__device__ __forceinline__ void add_dot(cx<float>& acc, const Vec& t, const float o[3], cx<float> x) {
+  const float re = o[0] * t.re[0] + o[1] * t.re[1] + o[2] * t.re[2];
+  const float im = o[0] * t.im[0] + o[1] * t.im[1] + o[2] * t.im[2];
+  acc.x = __fmaf_rn(im, x.y, __fmaf_rn(re, x.x, acc.x));
+  acc.y = __fmaf_rn(-im, x.x, __fmaf_rn(re, x.y, acc.y));
+}
+// acc += N~ x for the three components
+__device__ __forceinline__ void add_full(cx<float>* acc, const Row& r, float sy, const cx<float>* x) {
+  const float xy = sy * r.n[3], yz = sy * r.n[5], xz = r.n[4];
+  acc[0] = acc[0] + mk(r.n[0] * x[0].x + xy * x[1].x + xz * x[2].y, r.n[0] * x[0].y + xy * x[1].y - xz * x[2].x);
+  acc[1] = acc[1] + mk(xy * x[0].x + r.n[1] * x[1].x + yz * x[2].y, xy * x[0].y + r.n[1] * x[1].y - yz * x[2].x);
+  acc[2] = acc[2] + mk(xz * x[0].y + yz * x[1].y + r.n[2] * x[2].x, r.n[2] * x[2].y - xz * x[0].x - yz * x[1].x);
 }
 
-// One input, one output, one tensor component (the common case: constant M0 and
-// one weighted field component, or an axis-aligned M0): per streamed value one
-// load, one tensor load and one complex multiply-add, with running pointers.
-// c: the component; its coefficient and the column's sign are folded into `scale`.
-__global__ void __launch_bounds__(256) k_zdir_simple(ZDirArgs a, int c) {
-  // 32 kx x 2 columns x 4 z quarters per block
-  constexpr int ZS = 4;
-  const int kx = blockIdx.x * 32 + (threadIdx.x & 31);
-  const int part = (threadIdx.x >> 5) & (ZS - 1);
-  const int zc = blockIdx.y * 2 + (threadIdx.x >> 7);
-  __shared__ cx<float> red[2][ZS][32];
-  const bool valid = kx < a.P && zc < a.Ly;
-  const int2 col = valid ? a.zcol[zc] : make_int2(0, 0);
-  const bool lo = col.y <= a.Ly / 2;
-  const int kyf = lo ? col.y : a.Ly - col.y;
-  const bool imag = c >= 4;   // xz, yz: N~ = -i r
-  const bool odd_z = c >= 4;  // xz, yz change sign with dz
-  float scale = a.coef[0][0][c];
-  if ((c == 3 || c == 5) && !lo) scale = -scale;  // odd in y
-  const float* t = a.Tz + c * a.Tc + kyf * (long long)a.P + kx;
-  const long long colo = (long long)col.x * a.P + kx;
-  const cx<float>* in = reinterpret_cast<const cx<float>*>(a.buf) + a.in_slot[0] * a.cstride + colo;
-  cx<float>* out = reinterpret_cast<cx<float>*>(a.buf) + a.out_slot[0] * a.cstride + colo;
-  auto fac = [&](int dz) {
-    const int adz = dz < 0 ? -dz : dz;
-    float v = scale * t[adz * a.Tdz];
-    if (odd_z && dz < 0) v = -v;
-    return v;
+enum { ONE_IN = 0, ONE_OUT = 1, FULL = 2 };  // one input; several inputs, one output; three and three
+
+constexpr int ZP = 8;  // z parts per block, one warp each
+
+// Blocks per SM: more warps against more registers, hence loads, per thread. One plane at
+// 256^3, both directions: three and three 4 blocks 452 us, 5 470, 6 494, no bound 543; one to
+// one with tilted M0 no bound 119, 6 blocks 103.
+__host__ __device__ constexpr int blocks_per_sm(int np, int mode) {
+  return np == 1 ? (mode == FULL ? 4 : 6) : np == 2 ? 4 : np == 4 ? 2 : 1;
+}
+
+// NP: planes on the short side (at most). COLS: columns per thread (ky, Ly - ky).
+// NK: inputs (ONE_OUT), outputs (ONE_IN) held: 1 or 3.
+template <int NP, int COLS, int MODE, int NK>
+__global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const __grid_constant__ ZDirArgs a) {
+  constexpr int NI = MODE == ONE_IN ? 1 : NK, NO = MODE == ONE_OUT ? 1 : NK;
+  constexpr int UNR = MODE == FULL ? 1 : 2;  // z per round of loads; the others measured slower
+  __shared__ cx<float> red[ZP][NP][32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+  const int kx = blockIdx.x * 32 + lane;
+  const bool valid = kx < a.P;
+  // zcol holds ky = 0, then the pairs (ky, Ly - ky), then Ly / 2
+  const int c0 = COLS == 1 ? blockIdx.y : (blockIdx.y == 0 ? 0 : 2 * blockIdx.y - 1);
+  const int nc = COLS == 1 || blockIdx.y == 0 || c0 == a.Ly - 1 ? 1 : 2;
+  long long colo[COLS];
+  float sy[COLS];
+  int kyf = 0;
+#pragma unroll
+  for (int c = 0; c < COLS; c++) {
+    const int2 col = a.zcol[c0 + (c < nc ? c : 0)];
+    const bool lo = col.y <= a.Ly / 2;
+    kyf = lo ? col.y : a.Ly - col.y;
+    sy[c] = lo ? 1.0f : -1.0f;
+    colo[c] = (long long)col.x * a.P + kx;
+  }
+  const cx<float>* buf = reinterpret_cast<const cx<float>*>(a.buf);
+  cx<float>* obuf = reinterpret_cast<cx<float>*>(a.buf);
+  // A component that no product uses is read from the place of one that some product uses (its
+  // weights are zero): a test per load kept the loads of successive rows apart (varying M0
+  // at 256^3, one plane, both directions: 726 us with tests, 543 without).
+  const float* T = a.Tz + kyf * (long long)a.P + kx;
+  unsigned comp[6];
+#pragma unroll
+  for (int c = 0; c < 6; c++) comp[c] = (unsigned)((a.need & (1 << c) ? c : a.need ? __ffs(a.need) - 1 : 0) * a.Tc);
+  auto row = [&](int dz) {  // offsets past the stored ones belong to planes that are not wanted
+    Row r;
+    const unsigned at = (unsigned)(min(abs(dz), a.ndz - 1) * a.Tdz);
+#pragma unroll
+    for (int c = 0; c < 6; c++) r.n[c] = T[comp[c] + at];
+    if (dz < 0) {
+      r.n[4] = -r.n[4];
+      r.n[5] = -r.n[5];
+    }
+    return r;
   };
-  if (a.nzout == 1) {  // stream the inputs onto one output plane; quarters summed in order
-    const int zo = a.zout0;
-    const int per = (a.nzin + ZS - 1) / ZS;
+  // acc[o] += the contribution of the inputs x through row r
+  auto add = [&](cx<float>* acc, const Row& r, float s, const cx<float>* x) {
+    if constexpr (MODE == FULL) {
+      add_full(acc, r, s, x);
+    } else {
+      const Vec t = apply_w(r, MODE == ONE_IN ? a.u[0] : a.v[0], s);
+#pragma unroll
+      for (int k = 0; k < NK; k++)
+        add_dot(acc[MODE == ONE_IN ? k : 0], t, MODE == ONE_IN ? a.v[k] : a.u[k], x[MODE == ONE_IN ? 0 : k]);
+    }
+  };
+  if (a.nzout <= a.nzin) {  // few outputs: stream the inputs onto NP x NO sums
+    cx<float> acc[COLS][NP][NO];
+#pragma unroll
+    for (int c = 0; c < COLS; c++)
+#pragma unroll
+      for (int p = 0; p < NP; p++)
+#pragma unroll
+        for (int o = 0; o < NO; o++) acc[c][p][o] = zero<float>();
+    const int per = (a.nzin + ZP - 1) / ZP;
     const int z0 = a.zin0 + part * per, z1 = min(z0 + per, a.zin0 + a.nzin);
-    float ar = 0.0f, ai = 0.0f;
-    if (valid) {
-      const cx<float>* ip = in + (long long)z0 * a.zstride;
-#pragma unroll 8
+    if (valid && z0 < z1) {
+      Row r[NP];
+#pragma unroll
+      for (int p = 0; p < NP - 1; p++) r[p] = row(a.zout0 + p + 1 - z0);  // shifted into place below
+#pragma unroll UNR
       for (int z = z0; z < z1; z++) {
-        const cx<float> v = *ip;
-        ip += a.zstride;
-        const float f = fac(zo - z);
-        if (imag) {  // (-i f) v
-          ar += f * v.y;
-          ai -= f * v.x;
-        } else {
-          ar += f * v.x;
-          ai += f * v.y;
+#pragma unroll
+        for (int p = NP - 1; p > 0; p--) r[p] = r[p - 1];
+        r[0] = row(a.zout0 - z);
+#pragma unroll
+        for (int c = 0; c < COLS; c++) {
+          cx<float> x[NI];
+#pragma unroll
+          for (int i = 0; i < NI; i++)
+            x[i] = NI == 1 || i < a.nin ? buf[a.in_slot[i] * a.cstride + z * a.zstride + colo[c]] : zero<float>();
+#pragma unroll
+          for (int p = 0; p < NP; p++) add(acc[c][p], r[p], sy[c], x);
         }
       }
     }
-    red[threadIdx.x >> 7][part][threadIdx.x & 31] = mk(ar, ai);
-    __syncthreads();
-    if (part == 0 && valid) {
-      cx<float> s = red[threadIdx.x >> 7][0][threadIdx.x & 31];
-      for (int q = 1; q < ZS; q++) s = s + red[threadIdx.x >> 7][q][threadIdx.x & 31];
-      out[(long long)zo * a.zstride] = s;
-    }
-  } else {  // one input plane streamed onto every output plane; quarters of the planes
-    if (!valid) return;
-    const int zi = a.zin0;
-    const cx<float> v = in[(long long)zi * a.zstride];
-    const int per = (a.nzout + ZS - 1) / ZS;
-    const int z0 = a.zout0 + part * per, z1 = min(z0 + per, a.zout0 + a.nzout);
-    cx<float>* op = out + (long long)z0 * a.zstride;
-#pragma unroll 8
-    for (int z = z0; z < z1; z++) {
-      const float f = fac(z - zi);
-      *op = imag ? mk(f * v.y, -f * v.x) : mk(f * v.x, f * v.y);
-      op += a.zstride;
-    }
-  }
-}
-
-
-// Three inputs, three outputs with coefficients v_o = e_o, u_i = e_i (a spatially
-// varying M0: the magnetization enters and the field leaves component by component):
-// s_oi is the tensor component (o, i) itself, so per streamed column value the six
-// components are loaded once and out_o = sum_i N_oi in_i, with N_xz = -i b4 and
-// N_yz = -i b5 (odd in z; xy and yz odd in y). Same 4-way z split as k_zdir_simple.
-__device__ __forceinline__ void apply_n(const cx<float> in[3], const float t[6], cx<float> out[3]) {
-  // (-i b) v = (b v.y, -b v.x)
-  out[0] = mk(t[0] * in[0].x + t[3] * in[1].x + t[4] * in[2].y, t[0] * in[0].y + t[3] * in[1].y - t[4] * in[2].x);
-  out[1] = mk(t[3] * in[0].x + t[1] * in[1].x + t[5] * in[2].y, t[3] * in[0].y + t[1] * in[1].y - t[5] * in[2].x);
-  out[2] = mk(t[4] * in[0].y + t[5] * in[1].y + t[2] * in[2].x, -t[4] * in[0].x - t[5] * in[1].x + t[2] * in[2].y);
-}
-
-__global__ void __launch_bounds__(256) k_zdir_id(ZDirArgs a) {
-  constexpr int ZS = 4;
-  const int kx = blockIdx.x * 32 + (threadIdx.x & 31);
-  const int part = (threadIdx.x >> 5) & (ZS - 1);
-  const int zc = blockIdx.y * 2 + (threadIdx.x >> 7);
-  __shared__ cx<float> red[2][ZS][3][32];
-  const bool valid = kx < a.P && zc < a.Ly;
-  const int2 col = valid ? a.zcol[zc] : make_int2(0, 0);
-  const bool lo = col.y <= a.Ly / 2;
-  const int kyf = lo ? col.y : a.Ly - col.y;
-  const float sy = lo ? 1.0f : -1.0f;
-  const float* t0 = a.Tz + kyf * (long long)a.P + kx;
-  const long long colo = (long long)col.x * a.P + kx;
-  const cx<float>* buf = reinterpret_cast<const cx<float>*>(a.buf);
-  cx<float>* obuf = reinterpret_cast<cx<float>*>(a.buf);
-  auto tensor = [&](int dz, float t[6]) {
-    const int adz = dz < 0 ? -dz : dz;
-    const float sz = dz < 0 ? -1.0f : 1.0f;
-    const float* p = t0 + adz * a.Tdz;
 #pragma unroll
-    for (int c = 0; c < 6; c++) t[c] = p[c * a.Tc];
-    t[3] *= sy;
-    t[4] *= sz;
-    t[5] *= sy * sz;
-  };
-  if (a.nzout == 1) {  // stream the inputs onto one output plane; quarters summed in order
-    const int zo = a.zout0;
-    const int per = (a.nzin + ZS - 1) / ZS;
-    const int z0 = a.zin0 + part * per, z1 = min(z0 + per, a.zin0 + a.nzin);
-    cx<float> acc[3] = {zero<float>(), zero<float>(), zero<float>()};
-    if (valid) {
-#pragma unroll 4
-      for (int z = z0; z < z1; z++) {
-        cx<float> in[3];
+    for (int c = 0; c < COLS; c++)
 #pragma unroll
-        for (int i = 0; i < 3; i++) in[i] = buf[a.in_slot[i] * a.cstride + z * a.zstride + colo];
-        float t[6];
-        tensor(zo - z, t);
-        cx<float> o[3];
-        apply_n(in, t, o);
+      for (int o = 0; o < NO; o++) {  // the parts in order
+        if (c < nc && o < a.nout) {   // (the same for the whole block)
 #pragma unroll
-        for (int k = 0; k < 3; k++) acc[k] = acc[k] + o[k];
-      }
-    }
+          for (int p = 0; p < NP; p++) red[part][p][lane] = acc[c][p][o];
+          __syncthreads();
+          if (part < NP && part < a.nzout && valid) {
+            cx<float> s = red[0][part][lane];
 #pragma unroll
-    for (int k = 0; k < 3; k++) red[threadIdx.x >> 7][part][k][threadIdx.x & 31] = acc[k];
-    __syncthreads();
-    if (part == 0 && valid) {
-#pragma unroll
-      for (int k = 0; k < 3; k++) {
-        cx<float> sum = red[threadIdx.x >> 7][0][k][threadIdx.x & 31];
-        for (int q = 1; q < ZS; q++) sum = sum + red[threadIdx.x >> 7][q][k][threadIdx.x & 31];
-        obuf[a.out_slot[k] * a.cstride + zo * a.zstride + colo] = sum;
-      }
-    }
-  } else {  // one input plane onto every output plane; quarters of the planes
-    if (!valid) return;
-    const int zi = a.zin0;
-    cx<float> in[3];
-#pragma unroll
-    for (int i = 0; i < 3; i++) in[i] = buf[a.in_slot[i] * a.cstride + zi * a.zstride + colo];
-    const int per = (a.nzout + ZS - 1) / ZS;
-    const int z0 = a.zout0 + part * per, z1 = min(z0 + per, a.zout0 + a.nzout);
-#pragma unroll 4
-    for (int z = z0; z < z1; z++) {
-      float t[6];
-      tensor(z - zi, t);
-      cx<float> o[3];
-      apply_n(in, t, o);
-#pragma unroll
-      for (int k = 0; k < 3; k++) obuf[a.out_slot[k] * a.cstride + z * a.zstride + colo] = o[k];
-    }
-  }
-}
-
-template <int NP>
-__global__ void __launch_bounds__(256) k_zdir(ZDirArgs a) {
-  const int kx = blockIdx.x * 32 + (threadIdx.x & 31);
-  const int zc = blockIdx.y * 8 + (threadIdx.x >> 5);
-  if (kx >= a.P || zc >= a.Ly) return;
-  const int2 col = a.zcol[zc];
-  const int kyf = col.y <= a.Ly / 2 ? col.y : a.Ly - col.y;
-  ZTensor zt{a.Tz + kyf * (long long)a.P + kx, a.Tc, a.Tdz, col.y <= a.Ly / 2 ? 1.0f : -1.0f};
-  const long long colo = (long long)col.x * a.P + kx;
-  const cx<float>* buf = reinterpret_cast<const cx<float>*>(a.buf);
-  cx<float>* obuf = reinterpret_cast<cx<float>*>(a.buf);
-
-  if (a.nzout <= a.nzin) {  // few outputs: stream the inputs, keep NP x nout sums
-    cx<float> acc[3][NP];
-#pragma unroll
-    for (int o = 0; o < 3; o++)
-#pragma unroll
-      for (int p = 0; p < NP; p++) acc[o][p] = zero<float>();
-#pragma unroll 8
-    for (int z = a.zin0; z < a.zin0 + a.nzin; z++) {
-      cx<float> in[3];
-#pragma unroll
-      for (int i = 0; i < 3; i++)
-        if (i < a.nin) in[i] = buf[a.in_slot[i] * a.cstride + z * a.zstride + colo];
-#pragma unroll
-      for (int p = 0; p < NP; p++) {
-        if (p >= a.nzout) break;
-        const int dz = a.zout0 + p - z;
-#pragma unroll
-        for (int o = 0; o < 3; o++) {
-          if (o >= a.nout) break;
-#pragma unroll
-          for (int i = 0; i < 3; i++) {
-            if (i >= a.nin) break;
-            float sa, sb;
-            zt.at(dz, a.coef[o][i], a.need[o][i], sa, sb);
-            acc[o][p] = acc[o][p] + apply_s(in[i], sa, sb);
+            for (int q = 1; q < ZP; q++) s = s + red[q][part][lane];
+            obuf[a.out_slot[o] * a.cstride + (a.zout0 + part) * a.zstride + colo[c]] = s;
           }
+          __syncthreads();
         }
       }
-    }
-#pragma unroll
-    for (int p = 0; p < NP; p++) {
-      if (p >= a.nzout) break;
-#pragma unroll
-      for (int o = 0; o < 3; o++)
-        if (o < a.nout) obuf[a.out_slot[o] * a.cstride + (a.zout0 + p) * a.zstride + colo] = acc[o][p];
-    }
   } else {  // few inputs: keep them, stream the outputs
-    cx<float> in[3][NP];
+    if (!valid) return;
+    cx<float> x[COLS][NP][NI];
 #pragma unroll
-    for (int p = 0; p < NP; p++)
+    for (int c = 0; c < COLS; c++)
 #pragma unroll
-      for (int i = 0; i < 3; i++)
-        in[i][p] = (p < a.nzin && i < a.nin) ? buf[a.in_slot[i] * a.cstride + (a.zin0 + p) * a.zstride + colo]
-                                               : zero<float>();
-#pragma unroll 8
-    for (int z = a.zout0; z < a.zout0 + a.nzout; z++) {
-      cx<float> acc[3] = {zero<float>(), zero<float>(), zero<float>()};
+      for (int p = 0; p < NP; p++)
 #pragma unroll
-      for (int p = 0; p < NP; p++) {
-        if (p >= a.nzin) break;
-        const int dz = z - (a.zin0 + p);
+        for (int i = 0; i < NI; i++)
+          x[c][p][i] = p < a.nzin && (NI == 1 || i < a.nin)
+                           ? buf[a.in_slot[i] * a.cstride + (a.zin0 + p) * a.zstride + colo[c]]
+                           : zero<float>();
+    const int per = (a.nzout + ZP - 1) / ZP;
+    const int z0 = a.zout0 + part * per, z1 = min(z0 + per, a.zout0 + a.nzout);
+    if (z0 >= z1) return;
+    Row r[NP];
 #pragma unroll
-        for (int o = 0; o < 3; o++) {
-          if (o >= a.nout) break;
+    for (int p = 0; p < NP - 1; p++) r[p] = row(z0 - 1 - a.zin0 - p);  // shifted into place below
+#pragma unroll UNR
+    for (int z = z0; z < z1; z++) {
 #pragma unroll
-          for (int i = 0; i < 3; i++) {
-            if (i >= a.nin) break;
-            float sa, sb;
-            zt.at(dz, a.coef[o][i], a.need[o][i], sa, sb);
-            acc[o] = acc[o] + apply_s(in[i][p], sa, sb);
-          }
+      for (int p = NP - 1; p > 0; p--) r[p] = r[p - 1];
+      r[0] = row(z - a.zin0);
+#pragma unroll
+      for (int c = 0; c < COLS; c++) {
+        cx<float> acc[NO];
+#pragma unroll
+        for (int o = 0; o < NO; o++) acc[o] = zero<float>();
+#pragma unroll
+        for (int p = 0; p < NP; p++) add(acc, r[p], sy[c], x[c][p]);
+        if (c < nc) {
+#pragma unroll
+          for (int o = 0; o < NO; o++)
+            if (NO == 1 || o < a.nout) obuf[a.out_slot[o] * a.cstride + z * a.zstride + colo[c]] = acc[o];
         }
       }
-#pragma unroll
-      for (int o = 0; o < 3; o++)
-        if (o < a.nout) obuf[a.out_slot[o] * a.cstride + z * a.zstride + colo] = acc[o];
     }
   }
+}
+
+template <int NP, int COLS, int MODE, int NK>
+int run_zdir(const ZDirArgs& a, cudaStream_t s) {
+  const dim3 grid((a.P + 31) / 32, COLS == 1 ? a.Ly : a.Ly / 2 + 1);
+  return launch_k(k_zdir<NP, COLS, MODE, NK>, grid, dim3(32 * ZP), 0, s, a.pdl != 0, a) == cudaSuccess ? 0 : -1;
+}
+
+template <int NP, int COLS>
+int run_planes(const ZDirArgs& a, cudaStream_t s) {
+  if (a.nin == 1) return a.nout == 1 ? run_zdir<NP, COLS, ONE_IN, 1>(a, s) : run_zdir<NP, COLS, ONE_IN, 3>(a, s);
+  if (a.nout == 1) return run_zdir<NP, COLS, ONE_OUT, 3>(a, s);
+  return run_zdir<NP, COLS, FULL, 3>(a, s);
 }
 
 }  // namespace
@@ -292,35 +236,16 @@ int launch_zdir(const ZDirArgs& a, cudaStream_t s) {
   const int small = a.nzout <= a.nzin ? a.nzout : a.nzin;
   if (small < 0 || small > kDirectPlanesMax) return -2;
   if (small == 0) return 0;
-  dim3 grid((a.P + 31) / 32, (a.Ly + 7) / 8);
-  if (a.nin == 3 && a.nout == 3 && small == 1) {  // coefficients e_o^T N e_i: each the component (o, i)
-    bool id = true;
-    for (int o = 0; o < 3; o++)
-      for (int i = 0; i < 3; i++) {
-        const int c = o == i ? o : (o + i == 1 ? 3 : (o + i == 2 ? 4 : 5));
-        id = id && a.need[o][i] == (1 << c) && a.coef[o][i][c] == 1.0f;
-      }
-    if (id) {
-      k_zdir_id<<<dim3((a.P + 31) / 32, (a.Ly + 1) / 2), 256, 0, s>>>(a);
-      return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
-    }
+  if (a.nin > 1 && a.nout > 1) {  // the components go in and out: u_i = e_i, v_o = e_o
+    if (a.nin != 3 || a.nout != 3) return -2;
+    for (int k = 0; k < 3; k++)
+      for (int c = 0; c < 3; c++)
+        if (a.u[k][c] != (k == c ? 1.0f : 0.0f) || a.v[k][c] != (k == c ? 1.0f : 0.0f)) return -2;
   }
-  if (a.nin == 1 && a.nout == 1 && small == 1) {
-    const int need = a.need[0][0];
-    if (need != 0 && (need & (need - 1)) == 0) {
-      k_zdir_simple<<<dim3((a.P + 31) / 32, (a.Ly + 1) / 2), 256, 0, s>>>(a, __builtin_ctz(need));
-      return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
-    }
-  }
-  if (small == 1)
-    k_zdir<1><<<grid, 256, 0, s>>>(a);
-  else if (small == 2)
-    k_zdir<2><<<grid, 256, 0, s>>>(a);
-  else if (small <= 4)
-    k_zdir<4><<<grid, 256, 0, s>>>(a);
-  else
-    k_zdir<kDirectPlanesMax><<<grid, 256, 0, s>>>(a);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+  if (small == 1) return run_planes<1, 2>(a, s);
+  if (small == 2) return run_planes<2, 2>(a, s);
+  if (small <= 4) return run_planes<4, 2>(a, s);
+  return run_planes<kDirectPlanesMax, 1>(a, s);  // two columns would not fit in registers
 }
 
 }  // namespace tmk

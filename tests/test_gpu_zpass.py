@@ -92,3 +92,29 @@ def test_one_shot_planes(Lz, nz, z0, z1):
         J, G = m.objective_and_gradient(up(rho), up(mask), Ht=up(Ht), w=w)
         assert abs(J - Jr) <= 1e-5 * abs(Jr)
         assert rel(G.cpu().numpy(), Gr) <= 1e-5
+
+
+@pytest.mark.parametrize("n,nzd,z0,np_", [((9, 6, 13), 10, 12, 1), ((9, 6, 13), 13, 4, 2), ((30, 7, 9), 9, 0, 3),
+                                          ((20, 16, 11), 8, 6, 5), ((8, 8, 40), 33, 32, 8), ((36, 5, 4), 4, 0, 4)])
+def test_direct_planes(n, nzd, z0, np_):
+    """Prepared targets on one to eight planes (above, inside and below the design), one and
+    three components, constant and varying M0, fused with the y pass and not."""
+    from paper_1707_09898_gb300 import Magnet
+
+    nx, ny, nz = n
+    rho, gH, M0v = case(nx, ny, nz, nzd, nx + np_)
+    op = C.FFTOperator(C.Geometry(n, nzd, (1e-3,) * 3))
+    m = Magnet(n, nzd, (1e-3,) * 3, M0=tuple(TILTED), p=3.0, device=0)
+    mask = np.zeros((nz, ny, nx), np.uint8)
+    mask[z0:z0 + np_, 1:ny - 1, 1:nx - 2] = 1
+    Ht = (0.05 * W.MS * gH).astype(np.float32)
+    for M0 in (np.array([0.0, 0.0, W.MS]), TILTED, M0v):
+        m.set_M0(up(M0) if M0.ndim == 4 else tuple(M0))
+        for w in ((0.0, 0.0, 1.0), (1.0, 0.0, 0.5), (1.0, 0.5, 2.0)):
+            Jr, Gr, _ = O.objective_and_gradient(op, rho, M0, 3.0, mask, Ht, w)
+            m.set_target(up(mask), Ht=up(Ht), w=w)
+            for fused in (True, False):
+                m.set_fused(fused)
+                J, G = m.evaluate(up(rho))
+                assert abs(J - Jr) <= 1e-5 * abs(Jr)
+                assert rel(G.cpu().numpy(), Gr) <= 1e-5
