@@ -14,7 +14,6 @@
 //             the loader of the inverse transform and writes the real-y rows.
 // Same discrete convolution as the unfused passes, without the round trip of the
 // y spectra of all design planes through HBM.
-#include <cuda.h>  // CUtensorMap and its enums (the encoder is taken from the driver at run time)
 
 #include "fft.cuh"
 #include "internal.h"
@@ -820,24 +819,6 @@ int launch_adj(const ZYArgs& a, int c, cudaStream_t s) {
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
 
-// cuTensorMapEncodeTiled from the driver (no link-time dependency on libcuda)
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn encoder() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(f);
-  }
-  return fn;
-}
 // 2-D map over a row-major array of `outer` rows of `inner` elements, row pitch `pitch`
 // bytes, boxes of box_inner x box_outer elements; false if it cannot be encoded
 bool map_2d(CUtensorMap* m, CUtensorMapDataType type, const void* base, unsigned long long inner,

@@ -1,6 +1,6 @@
 // Tensor-memory-accelerator copies and mbarrier waits for the FFT passes (sm_103a).
 #pragma once
-#include <cuda.h>  // CUtensorMap (the type only)
+#include <cuda.h>  // CUtensorMap and its enums (the encoder is taken from the driver at run time)
 #include <cuda_runtime.h>
 
 namespace tmk {
@@ -22,6 +22,14 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::"r"(
           smem_u32(dst)),
       "l"(map), "r"(x), "r"(y), "r"(smem_u32(mb))
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, int c4,
+                                            unsigned long long* mb) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
+      "[%7];\n" ::"r"(smem_u32(dst)),
+      "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(mb))
       : "memory");
 }
 // Wait for phase `parity` of the barrier to complete: at most kSpin polls of about a
@@ -78,6 +86,22 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
                    smem_u32(dst)),
                "l"(src), "r"(bytes), "r"(smem_u32(mb))
                : "memory");
+}
+
+// cuTensorMapEncodeTiled from the driver (no link-time dependency on libcuda)
+using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn encoder() {
+  static const EncodeTiledFn fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    return cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+                   q == cudaDriverEntryPointSuccess
+               ? reinterpret_cast<EncodeTiledFn>(f)
+               : nullptr;
+  }();
+  return fn;
 }
 
 }  // namespace

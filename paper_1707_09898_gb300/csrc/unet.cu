@@ -260,22 +260,31 @@ int launch_conv_tc(const void* src, const bf16* Wc, const float* bias, void* dst
 }
 
 // Halo-tile implicit GEMM for grids whose rows hold W = 8, 16, 32 or 64 voxels (128 % W ==
-// 0). A block owns TZ = 2 planes of RY = 128 / W rows of one batch item: two M = 128 tiles,
-// tile m = the RY rows of plane z0 + m in (y, x) order, one tensor-memory lane per voxel.
-// Per 16-channel chunk of the reduced dimension, the (TZ + 2) x (RY + 2) rows around the
-// tiles are staged in shared memory once, as three copies shifted by dx = -1, 0, +1 (zero
-// where x + dx leaves the grid), each in the K-major core-matrix layout
-// [channel half][z][y][x][8 channels]: the A operand of tap (dz, dy, dx) for tile m is copy
-// dx from row (m + dz + 1, dy + 1) on (16-byte voxel rows, row groups 128 bytes apart, the
-// two channel halves one box apart), so all 27 taps read the same staged rows instead of
-// gathering them again. Each staged voxel's 8 channels are read from memory once: MODE 0
-// copies the unshifted rows asynchronously (all copies in flight) and builds the two
-// shifted copies from them in shared memory; MODE 1 loads the float32 output gradient,
-// rounds it to bfloat16 and stores it into the three copies. (TMA boxes of these 16-byte
-// rows measured slower: 86 us against 77 us on a 64^3 x 2 layer.)
-// The chunk's 27 packed weight blocks arrive by bulk copies (mbarrier completion). Thread 0
-// issues 27 x TZ MMAs per chunk (K = 16 each); the epilogue is that of k_conv_tc. Same
-// arithmetic as k_conv_tc: the same products, float32 sums in the tensor core's order.
+// 0). A tile is TZ planes of RY = 128 / W rows of one batch item: TZ MMA tiles of M = 128, the
+// RY rows of plane z0 + m in (y, x) order, one tensor-memory lane per voxel. A stage holds the
+// (TZ + 2) x (RY + 2) rows around a tile for 16 channels of the reduced dimension: MODE 0 as one
+// box copy brings them (32-byte rows, 32-byte swizzle, zero outside the grid), MODE 1 in the
+// K-major core-matrix layout [channel half][z][y][x][8 channels], the float32 output gradient
+// rounded to bfloat16 by the staging warps.
+// The three taps of a row, dx = -1, 0, +1, are columns of one MMA (N = 3 NO): the A operand of
+// a (dz, dy) pair is the staged rows from (m + dz + 1, dy + 1) on, unshifted, and the product
+// with W(dz, dy, dx) is accumulated per dx; the epilogue adds the three, each taken from the
+// lane one voxel to its side (warp shuffles, and shared memory between the two warps of a
+// 64-voxel row; a voxel past the row's end is the zero padding). So 9 MMAs per stage and M
+// tile instead of 27, and no dx-shifted copies of the rows: an MMA of so few columns is bound
+// by reading A from shared memory (4 KB for M = 128, K = 16), and the copies were two thirds
+// of the staging.
+// One persistent block per SM, its warps specialized: staging (one thread for the box copies,
+// or four groups of two warps, a buffer each), one thread per M tile that issues the MMAs, one
+// that copies weights, and groups of four warps that read alternate accumulators (a ring in
+// tensor memory) and write the output, which for MODE 1 is one bulk copy per M tile; mbarriers
+// between them. The packed weights stay in shared memory where they fit, otherwise each stage
+// brings its chunk's.
+// Measured, 64^3 x 2: forward 48 -> 16 channels 139 -> 33 us, of which the MMAs' operand reads
+// are 16 (44 cycles for M = 128, N = 48); data gradient 16 -> 48 113 -> 70 us, bound by the
+// epilogue (60 us alone). Before: one block per two tiles, three shifted copies, 27 MMAs a chunk
+// and nothing overlapped inside a block. On the way: 9 MMAs without the pipeline 88 and 139,
+// rows staged by threads in MODE 0 59, 54 weight copies a chunk instead of one box 39.
 // compile-time loop: f(std::integral_constant<int, i>) for i in [B, E)
 template <int B, int E, class F>
 __device__ __forceinline__ void static_for(F&& f) {
@@ -284,7 +293,6 @@ __device__ __forceinline__ void static_for(F&& f) {
     static_for<B + 1, E>(f);
   }
 }
-constexpr int kPartSplit = 13;  // taps [0, 13) and [13, 27) go to two accumulators
 // Stage the rows (z0 - 1 + r / RP, y0 - 1 + r % RP), r < ROWS, of batch item n, channels
 // [c0, c0 + 16), into three copies shifted by dx = -1, 0, +1 in the K-major core-matrix
 // layout [copy][channel half][r][x][8 channels] (copy c holds x + c - 1 at position x; zero
@@ -324,213 +332,454 @@ __device__ __forceinline__ void stage_halo_finish(unsigned char* As) {
   }
 }
 
-template <int W>
+template <int MODE, int W, int TZ, int NO>
 struct Halo {
-  static constexpr int RY = 128 / W, TZ = 2, ROWS = (TZ + 2) * (RY + 2);
-  static constexpr int BOX = 16 * W * ROWS;  // bytes of one channel half of one copy
-  static constexpr int ABYTES = 6 * BOX;     // 3 copies x 2 halves
+  static constexpr int RY = 128 / W, ROWS = (TZ + 2) * (RY + 2);
+  static constexpr int BOX = 16 * W * ROWS;            // bytes of one channel half
+  static constexpr int ABYTES = 2 * BOX;               // of one stage's rows
+  static constexpr int BB = 27 * NO * 32;              // weights of one chunk
+  static constexpr int CS = 3 * NO;                    // tensor-memory columns per M tile
+  static constexpr int SLOTS = 512 / (TZ * CS) < 4 ? 512 / (TZ * CS) : 4;  // accumulators in the ring
+  static constexpr int SW = MODE == 0 ? 0 : 8;         // staging warps
+  static constexpr int EG = SLOTS >= 4 && MODE == 0 ? 4 : SLOTS > 1 ? 2 : 1;  // epilogue groups of four warps
+  // the data gradient's rows of an M tile are one contiguous piece of memory: staged in shared
+  // memory and written by one bulk copy
+  static constexpr int OBYTES = 128 * NO * 4;
+  static constexpr int THREADS = 32 * (SW + 4 * EG + TZ + 1 + (MODE == 0 ? 1 : 0));
+  static_assert(SLOTS >= 1 && BB % 128 == 0, "accumulators; 128-byte aligned weights");
 };
-template <int NO>
-__host__ __device__ constexpr int halo_cs() {  // tensor-memory columns per tile
-  return NO <= 32 ? 32 : (NO <= 64 ? 64 : 128);
+constexpr int kHaloStages = 4;
+constexpr size_t kHaloTail = 8 * 64 * 4 + 64 * 4 + (2 * kHaloStages + 2 * 4 + 1) * 8 + 16;
+// shared memory with ns stages: 256 bytes of slack to align the staged rows
+template <int MODE, int NO>
+__host__ __device__ constexpr bool halo_staged_out() {
+  return MODE == 1;
 }
-template <int W, int NO>
-constexpr size_t halo_smem() {  // 128 bytes of slack to align the staged rows
-  return 128 + (size_t)Halo<W>::ABYTES + 27 * NO * 32 + 2 * 8 + 16;
+template <int MODE, int W, int TZ, int NO>
+constexpr size_t halo_smem(int ns, bool resident, int nk) {
+  using HT = Halo<MODE, W, TZ, NO>;
+  return 256 + (halo_staged_out<MODE, NO>() ? (size_t)HT::EG * HT::OBYTES : 0) + (size_t)ns * (HT::ABYTES + (resident ? 0 : HT::BB)) + (resident ? (size_t)nk * HT::BB : 0) + kHaloTail;
 }
-template <int MODE, int W, int NO>
-__global__ void __launch_bounds__(128) k_conv_halo(const void* src, const bf16* Wc, const float* bias, void* dst,
-                                                   int Nb, int D, int H, int KC, int flag) {
+// contiguous bulk copy shared -> global (16-byte aligned, size a multiple of 16), and the wait
+// until this thread's copies have read shared memory
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, unsigned bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n cp.async.bulk.commit_group;\n" ::"l"(dst),
+               "r"(tmk::smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_store_wait() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
+__device__ __forceinline__ void mbar_arrive(unsigned long long* mb) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tmk::smem_u32(mb)) : "memory");
+}
+
+template <int MODE, int W, int TZ, int NO>
+__global__ void __launch_bounds__(Halo<MODE, W, TZ, NO>::THREADS, 1)
+k_conv_halo(const __grid_constant__ CUtensorMap rows, const __grid_constant__ CUtensorMap wts, const void* src,
+            const float* bias, void* dst, int Nb, int D, int H, int KC, int NT,
+            int ns, int resident, int flag) {
   using namespace tmk;
-  using HT = Halo<W>;
-  constexpr int RY = HT::RY, TZ = HT::TZ, ROWS = HT::ROWS, BOX = HT::BOX, BB = NO * 32, CS = halo_cs<NO>();
-  constexpr unsigned NCOLS = 2 * TZ * CS;  // two accumulators (tap parts) per tile
-  constexpr unsigned IDESC = idesc_bf16(128, NO);
+  using HT = Halo<MODE, W, TZ, NO>;
+  constexpr int RY = HT::RY, ROWS = HT::ROWS, BOX = HT::BOX, ABYTES = HT::ABYTES, BB = HT::BB, CS = HT::CS;
+  constexpr int SLOTS = HT::SLOTS, EG = HT::EG;
+  constexpr unsigned IDESC = idesc_bf16(128, CS);
   extern __shared__ unsigned char smem_raw[];
-  unsigned char* As = smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127);  // [copy][half][z][y][x][16 B]
-  unsigned char* Bs = As + HT::ABYTES;                                         // [tap][2][NO/8][8][16 B]
-  unsigned long long* tma_bar = reinterpret_cast<unsigned long long*>(Bs + 27 * BB);
-  unsigned long long* mma_bar = tma_bar + 1;
-  unsigned* tslot = reinterpret_cast<unsigned*>(mma_bar + 1);
-  const int t = threadIdx.x, warp = t >> 5;
-  const int nyt = (H + RY - 1) / RY, nzt = (D + TZ - 1) / TZ;
-  const int yt = blockIdx.x % nyt, zt = (blockIdx.x / nyt) % nzt, n = blockIdx.x / (nyt * nzt);
-  const int y0 = yt * RY, z0 = zt * TZ;
+  // MODE 0: [stage][z][y][x][32 B], the halves of rows 4 .. 7 of every eight exchanged (32-byte
+  // swizzle); MODE 1: [stage][half][z][y][x][16 B]
+  unsigned char* As = smem_raw + ((256 - (smem_u32(smem_raw) & 255)) & 255);
+  const int nk = KC >> 4;
+  unsigned char* Bs = As + ns * ABYTES;  // [stage or chunk][dz dy][k half][dx][NO/8][8][16 B]
+  float* xs = reinterpret_cast<float*>(Bs + (resident ? nk : ns) * BB + (halo_staged_out<MODE, NO>() ? EG * HT::OBYTES : 0));  // [group][parity][row][voxel 31, 32][16] (W = 64)
+  float* bs = xs + 8 * 64;  // the bias (MODE 0)
+  unsigned long long* full = reinterpret_cast<unsigned long long*>(bs + 64);
+  unsigned long long *empty = full + kHaloStages, *accfull = empty + kHaloStages, *accempty = accfull + 4,
+                     *wbar = accempty + 4;
+  unsigned* tslot = reinterpret_cast<unsigned*>(wbar + 1);
+  constexpr bool STAGED = halo_staged_out<MODE, NO>();
+  const bool staged = STAGED && NT == NO;
+  unsigned char* Os = As + ns * ABYTES + (resident ? nk : ns) * BB;  // [group][128 voxels][NO] (STAGED)
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  constexpr int SW = HT::SW, MMA0 = SW + 4 * EG, WARP_W = MMA0 + TZ;  // first issuing warp, the weights' warp
   if (t == 0) {
-    mbar_init(tma_bar, 1);
-    mbar_init(mma_bar, 2 * TZ);  // one commit per issuer
+    for (int k = 0; k < ns; k++) {
+      mbar_init(full + k, (MODE == 0 ? 1 : 64) + (resident ? 0 : 1));  // the staging group, and the weights' warp
+      mbar_init(empty + k, TZ);
+    }
+    for (int k = 0; k < SLOTS; k++) {
+      mbar_init(accfull + k, TZ);
+      mbar_init(accempty + k, 128);
+    }
+    mbar_init(wbar, 1);
     mbar_init_fence();
   }
-  if (warp == 0) {
-    tmem_alloc(tslot, NCOLS);
+  if (MODE == 0 && t < NO) bs[t] = bias ? bias[blockIdx.y * NO + t] : 0.0f;
+  if (warp == MMA0) {
+    tmem_alloc(tslot, 512);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const unsigned taddr = *tslot;
-  bool dead = false;
+  bool dead = false;  // a wait ran out: no further waits in this thread, results flagged
   auto wait = [&](unsigned long long* mb, unsigned parity) {
-    if (!dead) dead = !mbar_wait_limit(mb, parity, 1 << 16, &g_net_status);
+    if (!dead) dead = !mbar_wait_limit(mb, parity & 1, 1 << 16, &g_net_status);
   };
-  const int nk = KC >> 4;
-  for (int kc = 0; kc < nk; kc++) {
-    if (kc > 0) wait(mma_bar, (kc - 1) & 1);  // the MMAs of the previous chunk have read the buffers
-    if (t == 0) {
-      if (kc == 0) fence_proxy_async_global();  // the source was written by ordinary stores
-      fence_proxy_async_smem();
-      mbar_expect_tx(tma_bar, 27 * BB);
-      for (int tap = 0; tap < 27; tap++) bulk_load(Bs + tap * BB, Wc + ((long long)tap * nk + kc) * NO * 16, BB, tma_bar);
-    }
-    if constexpr (MODE == 0) {
-      stage_halo_issue<W, RY + 2, ROWS>(As, reinterpret_cast<const bf16*>(src), n, z0, y0, D, H, KC, kc * 16);
-      stage_halo_finish<W, ROWS>(As);
-    } else {
-      // (half, row, x) items, x fastest: the 8 float32 values of one voxel are read once,
-      // rounded to bfloat16 and stored into the copies that hold them (copy c has the value
-      // of x + c - 1 at position x); the loads of kBatch items are in flight together
-      constexpr int XW = W + 2, ITEMS = 2 * ROWS * XW, kBatch = 8;
-      constexpr int NV = MODE == 0 ? 1 : 2;  // 16-byte loads per item (MODE 1: 8 float32 values)
-      for (int i0 = 0; i0 < ITEMS; i0 += 128 * kBatch) {
-        uint4 raw[kBatch][NV];  // loaded first, converted after the batch's loads are issued
-#pragma unroll
-        for (int b = 0; b < kBatch; b++) {
-          const int i = i0 + b * 128 + t;
-          const int x = i % XW - 1, r = (i / XW) % ROWS, h = i / (XW * ROWS);
-          const int z = z0 - 1 + r / (RY + 2), y = y0 - 1 + r % (RY + 2);
-#pragma unroll
-          for (int v = 0; v < NV; v++) raw[b][v] = make_uint4(0u, 0u, 0u, 0u);
-          if (i < ITEMS && z >= 0 && z < D && y >= 0 && y < H && x >= 0 && x < W) {
-            const long long e = ((((long long)n * D + z) * H + y) * W + x) * KC + kc * 16 + h * 8;
-            const uint4* q = MODE == 0 ? reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(src) + e)
-                                       : reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(src) + e);
-#pragma unroll
-            for (int v = 0; v < NV; v++) raw[b][v] = q[v];
-          }
-        }
-#pragma unroll
-        for (int b = 0; b < kBatch; b++) {
-          const int i = i0 + b * 128 + t;
-          const int x = i % XW - 1, r = (i / XW) % ROWS, h = i / (XW * ROWS);
-          uint4 pk = raw[b][0];
-          if constexpr (MODE == 1) {
-            const float4 f0 = *reinterpret_cast<const float4*>(&raw[b][0]);
-            const float4 f1 = *reinterpret_cast<const float4*>(&raw[b][NV - 1]);
-            pk = make_uint4(pack2(f0.x, f0.y), pack2(f0.z, f0.w), pack2(f1.x, f1.y), pack2(f1.z, f1.w));
-          }
-#pragma unroll
-          for (int c = 0; c < 3; c++) {
-            const int xs = x + 1 - c;
-            if (i < ITEMS && xs >= 0 && xs < W)
-              *reinterpret_cast<uint4*>(As + (c * 2 + h) * BOX + (r * W + xs) * 16) = pk;
+  const int nyt = (H + RY - 1) / RY, nzt = (D + TZ - 1) / TZ;
+  const int ntiles = Nb * nzt * nyt;
+  // one chunk's weights, this block's window of output channels: one copy of a box that takes the
+  // packed blocks [tap][chunk][k half][NT/8][8][8] in the order [dz dy][k half][dx] (54 copies of
+  // NO x 16 bytes, issued by one thread, took 2 us a chunk)
+  auto load_weights = [&](unsigned char* b, int kc, unsigned long long* mb) {
+    tma_load_5d(b, &wts, blockIdx.y * (NO * 2), 0, 0, 0, kc, mb);
+  };
+  if (MODE == 0 && warp == WARP_W + 1) {
+    // ---- staging, MODE 0: one copy of a box of rows per stage, zero outside the grid
+    if (lane == 0) {
+      fence_proxy_async_global();  // the rows were written by ordinary stores
+      int s = 0;
+      unsigned phase = 0;
+      for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int yt = tile % nyt, zt = (tile / nyt) % nzt, n = tile / (nyt * nzt);
+        for (int kc = 0; kc < nk; kc++) {
+          if (phase > 0) wait(empty + s, phase - 1);
+          mbar_expect_tx(full + s, ABYTES);
+          tma_load_5d(As + s * ABYTES, &rows, kc * 16, 0, yt * RY - 1, zt * TZ - 1, n, full + s);
+          if (++s == ns) {
+            s = 0;
+            phase++;
           }
         }
       }
     }
-    fence_proxy_async_smem();  // the staged rows, written through the generic proxy, for the tensor core
-    __syncthreads();
-    if ((t & 31) == 0) {
-      // lane 0 of warp w issues the MMAs of tile m = w % TZ for the taps of part w / TZ into
-      // that part's own accumulator (the issue of one MMA takes tens of cycles, so four
-      // issuers work side by side; the epilogue adds the parts); descriptors are a base plus
-      // compile-time offsets (16-byte units; every address stays below 2^18 bytes)
-      const int m = warp % TZ, part = warp / TZ;
-      wait(tma_bar, kc & 1);
+  } else if (warp < SW) {
+    // ---- staging: group g of two warps fills buffer g (a group that took turns on several
+    // buffers could wait for an empty one two phases ahead of its barrier); two lanes per
+    // voxel, one per channel half
+    const int g = warp >> 1, tg = t & 63;
+    constexpr int VPR = 32;  // voxels per round of the group
+    constexpr int XP = W < VPR ? 1 : W / VPR, RPI = VPR / W < 1 ? 1 : VPR / W;  // rounds per row, rows per round
+    constexpr int RIT = (ROWS + RPI - 1) / RPI, ITER = RIT * XP;
+    const int h = tg & 1, xv = (tg >> 1) % W, r0 = (tg >> 1) / W;
+    const long long rowp = (long long)W * KC, planep = H * rowp;
+    int kc = g < ns ? g : nk;  // the group's next chunk, counted from the current tile's first
+    unsigned phase = 0;        // uses of the buffer so far
+    const int s = g;
+    unsigned char* as = As + s * ABYTES + h * BOX + xv * 16;
+    for (int tile = blockIdx.x; tile < ntiles && g < ns; tile += gridDim.x) {
+      if (kc < nk) {
+        const int yt = tile % nyt, zt = (tile / nyt) % nzt, n = tile / (nyt * nzt);
+        const int y0 = yt * RY - 1, z0 = zt * TZ - 1;
+        unsigned zok = 0, yok = 0;
+#pragma unroll
+        for (int q = 0; q < TZ + 2; q++) zok |= (unsigned)((unsigned)(z0 + q) < (unsigned)D) << q;
+#pragma unroll
+        for (int q = 0; q < RY + 2; q++) yok |= (unsigned)((unsigned)(y0 + q) < (unsigned)H) << q;
+        const long long base0 = (((long long)n * D + z0) * H + y0) * rowp + (long long)xv * KC + h * 8;
+        for (; kc < nk; kc += ns) {
+          if (phase > 0) wait(empty + s, phase - 1);
+          phase++;
+          const long long base = base0 + kc * 16;
+          auto row_of = [&](int it, int& r, int& zr, int& yr) {
+            r = (it / XP) * RPI + r0;
+            zr = r / (RY + 2);
+            yr = r % (RY + 2);
+          };
+          {
+            const float* in = reinterpret_cast<const float*>(src);
+            constexpr int BATCH = 8;  // rounds whose loads are in flight together
+#pragma unroll
+            for (int i0 = 0; i0 < ITER; i0 += BATCH) {
+              float4 f[BATCH][2];
+#pragma unroll
+              for (int b = 0; b < BATCH; b++) {
+                int r, zr, yr;
+                row_of(i0 + b, r, zr, yr);
+                f[b][0] = f[b][1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (i0 + b < ITER && r < ROWS && ((zok >> zr) & (yok >> yr) & 1)) {
+                  const float4* q = reinterpret_cast<const float4*>(in + base + zr * planep + yr * rowp +
+                                                                    ((i0 + b) % XP) * (VPR * KC));
+                  f[b][0] = q[0];
+                  f[b][1] = q[1];
+                }
+              }
+#pragma unroll
+              for (int b = 0; b < BATCH; b++) {
+                int r, zr, yr;
+                row_of(i0 + b, r, zr, yr);
+                if (i0 + b < ITER && (ROWS % RPI == 0 || r < ROWS))
+                  *reinterpret_cast<uint4*>(as + (r * W + ((i0 + b) % XP) * VPR) * 16) =
+                      make_uint4(pack2(f[b][0].x, f[b][0].y), pack2(f[b][0].z, f[b][0].w), pack2(f[b][1].x, f[b][1].y),
+                                 pack2(f[b][1].z, f[b][1].w));
+              }
+            }
+          }
+          fence_proxy_async_smem();  // the rows, written through the generic proxy, for the tensor core
+          mbar_arrive(full + s);
+        }
+      }
+      kc -= nk;
+    }
+  } else if (warp == WARP_W) {
+    // ---- weights: all chunks once, or each stage's chunk
+    if (lane == 0) {
+      fence_proxy_async_global();  // they were written by ordinary stores
+      if (resident) {
+        mbar_expect_tx(wbar, nk * BB);
+        for (int kc = 0; kc < nk; kc++) load_weights(Bs + kc * BB, kc, wbar);
+      } else {
+        int s = 0;
+        unsigned phase = 0;
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+          for (int kc = 0; kc < nk; kc++) {
+            if (phase > 0) wait(empty + s, phase - 1);
+            mbar_expect_tx(full + s, BB);
+            load_weights(Bs + s * BB, kc, full + s);
+            if (++s == ns) {
+              s = 0;
+              phase++;
+            }
+          }
+      }
+    }
+  } else if (warp >= MMA0) {
+    // ---- MMAs of M tile m: one thread
+    const int m = warp - MMA0;
+    if (lane == 0) {
+      if (resident) wait(wbar, 0);
+      // MODE 0: rows of 32 bytes in the 32-byte swizzle (layout type 6), eight rows 256 bytes
+      const uint64_t a00 = MODE == 0 ? smem_desc(As + m * (RY + 2) * W * 32, 16, 256) | (uint64_t)6 << 61
+                                     : smem_desc(As + m * (RY + 2) * W * 16, BOX, 128);
+      const uint64_t b00 = smem_desc(Bs, 3 * NO * 16, 128);
+      int u = 0, s = 0;
+      unsigned phase = 0;
+      for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, u++) {
+        const int slot = u % SLOTS;
+        if (u >= SLOTS) wait(accempty + slot, u / SLOTS - 1);
+        const unsigned acc = taddr + (slot * TZ + m) * CS;
+        for (int kc = 0; kc < nk; kc++) {
+          wait(full + s, phase);
+          tc_fence_after();
+          const uint64_t a0 = a00 + (unsigned)(s * (ABYTES >> 4)), b0 = b00 + (unsigned)((resident ? kc : s) * (BB >> 4));
+          static_for<0, 9>([&](auto pair_c) {
+            constexpr int pair = decltype(pair_c)::value, sg = MODE == 1 ? -1 : 1;
+            constexpr int dz = sg * (pair / 3 - 1), dy = sg * (pair % 3 - 1);
+            constexpr unsigned aoff = (unsigned)(((dz + 1) * (RY + 2) + dy + 1) * W) * (MODE == 0 ? 2 : 1);
+            tc_mma(acc, a0 + aoff, b0 + (unsigned)(pair * NO * 6), IDESC, kc > 0 || pair > 0);
+          });
+          tc_commit(empty + s);
+          if (++s == ns) {
+            s = 0;
+            phase++;
+          }
+        }
+        tc_commit(accfull + slot);
+      }
+    }
+  } else {
+    // ---- epilogue: group e takes accumulators e, e + EG, ..
+    const int e = (warp - SW) >> 2, w4 = warp & 3, v = w4 * 32 + lane, x = v % W;
+    const bool pl = x > 0, pr = x < W - 1;
+    unsigned step = 0;
+    int u = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, u++) {
+      if (u % EG != e) continue;
+      const int slot = u % SLOTS;
+      const int yt = tile % nyt, zt = (tile / nyt) % nzt, n = tile / (nyt * nzt);
+      const int y = yt * RY + v / W;
+      wait(accfull + slot, u / SLOTS);
+      __syncwarp();
       tc_fence_after();
-      const uint64_t a0 = smem_desc(As + m * (RY + 2) * W * 16, BOX, 128);
-      const uint64_t b0 = smem_desc(Bs, NO * 16, 128);
-      const unsigned acc = taddr + (part * TZ + m) * CS;
-      auto issue = [&](auto tap_c) {
-        constexpr int tap = decltype(tap_c)::value;
-        constexpr int sg = MODE == 1 ? -1 : 1;
-        constexpr int dz = sg * (tap / 9 - 1), dy = sg * ((tap / 3) % 3 - 1), dx = sg * (tap % 3 - 1);
-        constexpr unsigned aoff = (unsigned)((dx + 1) * 2 * BOX + ((dz + 1) * (RY + 2) + dy + 1) * W * 16) >> 4;
-        tc_mma(acc, a0 + aoff, b0 + (unsigned)(tap * BB >> 4), IDESC, kc > 0 || (tap != 0 && tap != kPartSplit));
-      };
-      if (part == 0) {
-        static_for<0, kPartSplit>(issue);
-      } else {
-        static_for<kPartSplit, 27>(issue);
+#pragma unroll 1
+      for (int m = 0; m < TZ; m++) {
+        const int z = zt * TZ + m;
+        const bool valid = z < D && y < H;
+        const long long o0 = ((((long long)n * D + z) * H + y) * W + x) * NT + blockIdx.y * NO;
+        const unsigned trow = taddr + ((unsigned)(w4 * 32) << 16) + (slot * TZ + m) * CS;
+        if (staged && (u != e || m > 0)) {  // the last copy has read the buffer
+          if (w4 == 0 && lane == 0) bulk_store_wait();
+          __syncwarp();
+          bar_named(5 + e, 128);
+        }
+#pragma unroll 1
+        for (int c0 = 0; c0 < NO; c0 += 16) {
+          // lf: the products of the voxel at x - 1, taken from its lane; rt: of the one at x + 1
+          float r[16], lf[16], rt[16];
+          tc_ld16(trow + (MODE == 0 ? 0 : 2) * NO + c0, lf);
+          tc_ld16(trow + NO + c0, r);
+          tc_ld16(trow + (MODE == 0 ? 2 : 0) * NO + c0, rt);
+          tc_wait_ld();
+          if (m == TZ - 1 && c0 == NO - 16) {  // the accumulator has been read
+            tc_fence_before();
+            mbar_arrive(accempty + slot);
+          }
+          if constexpr (W == 64) {  // voxels 31 and 32 of a row belong to two warps
+            float* xr = xs + (e * 2 + (step & 1)) * 64 + (w4 >> 1) * 32;  // the other parity may still be read
+            if ((w4 & 1) == 0 && lane == 31) {
+#pragma unroll
+              for (int i = 0; i < 4; i++)
+                reinterpret_cast<float4*>(xr)[i] = make_float4(lf[4 * i], lf[4 * i + 1], lf[4 * i + 2], lf[4 * i + 3]);
+            }
+            if ((w4 & 1) == 1 && lane == 0) {
+#pragma unroll
+              for (int i = 0; i < 4; i++)
+                reinterpret_cast<float4*>(xr + 16)[i] = make_float4(rt[4 * i], rt[4 * i + 1], rt[4 * i + 2], rt[4 * i + 3]);
+            }
+            __syncwarp();
+            bar_named(1 + e * 2 + (w4 >> 1), 64);
+            step++;
+#pragma unroll
+            for (int i = 0; i < 16; i++) {
+              const float a = __shfl_up_sync(0xffffffffu, lf[i], 1), b = __shfl_down_sync(0xffffffffu, rt[i], 1);
+              lf[i] = a;
+              rt[i] = b;
+            }
+            if ((w4 & 1) == 1 && lane == 0) {
+#pragma unroll
+              for (int i = 0; i < 4; i++) {
+                const float4 q = reinterpret_cast<const float4*>(xr)[i];
+                lf[4 * i] = q.x, lf[4 * i + 1] = q.y, lf[4 * i + 2] = q.z, lf[4 * i + 3] = q.w;
+              }
+            }
+            if ((w4 & 1) == 0 && lane == 31) {
+#pragma unroll
+              for (int i = 0; i < 4; i++) {
+                const float4 q = reinterpret_cast<const float4*>(xr + 16)[i];
+                rt[4 * i] = q.x, rt[4 * i + 1] = q.y, rt[4 * i + 2] = q.z, rt[4 * i + 3] = q.w;
+              }
+            }
+            __syncwarp();
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; i++) {
+              lf[i] = __shfl_up_sync(0xffffffffu, lf[i], 1);
+              rt[i] = __shfl_down_sync(0xffffffffu, rt[i], 1);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 16; i++) {
+            if (pl) r[i] += lf[i];
+            if (pr) r[i] += rt[i];
+          }
+          if (!valid) {
+          } else if constexpr (MODE == 0) {
+            uint32_t pk[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+              const float2 bb = *reinterpret_cast<const float2*>(bs + c0 + 2 * i);
+              float a = r[2 * i] + bb.x, b = r[2 * i + 1] + bb.y;
+              if (flag) {
+                a = fmaxf(a, 0.0f);
+                b = fmaxf(b, 0.0f);
+              }
+              pk[i] = pack2(a, b);
+            }
+            uint4* o = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(dst) + o0 + c0);
+            o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+          } else {
+            float4* o = reinterpret_cast<float4*>(reinterpret_cast<float*>(dst) + o0 + c0);
+            if (flag) {  // accumulate into an existing gradient
+#pragma unroll
+              for (int i = 0; i < 4; i++) {
+                const float4 old = o[i];
+                r[4 * i] += old.x, r[4 * i + 1] += old.y, r[4 * i + 2] += old.z, r[4 * i + 3] += old.w;
+              }
+            }
+            if (staged) o = reinterpret_cast<float4*>(Os + e * HT::OBYTES + (v * NO + c0) * 4);
+#pragma unroll
+            for (int i = 0; i < 4; i++) o[i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+          }
+          __syncwarp();
+        }
+        if (staged) {  // one bulk copy of the M tile's rows that lie in the grid
+          fence_proxy_async_smem();
+          bar_named(5 + e, 128);
+          const int rows = z < D ? min(RY, H - yt * RY) : 0;
+          if (w4 == 0 && lane == 0 && rows > 0)
+            bulk_store(reinterpret_cast<float*>(dst) + ((((long long)n * D + z) * H + yt * RY) * W) * NO, Os + e * HT::OBYTES,
+                       rows * W * NO * 4);
+        }
       }
-      tc_commit(mma_bar);
     }
   }
-  wait(mma_bar, (nk - 1) & 1);  // every MMA has completed
-  tc_fence_after();
-  const unsigned trow = taddr + ((unsigned)(warp * 32) << 16);
-  const int y = y0 + t / W, x = t % W;
-#pragma unroll
-  for (int m = 0; m < TZ; m++) {
-    const int z = z0 + m;
-    const bool valid = z < D && y < H;
-    const long long v = (((long long)n * D + z) * H + y) * W + x;
-#pragma unroll
-    for (int c0 = 0; c0 < NO; c0 += 16) {
-      float r[16], r2[16];
-      tc_ld16(trow + m * CS + c0, r);
-      tc_ld16(trow + (TZ + m) * CS + c0, r2);
-      tc_wait_ld();
-      if (!valid) continue;
-#pragma unroll
-      for (int i = 0; i < 16; i++) r[i] += r2[i];  // taps 0 .. 12 and 13 .. 26
-      if constexpr (MODE == 0) {
-        uint32_t pk[8];
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-          float o0 = r[2 * i], o1 = r[2 * i + 1];
-          if (bias) {
-            o0 += bias[c0 + 2 * i];
-            o1 += bias[c0 + 2 * i + 1];
-          }
-          if (flag) {
-            o0 = fmaxf(o0, 0.0f);
-            o1 = fmaxf(o1, 0.0f);
-          }
-          pk[i] = pack2(o0, o1);
-        }
-        uint4* o = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(dst) + v * NO + c0);
-        o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-        o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-      } else {
-        float4* o = reinterpret_cast<float4*>(reinterpret_cast<float*>(dst) + v * NO + c0);
-#pragma unroll
-        for (int i = 0; i < 4; i++) {
-          float4 w = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-          if (flag) {  // accumulate into an existing gradient
-            const float4 e = o[i];
-            w.x += e.x;
-            w.y += e.y;
-            w.z += e.z;
-            w.w += e.w;
-          }
-          o[i] = w;
-        }
-      }
-    }
-  }
+  if (staged && (t & 31) == 0) bulk_store_wait();
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(taddr, NCOLS);
+  if (warp == MMA0) {
+    tc_fence_after();
+    tmem_dealloc(taddr, 512);
+  }
 }
 
-template <int MODE, int W, int NO>
-int launch_conv_halo(const void* src, const bf16* Wc, const float* bias, void* dst, int Nb, int D, int H, int KC,
-                     int flag, cudaStream_t s) {
-  using HT = Halo<W>;
-  constexpr size_t sm = halo_smem<W, NO>();
-  static_assert(sm <= 227 * 1024, "shared memory of one block");
+int sm_count() {  // of the current device
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 148;
+  return n > 0 ? n : 148;
+}
+
+template <int MODE, int W, int TZ, int NO>
+int launch_conv_halo_tz(const void* src, const bf16* Wc, const float* bias, void* dst, int Nb, int D, int H, int KC,
+                        int NT, int flag, cudaStream_t s) {
+  using HT = Halo<MODE, W, TZ, NO>;
+  constexpr size_t kMost = 227 * 1024;
+  const int nk = KC >> 4;
+  // weights resident if they leave room for three stages of rows; at least two stages either way
+  const bool resident = halo_smem<MODE, W, TZ, NO>(3, true, nk) <= kMost;
+  int ns = kHaloStages;
+  while (ns > 2 && halo_smem<MODE, W, TZ, NO>(ns, resident, nk) > kMost) ns--;
+  const size_t sm = halo_smem<MODE, W, TZ, NO>(ns, resident, nk);
+  static_assert(halo_smem<MODE, W, TZ, NO>(2, false, 1) <= kMost, "shared memory of one block");
   static bool init = false;
   if (!init) {
-    if (cudaFuncSetAttribute(k_conv_halo<MODE, W, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
+    if (cudaFuncSetAttribute(k_conv_halo<MODE, W, TZ, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost) !=
         cudaSuccess)
       return -4;
     init = true;
   }
-  const long long blocks = (long long)Nb * ((D + HT::TZ - 1) / HT::TZ) * ((H + HT::RY - 1) / HT::RY);
-  if (blocks > 0x7fffffffLL) return -1;
-  if (blocks > 0)
-    k_conv_halo<MODE, W, NO><<<(unsigned)blocks, 128, sm, s>>>(src, Wc, bias, dst, Nb, D, H, KC, flag);
+  const long long tiles = (long long)Nb * ((D + TZ - 1) / TZ) * ((H + HT::RY - 1) / HT::RY);
+  if (tiles > 0x7fffffffLL) return -1;
+  if (tiles <= 0) return 0;
+  CUtensorMap rows = {}, wts = {};
+  tmk::EncodeTiledFn fn = tmk::encoder();
+  if (!fn) return -4;
+  {  // in units of 8 bytes: channel groups, dx, k half, (dz, dy), chunk
+    const cuuint64_t dims[5] = {2ull * NT, 3, 2, 9, (cuuint64_t)nk};
+    const cuuint64_t pitch[4] = {32ull * NT * nk, 16ull * NT, 96ull * NT * nk, 32ull * NT};
+    const cuuint32_t box[5] = {2 * NO, 3, 2, 9, 1}, step[5] = {1, 1, 1, 1, 1};
+    if (fn(&wts, CU_TENSOR_MAP_DATA_TYPE_UINT64, 5, const_cast<bf16*>(Wc), dims, pitch, box, step,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return -4;
+  }
+  if (MODE == 0) {
+    const cuuint64_t dims[5] = {(cuuint64_t)KC, W, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)Nb};
+    const cuuint64_t pitch[4] = {2ull * KC, 2ull * KC * W, 2ull * KC * W * H, 2ull * KC * W * H * D};
+    const cuuint32_t box[5] = {16, W, HT::RY + 2, TZ + 2, 1}, step[5] = {1, 1, 1, 1, 1};
+    if (fn(&rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(src), dims, pitch, box, step,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return -4;
+  }
+  const int windows = NT / NO, gx = sm_count() / windows;  // one block per SM
+  k_conv_halo<MODE, W, TZ, NO><<<dim3((unsigned)(tiles < gx ? tiles : gx), windows), HT::THREADS, sm, s>>>(
+        rows, wts, src, bias, dst, Nb, D, H, KC, NT, ns, resident, flag);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
+}
+// Two planes per tile read each staged row for more of its taps, as far as two accumulators fit
+// in tensor memory; one plane where two would leave SMs without a tile (16^3 x 2). 96 channels
+// go as two windows of 48 on their own blocks: their accumulator alone would be 288 columns
+// wide, so that no epilogue could run beside the next tile's MMAs.
+template <int MODE, int W, int NO>
+int launch_conv_halo(const void* src, const bf16* Wc, const float* bias, void* dst, int Nb, int D, int H, int KC,
+                     int flag, cudaStream_t s) {
+  constexpr int NW = NO == 96 ? 48 : NO;
+  if constexpr (NW <= 32) {
+    if ((long long)Nb * ((D + 1) / 2) * ((H + 128 / W - 1) / (128 / W)) >= sm_count())
+      return launch_conv_halo_tz<MODE, W, 2, NW>(src, Wc, bias, dst, Nb, D, H, KC, NO, flag, s);
+  }
+  return launch_conv_halo_tz<MODE, W, 1, NW>(src, Wc, bias, dst, Nb, D, H, KC, NO, flag, s);
 }
 
 // the halo kernel for rows of 8 .. 64 voxels, else the per-voxel gather kernel
@@ -1124,12 +1373,7 @@ int tmn_conv3d_backward_weight(const void* in, const float* dout, float* dW, flo
   if (nvox < 1) return -1;
   if (work_floats < tmn_conv3d_backward_weight_work(nvox, Cin, Cout)) return -5;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  static int nsm = 0;
-  if (!nsm) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 148;
-  }
+  const int nsm = sm_count();
   if ((W == 8 || W == 16 || W == 32 || W == 64) && (reinterpret_cast<uintptr_t>(in) & 15) == 0) {
     // halo tiles: one persistent block per SM, as many as the work buffer holds partials for
     const long long per = 27LL * Cin * Cout, ntl = (long long)N * D * ((H + 128 / W - 1) / (128 / W));
