@@ -11,9 +11,9 @@
 // 3x3x3 convolutions (stride 1, zero padding 1), forward, data gradient and weight
 // gradient, are implicit GEMMs on the fifth-generation tensor cores (tcgen05.mma,
 // bfloat16 operands, float32 accumulators in tensor memory): k_conv_halo (rows of 8..64
-// voxels: halo rows staged once per block), k_conv_tc (any grid: per-voxel gathers) and
-// k_conv_dw_tc (weight gradient, the output gradient rounded to bfloat16 as in the data
-// gradient).
+// voxels: staged halo rows, a warp-specialized pipeline) and k_conv_dw_rows (their weight
+// gradient, rows of 16..64), k_conv_dw_halo (rows of 8), k_conv_tc and k_conv_dw_tc (any grid:
+// per-voxel gathers). The output gradient is rounded to bfloat16 where it is an operand.
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -951,7 +951,276 @@ __global__ void __launch_bounds__(128) k_conv_dw_tc(const bf16* in, const bf16* 
   if (warp == 0) tmem_dealloc(taddr, NCOLS);
 }
 
-// Weight gradient for rows of 8..64 voxels (128 % W == 0): dW[tap][ci][co] =
+// Weight gradient for rows of 16, 32 or 64 voxels: dW[tap][ci][co] =
+// sum_v in[v + off(tap)][ci] q(dout[v][co]) as MMAs with K = 16 voxels of one row of dout, M = 8
+// input rows x 16 channels and N = 3 NO, the output channels for the three dx. A tile is TZ
+// planes of RT rows; a stage holds the (TZ + 2) x (RT + 2) input rows around it for one
+// 16-channel chunk, [z][y][x][16 channels] in the 32-byte swizzle as one box copy brings them.
+// Read as an MN-major operand, the rows from (z, y) on are M groups one row apart: with PR = RT
+// + 2 rows per plane, the input row of (dz, dy) is group dz PR + dy, so two MMAs of M = 128
+// (groups 0-7 and 8-15) hold all nine for every row of the tile; the groups between are
+// products that nothing reads. The output gradient, rounded to bfloat16, lies in shared memory
+// as [row][dx][8 channels][x], dx-shifted (zero past the row's ends), which makes dx part of N.
+// So each MMA does 9/16 x 128 x 48 useful products for NO = 16, where M = 16 output channels
+// padded to 128 against N = 48 did an eighth of its columns' work and 9 MMAs per 16 voxels.
+// One persistent block per SM: one thread copies input rows, eight warps round and store the
+// output gradient (and add up the bias gradient from the float32 values they read), one thread
+// per M tile issues MMAs; the accumulators stay in tensor memory over all tiles of the block.
+// Channel chunks go in groups of 512 / (6 NO), each on its own blocks. Each block writes its
+// sums as one partial, added in block order by k_dw_finish.
+// What bounds it: reading the operands of the MMAs from shared memory (44 cycles for M = 128, N =
+// 48, K = 16). Measured, 64^3 x 2, 48 -> 16 channels with db: 432 -> 49 us.
+template <int W, int NO>
+struct DwRows {
+  static constexpr int ROWB = 6 * NO * W;                     // bytes of one staged output-gradient row
+  static constexpr int MAXR = 50 * 1024 / ROWB;               // rows of a tile, two buffers of them
+  static constexpr int TZ = MAXR >= 8 ? 2 : 1, RT = MAXR >= 4 ? 4 : 2;
+  static constexpr int PR = RT + 2, DROWS = TZ * RT;
+  static constexpr int ABYTES = (TZ + 2) * PR * W * 32;       // one stage of input rows
+  static constexpr int GBYTES = DROWS * ROWB;                 // one buffer of output-gradient rows
+  static constexpr int NS = 2 * ABYTES + 2 * GBYTES > 150 * 1024 ? 2 : 3;
+  static constexpr int GROUP = 512 / (6 * NO);                // channel chunks per block
+  static constexpr int THREADS = 256 + 64 + 32;
+  // the second M tile of the last row reads up to 16 rows past its first: they stay inside
+  static constexpr size_t SMEM = 256 + (size_t)NS * ABYTES + 2 * GBYTES + 256 * 8 * 4 + (2 * NS + 5) * 8 + 16;
+  static_assert(MAXR >= 2 && GROUP >= 1 && 2 * PR + 2 <= 15 && SMEM <= 227 * 1024, "tile");
+  static_assert(2 * GBYTES + 256 * 8 * 4 >= 8 * W * 32, "rows read past the stages");
+};
+template <int W, int NO>
+__global__ void __launch_bounds__(DwRows<W, NO>::THREADS, 1)
+k_conv_dw_rows(const __grid_constant__ CUtensorMap rows, const float* dout, float* part, int Nb, int D, int H, int Cin) {
+  using namespace tmk;
+  using T = DwRows<W, NO>;
+  constexpr int TZ = T::TZ, RT = T::RT, PR = T::PR, DROWS = T::DROWS, ROWB = T::ROWB, NS = T::NS, CG = NO / 8;
+  constexpr unsigned IDESC = idesc_bf16(128, 3 * NO, true);
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* As = smem_raw + ((256 - (smem_u32(smem_raw) & 255)) & 255);  // [stage][z][y][x][32 B], swizzled
+  unsigned char* Gs = As + NS * T::ABYTES;                                     // [buffer][row][dx][CG][x][16 B]
+  float* dbs = reinterpret_cast<float*>(Gs + 2 * T::GBYTES);                   // [256][8] bias sums
+  unsigned long long* full = reinterpret_cast<unsigned long long*>(dbs + 256 * 8);
+  unsigned long long *empty = full + NS, *gfull = empty + NS, *gempty = gfull + 2, *done = gempty + 2;
+  unsigned* tslot = reinterpret_cast<unsigned*>(done + 1);
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  if (t == 0) {
+    for (int k = 0; k < NS; k++) {
+      mbar_init(full + k, 1);
+      mbar_init(empty + k, 2);
+    }
+    for (int k = 0; k < 2; k++) {
+      mbar_init(gfull + k, 256);
+      mbar_init(gempty + k, 2);
+    }
+    mbar_init(done, 2);
+    mbar_init_fence();
+  }
+  if (warp == 8) {
+    tmem_alloc(tslot, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned taddr = *tslot;
+  bool dead = false;  // a wait ran out: no further waits in this thread, results flagged
+  auto wait = [&](unsigned long long* mb, unsigned parity) {
+    if (!dead) dead = !mbar_wait_limit(mb, parity & 1, 1 << 16, &g_net_status);
+  };
+  const int nyt = (H + RT - 1) / RT, nzt = (D + TZ - 1) / TZ, ntiles = Nb * nzt * nyt;
+  const int kc0 = blockIdx.y * T::GROUP, kc1 = min(kc0 + T::GROUP, Cin >> 4);
+  if (warp == 10) {
+    if (lane == 0) {
+      fence_proxy_async_global();  // the input was written by ordinary stores
+      int s = 0;
+      unsigned phase = 0;
+      for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int yt = tile % nyt, zt = (tile / nyt) % nzt, n = tile / (nyt * nzt);
+        for (int kc = kc0; kc < kc1; kc++) {
+          if (phase > 0) wait(empty + s, phase - 1);
+          mbar_expect_tx(full + s, T::ABYTES);
+          tma_load_5d(As + s * T::ABYTES, &rows, kc * 16, 0, yt * RT - 1, zt * TZ - 1, n, full + s);
+          if (++s == NS) {
+            s = 0;
+            phase++;
+          }
+        }
+      }
+    }
+  } else if (warp >= 8) {
+    const int m = warp - 8;  // M tile: row groups 8 m .. 8 m + 7
+    if (lane == 0) {
+      const uint64_t a00 = smem_desc(As + m * 8 * W * 32, W * 32, 256) | (uint64_t)6 << 61;
+      const uint64_t b00 = smem_desc(Gs, 128, W * 16);
+      int s = 0, it = 0;
+      unsigned phase = 0;
+      for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, it++) {
+        const int d = it & 1;
+        wait(gfull + d, it >> 1);
+        for (int kc = kc0; kc < kc1; kc++) {
+          wait(full + s, phase);
+          tc_fence_after();
+          const unsigned acc = taddr + ((kc - kc0) * 2 + m) * 3 * NO;
+          const uint64_t a0 = a00 + (unsigned)(s * (T::ABYTES >> 4)), b0 = b00 + (unsigned)(d * (T::GBYTES >> 4));
+          static_for<0, DROWS>([&](auto row_c) {
+            constexpr int r = decltype(row_c)::value, slot = r / RT * PR + r % RT;
+#pragma unroll
+            for (int ks = 0; ks < W / 16; ks++)
+              tc_mma(acc, a0 + (unsigned)((slot * W * 32 + ks * 512) >> 4), b0 + (unsigned)((r * ROWB + ks * 256) >> 4),
+                     IDESC, it > 0 || r > 0 || ks > 0);
+          });
+          tc_commit(empty + s);
+          if (++s == NS) {
+            s = 0;
+            phase++;
+          }
+        }
+        tc_commit(gempty + d);
+      }
+      tc_commit(done);
+    }
+  } else {
+    // the output gradient: thread t takes channel group t % CG of every (256 / CG)-th voxel
+    const int cg = t % CG, v0 = t / CG;
+    float db[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    int it = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, it++) {
+      const int d = it & 1;
+      if (it >= 2) wait(gempty + d, (it >> 1) - 1);
+      const int yt = tile % nyt, zt = (tile / nyt) % nzt, n = tile / (nyt * nzt);
+      constexpr int VP = 256 / CG, ITER = (DROWS * W + VP - 1) / VP, BATCH = ITER < 4 ? ITER : 4;
+#pragma unroll
+      for (int i0 = 0; i0 < ITER; i0 += BATCH) {
+        float4 f[BATCH][2];
+#pragma unroll
+        for (int b = 0; b < BATCH; b++) {
+          const int v = (i0 + b) * VP + v0, r = v / W, x = v % W, z = zt * TZ + r / RT, y = yt * RT + r % RT;
+          f[b][0] = f[b][1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          if (i0 + b < ITER && v < DROWS * W && z < D && y < H) {
+            const float4* g = reinterpret_cast<const float4*>(dout + ((((long long)n * D + z) * H + y) * W + x) * NO + cg * 8);
+            f[b][0] = g[0];
+            f[b][1] = g[1];
+          }
+        }
+#pragma unroll
+        for (int b = 0; b < BATCH; b++) {
+          const int v = (i0 + b) * VP + v0, r = v / W, x = v % W;
+          if (i0 + b >= ITER || v >= DROWS * W) continue;
+          const float4 f0 = f[b][0], f1 = f[b][1];
+          db[0] += f0.x, db[1] += f0.y, db[2] += f0.z, db[3] += f0.w;
+          db[4] += f1.x, db[5] += f1.y, db[6] += f1.z, db[7] += f1.w;
+          const uint4 pk = make_uint4(pack2(f0.x, f0.y), pack2(f0.z, f0.w), pack2(f1.x, f1.y), pack2(f1.z, f1.w));
+          unsigned char* g = Gs + d * T::GBYTES + r * ROWB + cg * W * 16;  // copy c holds the value of x + 1 - c at x
+          constexpr int CP = CG * W * 16;
+          *reinterpret_cast<uint4*>(g + CP + x * 16) = pk;
+          if (x >= 1) *reinterpret_cast<uint4*>(g + (x - 1) * 16) = pk;
+          if (x + 1 < W) *reinterpret_cast<uint4*>(g + 2 * CP + (x + 1) * 16) = pk;
+          if (x == 0) *reinterpret_cast<uint4*>(g + 2 * CP) = make_uint4(0u, 0u, 0u, 0u);
+          if (x == W - 1) *reinterpret_cast<uint4*>(g + (W - 1) * 16) = make_uint4(0u, 0u, 0u, 0u);
+        }
+      }
+      fence_proxy_async_smem();  // written through the generic proxy, read by the tensor core
+      mbar_arrive(gfull + d);
+    }
+    const long long per = 27LL * Cin * NO, stride = per + NO;
+    float* pb = part + (long long)blockIdx.x * stride;
+    if (blockIdx.y == 0) {  // bias sums of the threads with the same channel group, in order
+#pragma unroll
+      for (int i = 0; i < 8; i++) dbs[t * 8 + i] = db[i];
+      bar_named(1, 256);
+      if (t < NO) {
+        float a = 0.0f;
+        for (int k = t / 8; k < 256; k += CG) a += dbs[k * 8 + t % 8];
+        pb[per + t] = a;
+      }
+    }
+    wait(done, 0);
+    __syncwarp();
+    tc_fence_after();
+    // lane (16 g + ci) of M tile m: row group j = 8 m + g = dz PR + dy
+    const int mrow = (warp & 3) * 32 + lane, ci = mrow & 15;
+    for (int q = warp >> 2; q < 2 * (kc1 - kc0); q += 2) {
+      const int kc = kc0 + (q >> 1), j = 8 * (q & 1) + (mrow >> 4), dz = j / PR, dy = j % PR;
+      const bool used = dz < 3 && dy < 3;
+#pragma unroll 1
+      for (int c0 = 0; c0 < 3 * NO; c0 += 16) {
+        float r[16];
+        tc_ld16(taddr + ((unsigned)((warp & 3) * 32) << 16) + q * 3 * NO + c0, r);
+        tc_wait_ld();
+        if (used) {
+          float4* o = reinterpret_cast<float4*>(
+              pb + ((long long)(dz * 9 + dy * 3 + c0 / NO) * Cin + kc * 16 + ci) * NO + c0 % NO);
+#pragma unroll
+          for (int i = 0; i < 4; i++) o[i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+        }
+        __syncwarp();
+      }
+    }
+  }
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8) {
+    tc_fence_after();
+    tmem_dealloc(taddr, 512);
+  }
+}
+
+// dW (n values) and db (C values) = the block partials part[nblk][n + C]: 8 threads per value add
+// every eighth partial, and the eight sums are added in order (one thread per value and 152
+// loads in turn took 16 us for 48 -> 16 channels, beside 25 us for a bias gradient of its own)
+__global__ void __launch_bounds__(256) k_dw_finish(const float* part, int nblk, long long n, int C, float* dW, float* db) {
+  __shared__ float red[8][32];
+  const int x = threadIdx.x & 31, r = threadIdx.x >> 5;
+  const long long i = blockIdx.x * 32LL + x, stride = n + C;
+  float s = 0.0f;
+  if (i < stride)
+    for (int b = r; b < nblk; b += 8) s += part[b * stride + i];
+  red[r][x] = s;
+  __syncthreads();
+  if (r == 0 && i < stride) {
+    for (int k = 1; k < 8; k++) s += red[k][x];
+    if (i < n) dW[i] = s;
+    else db[i - n] = s;
+  }
+}
+
+template <int W, int NO>
+int launch_dw_rows(const bf16* in, const float* dout, float* dW, float* db, float* work, long long work_floats, int Nb,
+                   int D, int H, int Cin, cudaStream_t s) {
+  using T = DwRows<W, NO>;
+  const long long n = 27LL * Cin * NO;
+  const int skip = (int)(-(intptr_t)(reinterpret_cast<uintptr_t>(work) >> 2) & 3);  // partials from a 16-byte boundary
+  work += skip;
+  work_floats -= skip;
+  const long long tiles = (long long)Nb * ((D + T::TZ - 1) / T::TZ) * ((H + T::RT - 1) / T::RT);
+  const int groups = ((Cin >> 4) + T::GROUP - 1) / T::GROUP;
+  long long nblk = sm_count() / groups;  // one block per SM, and no more partials than work holds
+  if (nblk < 1) nblk = 1;
+  if (nblk > tiles) nblk = tiles;
+  if (nblk > work_floats / (n + NO)) nblk = work_floats / (n + NO);
+  if (nblk < 1 || tiles > 0x7fffffffLL) return -1;
+  CUtensorMap rows;
+  const cuuint64_t dims[5] = {(cuuint64_t)Cin, W, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)Nb};
+  const cuuint64_t pitch[4] = {2ull * Cin, 2ull * Cin * W, 2ull * Cin * W * H, 2ull * Cin * W * H * D};
+  const cuuint32_t box[5] = {16, W, T::PR, T::TZ + 2, 1}, step[5] = {1, 1, 1, 1, 1};
+  tmk::EncodeTiledFn fn = tmk::encoder();
+  if (!fn || fn(&rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16*>(in), dims, pitch, box, step,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return -4;
+  static bool init = false;
+  if (!init) {
+    if (cudaFuncSetAttribute(k_conv_dw_rows<W, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM) !=
+        cudaSuccess)
+      return -4;
+    init = true;
+  }
+  k_conv_dw_rows<W, NO><<<dim3((unsigned)nblk, groups), T::THREADS, T::SMEM, s>>>(rows, dout, work, Nb, D, H, Cin);
+  k_dw_finish<<<(unsigned)((n + NO + 31) / 32), 256, 0, s>>>(work, (int)nblk, n, NO, dW, db);
+  return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
+}
+
+// Weight gradient for rows of 8 voxels (half of a K = 16 step, which k_conv_dw_rows could not
+// cut from its rows): dW[tap][ci][co] =
 // sum_v in[v + off(tap)][ci] q(dout[v][co]) as MMAs with M = co (padded to 128), N = the
 // 16 input channels of a chunk for the three dx taps at once (48), K = 16 voxels. A
 // persistent block takes tiles of one plane x 128 / W rows (128 voxels): it stages the three
@@ -1374,7 +1643,20 @@ int tmn_conv3d_backward_weight(const void* in, const float* dout, float* dW, flo
   if (work_floats < tmn_conv3d_backward_weight_work(nvox, Cin, Cout)) return -5;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int nsm = sm_count();
-  if ((W == 8 || W == 16 || W == 32 || W == 64) && (reinterpret_cast<uintptr_t>(in) & 15) == 0) {
+  if ((reinterpret_cast<uintptr_t>(in) & 15) == 0) {
+    const bf16* x = reinterpret_cast<const bf16*>(in);
+#define TMN_DW_ROWS(WW)                                                                                    \
+  if (W == WW) {                                                                                           \
+    if (Cout == 16) return launch_dw_rows<WW, 16>(x, dout, dW, db, work, work_floats, N, D, H, Cin, s);     \
+    if (Cout == 32) return launch_dw_rows<WW, 32>(x, dout, dW, db, work, work_floats, N, D, H, Cin, s);     \
+    return launch_dw_rows<WW, 64>(x, dout, dW, db, work, work_floats, N, D, H, Cin, s);                     \
+  }
+    TMN_DW_ROWS(16)
+    TMN_DW_ROWS(32)
+    TMN_DW_ROWS(64)
+#undef TMN_DW_ROWS
+  }
+  if (W == 8 && (reinterpret_cast<uintptr_t>(in) & 15) == 0) {
     // halo tiles: one persistent block per SM, as many as the work buffer holds partials for
     const long long per = 27LL * Cin * Cout, ntl = (long long)N * D * ((H + 128 / W - 1) / (128 / W));
     long long nblk = work_floats / per;
@@ -1395,9 +1677,6 @@ int tmn_conv3d_backward_weight(const void* in, const float* dout, float* dW, flo
     if (Cout == 64) run(k_conv_dw_halo<WW, 64>, dw_halo_smem<WW>());                \
   }
     TMN_DW_HALO(8)
-    TMN_DW_HALO(16)
-    TMN_DW_HALO(32)
-    TMN_DW_HALO(64)
 #undef TMN_DW_HALO
     if (r) return r;
     k_dw_reduce_halo<<<grid_of(per), 256, 0, s>>>(work, (int)nblk, per, dW);
