@@ -281,8 +281,8 @@ int launch_conv_tc(const void* src, const bf16* Wc, const float* bias, void* dst
 // between them. The packed weights stay in shared memory where they fit, otherwise each stage
 // brings its chunk's.
 // Measured, 64^3 x 2: forward 48 -> 16 channels 139 -> 33 us, of which the MMAs' operand reads
-// are 16 (44 cycles for M = 128, N = 48); data gradient 16 -> 48 113 -> 70 us, bound by the
-// epilogue (60 us alone). Before: one block per two tiles, three shifted copies, 27 MMAs a chunk
+// are 16 (44 cycles for M = 128, N = 48); data gradient 16 -> 48 113 -> 56 us, most of it the
+// epilogue's instructions (shuffles and sums of three arrays). Before: one block per two tiles, three shifted copies, 27 MMAs a chunk
 // and nothing overlapped inside a block. On the way: 9 MMAs without the pipeline 88 and 139,
 // rows staged by threads in MODE 0 59, 54 weight copies a chunk instead of one box 39.
 // compile-time loop: f(std::integral_constant<int, i>) for i in [B, E)
@@ -633,21 +633,17 @@ k_conv_halo(const __grid_constant__ CUtensorMap rows, const __grid_constant__ CU
               lf[i] = a;
               rt[i] = b;
             }
-            if ((w4 & 1) == 1 && lane == 0) {
+            const bool ml = (w4 & 1) == 1 && lane == 0, mr = (w4 & 1) == 0 && lane == 31;
 #pragma unroll
-              for (int i = 0; i < 4; i++) {
-                const float4 q = reinterpret_cast<const float4*>(xr)[i];
-                lf[4 * i] = q.x, lf[4 * i + 1] = q.y, lf[4 * i + 2] = q.z, lf[4 * i + 3] = q.w;
+            for (int i = 0; i < 4; i++) {  // every lane reads (a broadcast), one keeps it
+              const float4 q = reinterpret_cast<const float4*>(xr + ((w4 & 1) ? 0 : 16))[i];
+              const float w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+              for (int k = 0; k < 4; k++) {
+                lf[4 * i + k] = ml ? w[k] : lf[4 * i + k];
+                rt[4 * i + k] = mr ? w[k] : rt[4 * i + k];
               }
             }
-            if ((w4 & 1) == 0 && lane == 31) {
-#pragma unroll
-              for (int i = 0; i < 4; i++) {
-                const float4 q = reinterpret_cast<const float4*>(xr + 16)[i];
-                rt[4 * i] = q.x, rt[4 * i + 1] = q.y, rt[4 * i + 2] = q.z, rt[4 * i + 3] = q.w;
-              }
-            }
-            __syncwarp();
           } else {
 #pragma unroll
             for (int i = 0; i < 16; i++) {
@@ -657,8 +653,9 @@ k_conv_halo(const __grid_constant__ CUtensorMap rows, const __grid_constant__ CU
           }
 #pragma unroll
           for (int i = 0; i < 16; i++) {
-            if (pl) r[i] += lf[i];
-            if (pr) r[i] += rt[i];
+            // (selects: as conditional adds these were 16 divergent branches a step, 1000 cycles)
+            r[i] += pl ? lf[i] : 0.0f;
+            r[i] += pr ? rt[i] : 0.0f;
           }
           if (!valid) {
           } else if constexpr (MODE == 0) {
