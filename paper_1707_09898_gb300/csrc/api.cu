@@ -322,6 +322,16 @@ struct ConvSpec {
   int in_ext, out_ext;
 };
 
+// one input, one output and one tensor component between them
+bool single_product(const ConvSpec& cs) {
+  if (cs.nin != 1 || cs.nout != 1) return false;
+  float c6[6];
+  coef6(c6, cs.v[0], cs.u[0]);
+  int n = 0;
+  for (int c = 0; c < 6; c++) n += c6[c] != 0.0f;
+  return n == 1;
+}
+
 // float copies of the vectors; returns the mask of the tensor components they use
 int product_vectors(const ConvSpec& cs, float u[3][3], float v[3][3]) {
   int need = 0;
@@ -423,7 +433,8 @@ int conv_yz(tm_ctx* ctx, const ConvSpec& cs, int zin, int zout, cudaStream_t s) 
 }
 
 // y pass (forward or inverse) over planes [z0, z0 + np) between A slots and B slots
-int ypass(tm_ctx* ctx, bool inv, int n, const int* aslot, const int* bslot, int z0, int np, cudaStream_t s) {
+int ypass(tm_ctx* ctx, bool inv, int n, const int* aslot, const int* bslot, int z0, int np, cudaStream_t s,
+          unsigned* zero_word = nullptr) {
   const int Lx = ctx->L[0], Ly = ctx->L[1];
   const long long P = ctx->P;
   YArgs y{};
@@ -445,6 +456,7 @@ int ypass(tm_ctx* ctx, bool inv, int n, const int* aslot, const int* bslot, int 
   }
   y.z0 = z0;
   y.tw = ctx->tw + Lx;
+  y.zero_word = zero_word;
   y.pdl = ctx->pdl;
   Timed t(ctx, inv ? KIND_YINV : KIND_YFWD, s);
   CKL(inv ? launch_yinv(Ly, y, n, s) : launch_yfwd(Ly, y, n, s));
@@ -475,6 +487,7 @@ int zdirect(tm_ctx* ctx, const ConvSpec& cs, int zi0, int nzi, int zo0, int nzo,
   z.nzin = nzi;
   z.zout0 = zo0;
   z.nzout = nzo;
+  z.pdl = ctx->pdl;
   Timed t(ctx, KIND_ZPASS, s);
   CKL(launch_zdir(z, s));
   return TM_OK;
@@ -500,10 +513,9 @@ int scaled_component(tm_ctx* ctx, int which, int c, float coef, cudaStream_t s, 
 
 int one_component(int need) { return (need != 0 && (need & (need - 1)) == 0) ? __builtin_ctz(need) : -1; }
 
-// forward y transform of the design planes fused with the direct z sum onto the
-// single target plane (cs.nout == 1); *yinv_done: the kernel also wrote the target
-// plane's inverse y transform into A
-int yz_forward(tm_ctx* ctx, const ConvSpec& cs, int zo, cudaStream_t s, bool* yinv_done) {
+// forward y transform of the design planes fused with the direct z sum onto the single target
+// plane (one spectrum, one tensor component), and the target plane's inverse y transform into A
+int yz_forward(tm_ctx* ctx, const ConvSpec& cs, int zo, cudaStream_t s) {
   const int Ly = ctx->L[1];
   const long long P = ctx->P;
   const int chunks = (int)(P / TB);
@@ -522,9 +534,6 @@ int yz_forward(tm_ctx* ctx, const ConvSpec& cs, int zo, cudaStream_t s, bool* yi
   y.in = ctx->A;
   y.in_cstride = (long long)ctx->nz * ctx->ny * P;
   y.in_zstride = (long long)ctx->ny * P;
-  y.out = ctx->B;
-  y.out_cstride = (long long)ctx->nz * Ly * P;
-  y.out_slot = cs.bout[0];
   y.part = ctx->yzpart;
   y.P = ctx->P;
   y.n_in = ctx->ny;
@@ -546,8 +555,8 @@ int yz_forward(tm_ctx* ctx, const ConvSpec& cs, int zo, cudaStream_t s, bool* yi
   y.tw = ctx->tw + ctx->L[0];
   if (!ctx->yzseg) CK(cudaMalloc(&ctx->yzseg, (size_t)2 * ctx->nsm * Ly * TB * sizeof(float2)));
   y.seg = ctx->yzseg;
-  const int c1 = cs.nin == 1 ? one_component(y.need[0]) : -1;
-  if (c1 >= 0) {
+  {
+    const int c1 = one_component(y.need[0]);
     int r;
     bool rebuilt;
     if ((r = scaled_component(ctx, 0, c1, y.coef[0][c1], s, &y.Ts, &rebuilt))) return r;
@@ -562,23 +571,18 @@ int yz_forward(tm_ctx* ctx, const ConvSpec& cs, int zo, cudaStream_t s, bool* yi
     r = launch_yz_fwd(Ly, y, s);
     if (r < 0) CKL(r);
   }
-  if (r == 1) {  // the target plane: partial sums added, inverse y transform
-    Timed t(ctx, KIND_YINV, s);
-    CKL(launch_yz_finish(Ly, y, s));
-  }
-  *yinv_done = r == 1;
+  // the target plane: partial sums added, inverse y transform
+  Timed t(ctx, KIND_YINV, s);
+  CKL(launch_yz_finish(Ly, y, r, s));
   return TM_OK;
 }
 
-// direct z sum from the source planes [zi0, zi0 + nzi) fused with the inverse y
-// transform of every design plane
-int zy_adjoint(tm_ctx* ctx, const ConvSpec& cs, int zi0, int nzi, cudaStream_t s, bool yfwd_inside) {
+// direct z sum from the source plane zi0 (x spectra in A, transformed along y by the kernel)
+// fused with the inverse y transform of every design plane
+int zy_adjoint(tm_ctx* ctx, const ConvSpec& cs, int zi0, cudaStream_t s) {
   const int Ly = ctx->L[1];
   const long long P = ctx->P;
   ZYArgs z{};
-  z.src = ctx->B;
-  z.src_cstride = (long long)ctx->nz * Ly * P;
-  z.src_zstride = (long long)Ly * P;
   z.out = ctx->A;
   z.out_cstride = (long long)ctx->nz * ctx->ny * P;
   z.out_zstride = (long long)ctx->ny * P;
@@ -600,7 +604,7 @@ int zy_adjoint(tm_ctx* ctx, const ConvSpec& cs, int zi0, int nzi, cudaStream_t s
   z.Tdz = (long long)(Ly / 2 + 1) * P;
   z.Tc = (long long)ctx->nz * z.Tdz;
   z.zin0 = zi0;
-  z.nzin = nzi;
+  z.nzin = 1;
   z.zout0 = 0;
   z.nzout = ctx->nzd;
   z.tw = ctx->tw + ctx->L[0];
@@ -617,10 +621,9 @@ int zy_adjoint(tm_ctx* ctx, const ConvSpec& cs, int zi0, int nzi, cudaStream_t s
     // after a rebuild it must start only once the scaling kernel has finished
     if (rebuilt) z.pdl = 0;
   }
-  if (yfwd_inside) {  // the source plane as x spectra: rows y < ny of plane zi0 of A slot ain[0]
-    z.gsrc = ctx->A + cs.ain[0] * ((long long)ctx->nz * ctx->ny * P) + (long long)zi0 * ctx->ny * P;
-    z.n_src = ctx->ny;
-  }
+  // the source plane as x spectra: rows y < ny of plane zi0 of A slot ain[0]
+  z.gsrc = ctx->A + cs.ain[0] * ((long long)ctx->nz * ctx->ny * P) + (long long)zi0 * ctx->ny * P;
+  z.n_src = ctx->ny;
   Timed t(ctx, KIND_ZYA, s);
   const int r = launch_zy_adj(Ly, z, s);
   if (r < 0) CKL(r);
@@ -1134,14 +1137,9 @@ int forward_planes(tm_ctx* ctx, const float* rho, const int* F, int nF, cudaStre
     cs.aout[o] = o;
     cs.v[o] = kUnit[F[o]];
   }
-  if (ctx->fuse_yz && np == 1 && nF == 1) {
-    bool done = false;
-    if ((r = yz_forward(ctx, cs, ctx->tz0, s, &done))) return r;
-    if (done) return TM_OK;
-  } else {
-    if ((r = ypass(ctx, false, cs.nin, cs.ain, cs.bin, 0, ctx->nzd, s))) return r;
-    if ((r = zdirect(ctx, cs, 0, ctx->nzd, ctx->tz0, np, s))) return r;
-  }
+  if (ctx->fuse_yz && np == 1 && single_product(cs)) return yz_forward(ctx, cs, ctx->tz0, s);
+  if ((r = ypass(ctx, false, cs.nin, cs.ain, cs.bin, 0, ctx->nzd, s))) return r;
+  if ((r = zdirect(ctx, cs, 0, ctx->nzd, ctx->tz0, np, s))) return r;
   return ypass(ctx, true, cs.nout, cs.aout, cs.bout, ctx->tz0, np, s);
 }
 
@@ -1174,26 +1172,17 @@ int adjoint_planes(tm_ctx* ctx, const float* rho, float* dJdrho, const int* F, c
     }
   }
   // fused only in its single-spectrum, single-component form; with several spectra or
-  // tensor components the separate passes measured faster
-  bool simple = ca.nin == 1 && ca.nout == 1 && np == 1;
-  if (simple) {
-    float c6[6];
-    coef6(c6, ca.v[0], ca.u[0]);
-    int nc = 0;
-    for (int c = 0; c < 6; c++) nc += c6[c] != 0.0f;
-    simple = nc == 1;
-  }
-  // on the warp-specialized path the fused adjoint runs the source's y transform itself;
-  // it then reads the source rows from A while it writes the design planes into A, so its
-  // output goes to another slot (the target plane may be a design plane)
-  const bool yfwd_inside = ctx->fuse_yz && simple && zy_adj_ws_length(ctx->L[1]) && ctx->ny <= ctx->L[1] / 2;
-  if (yfwd_inside) ca.aout[0] = (ca.ain[0] + 1) % kSlotsA;
-  if (!yfwd_inside && (r = ypass(ctx, false, ca.nin, ca.ain, ca.bin, ctx->tz0, np, s))) return r;
-  if (ctx->fuse_yz && simple) {
-    if ((r = zy_adjoint(ctx, ca, ctx->tz0, np, s, yfwd_inside))) return r;
+  // tensor components the separate passes measured faster. The fused kernel reads the source
+  // rows from A while it writes the design planes into A, so its output goes to another slot
+  // (the target plane may be a design plane).
+  if (ctx->fuse_yz && np == 1 && single_product(ca)) {
+    ca.aout[0] = (ca.ain[0] + 1) % kSlotsA;
+    if ((r = zy_adjoint(ctx, ca, ctx->tz0, s))) return r;
   } else {
+    if ((r = ypass(ctx, false, ca.nin, ca.ain, ca.bin, ctx->tz0, np, s))) return r;
     if ((r = zdirect(ctx, ca, ctx->tz0, np, 0, ctx->nzd, s))) return r;
-    if ((r = ypass(ctx, true, ca.nout, ca.aout, ca.bout, 0, ctx->nzd, s))) return r;
+    if ((r = ypass(ctx, true, ca.nout, ca.aout, ca.bout, 0, ctx->nzd, s, ctx->gmax))) return r;
+    ctx->gmax_zeroed = true;
   }
   return xinv_chain(ctx, rho, dJdrho, ca.nout, ca.aout, s);
 }

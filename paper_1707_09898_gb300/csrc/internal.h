@@ -121,6 +121,7 @@ struct YArgs {
   int z0;                   // first plane (host-known offset); planes z0 .. z0 + nplanes - 1
   const int* ext;           // device [zlo, zhi): process only those planes (null: all nplanes)
   const float2* tw;
+  unsigned* zero_word;      // if set, zeroed by the pass
   int pdl;                  // launch with programmatic dependent launch
 };
 
@@ -168,7 +169,8 @@ struct ZDirArgs {
 int launch_zdir(const ZDirArgs& a, cudaStream_t s);
 
 // Fused y transform + direct z sum (k_yzfused.cu).
-// Adjoint: from few source planes of B to the real-y rows of every output plane of A.
+// Adjoint: from one source plane, given as x spectra, to the real-y rows of every output
+// plane of A (one spectrum, one tensor component).
 struct ZYArgs {
   const float2* src;                        // B [slot][z][Ly][P]
   long long src_cstride, src_zstride;
@@ -185,24 +187,23 @@ struct ZYArgs {
   // warp-specialized path (one tensor component c): Ts = coef[0][0][c] * Tz[c], [nzin_total][Ly/2+1][P]
   const float* Ts;
   int nzin_total;                           // z offsets held by Ts
-  // if set (warp-specialized path only): the source plane as x spectra, rows [n_src][P]; the
-  // kernel runs its forward y transform itself and src is not read
+  // the source plane as x spectra, rows [n_src][P]: the kernel runs its forward y transform.
+  // Null (L = 512 only): the y spectrum is read from src. No caller does so now, but without
+  // that branch the compiler spills 48 bytes instead of 28 and the kernel takes 66.6 us instead
+  // of 61.8 for 256 planes of 256^2.
   const float2* gsrc;
   int n_src;
   unsigned* status;                         // device word: bit 0 set when a copy wait timed out
-  unsigned* zero_word;                      // if set, zeroed by the warp-specialized kernel (launch_zy_adj returns 1)
+  unsigned* zero_word;                      // if set, zeroed by the kernel (launch_zy_adj returns 1)
   int pdl;                                  // launch with programmatic dependent launch
 };
 // Forward: the design planes of A onto one plane and one output of B.
 struct YZArgs {
   const float2* in;                         // A [slot][z][ny][P]
   long long in_cstride, in_zstride;
-  float2* out;                              // B [slot][z][Ly][P]
-  long long out_cstride;
-  int out_slot;
   float2* part;                             // [z chunks][Ly][P]
   int P, n_in;
-  int nin, in_slot[3];
+  int nin, in_slot[3];                      // one input
   float coef[3][6];                         // s_i = v^T N u_i of the single output
   int need[3];
   const float* Tz;
@@ -221,13 +222,11 @@ struct YZArgs {
   int pdl;                                  // launch with programmatic dependent launch
 };
 int launch_zy_adj(int L, const ZYArgs& a, cudaStream_t s);
-// whether launch_zy_adj takes the warp-specialized path for length L (one source plane, one
-// spectrum and tensor component, Ts given), the path that can run the source's y transform
-bool zy_adj_ws_length(int L);
 int launch_yz_fwd(int L, const YZArgs& a, cudaStream_t s);
-// after launch_yz_fwd returned 1: the segment partials of each column block added in block
-// order, and the target plane's inverse y transform into a.yrows
-int launch_yz_finish(int L, const YZArgs& a, cudaStream_t s);
+// after launch_yz_fwd returned how = 1 (segment partials of the warp-specialized kernel) or 2
+// (partials of z chunks): the partials added in order, and the target plane's inverse y
+// transform into a.yrows
+int launch_yz_finish(int L, const YZArgs& a, int how, cudaStream_t s);
 
 int launch_xfwd(int L, const XFwdArgs& a, int ncomp, cudaStream_t s);
 int launch_xinv(int L, const XInvArgs& a, cudaStream_t s);

@@ -4,10 +4,11 @@
 //   half spectra of two real rows -> inverse x transform -> H, J, g -> forward x
 //   transform of g -> half spectra of the adjoint source.
 // The target rows are few (one or a few planes), so this kernel is bound by latency,
-// not bandwidth: a group of four warps per pair of rows runs an iterative mixed-radix
-// Stockham transform (radix 4, 2, 3 stages in natural order, loops rather than
-// unrolled stages) in its own shared-memory buffers, synchronising only the group
-// (named barrier). The code is a few hundred instructions for every length.
+// not bandwidth: one, two or four warps (a thread per radix-4 butterfly) take a pair of rows
+// and run a mixed-radix Stockham transform (radix 4, 2, 3 stages in natural order) in their own
+// shared-memory buffers, synchronising only their group. The stages are fixed at compile
+// time: with run-time lengths, divisions in every stage and four warps for every length a
+// launch took 10.6 us at L = 128 and 10.8 at 256, this 6.6 and 7.6.
 #include "fft.cuh"
 #include "internal.h"
 
@@ -15,35 +16,43 @@ namespace tmk {
 
 namespace {
 
-constexpr int OW = 8;   // warps per block
-constexpr int GW = 4;   // warps per row pair (one transform group)
-constexpr int GT = GW * 32;
-constexpr int NG = OW / GW;  // row pairs per block
-constexpr int KI = 3;   // ceil((576 / 2 + 1) / GT): half-spectrum values per thread
-constexpr int XI = 5;   // ceil(576 / GT): real values per thread
+constexpr int NG = 2;  // row pairs per block
+template <int L>
+struct ObjShape {
+  static constexpr int GT = L <= 128 ? 32 : L <= 256 ? 64 : 128;  // threads per row pair
+  static constexpr int NT = NG * GT;
+  static constexpr int KI = (L / 2 + GT) / GT;      // half-spectrum values per thread
+  static constexpr int XI = (L + GT - 1) / GT;      // real values per thread
+};
 
 __device__ __forceinline__ cx<float> cmul(cx<float> a, cx<float> b) {
   return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ cx<float> conjf(cx<float> a) { return mk(a.x, -a.y); }
 
-// barrier of the GT threads of transform group g (ids 1.. ; 0 is the block barrier)
-__device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(GT) : "memory"); }
+// barrier of the N threads of transform group g (ids 1.. ; 0 is the block barrier)
+template <int N>
+__device__ __forceinline__ void group_sync(int g) {
+  if (N == 32) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(N) : "memory");
+}
 __device__ __forceinline__ void group_sync8(int g) { asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(64) : "memory"); }
 
-// One group: length-L transform of src into dst (natural order both), sign -1 forward,
-// +1 inverse (unnormalised). Stockham stages: for j < L/R, the R inputs src[j + r L/R]
-// times W^(r (j mod Ns) L/(Ns R)) go through a radix-R DFT to dst[(j/Ns) Ns R + j mod
-// Ns + r Ns], Ns the product of the radices before. Returns the buffer holding the result.
-__device__ cx<float>* group_fft(cx<float>* src, cx<float>* dst, int L, const cx<float>* tw, bool inverse, int gt,
-                                int g) {
-  int rem = L, Ns = 1;
-  while (rem > 1) {
-    const int R = rem % 4 == 0 ? 4 : (rem % 2 == 0 ? 2 : 3);
-    const int M = L / R;
-    const int step = L / (Ns * R);
-#pragma unroll 1
-    for (int j = gt; j < M; j += GT) {
+// One group: length-L transform of src into dst (natural order both), forward or inverse
+// (unnormalised). Stockham stages: for j < L/R, the R inputs src[j + r L/R] times W^(r (j mod
+// Ns) L/(Ns R)) go through a radix-R DFT to dst[(j/Ns) Ns R + j mod Ns + r Ns], Ns the product
+// of the radices before. Returns the buffer holding the result.
+template <int L, bool inverse, int Ns = 1>
+__device__ __forceinline__ cx<float>* group_fft(cx<float>* src, cx<float>* dst, const cx<float>* tw, int gt, int g) {
+  if constexpr (Ns == L) {
+    return src;
+  } else {
+    constexpr int rem = L / Ns, R = rem % 4 == 0 ? 4 : (rem % 2 == 0 ? 2 : 3), M = L / R, step = L / (Ns * R);
+    constexpr int GT = ObjShape<L>::GT;
+#pragma unroll
+    for (int j0 = 0; j0 < M; j0 += GT) {
+      const int j = j0 + gt;
+      if (M % GT != 0 && j >= M) break;
       const int k = j % Ns;
       cx<float> v[4];
 #pragma unroll
@@ -82,31 +91,29 @@ __device__ cx<float>* group_fft(cx<float>* src, cx<float>* dst, int L, const cx<
       for (int r = 0; r < 4; r++)
         if (r < R) dst[base + r * Ns] = y[r];
     }
-    group_sync(g);
-    cx<float>* t = src;
-    src = dst;
-    dst = t;
-    Ns *= R;
-    rem /= R;
+    group_sync<GT>(g);
+    return group_fft<L, inverse, Ns * R>(dst, src, tw, gt, g);
   }
-  return src;
 }
 
-__global__ void __launch_bounds__(OW * 32) k_xobj(XInvArgs a, int L) {
+template <int L>
+__global__ void __launch_bounds__(ObjShape<L>::NT) k_xobj(XInvArgs a) {
+  using O = ObjShape<L>;
+  constexpr int GT = O::GT, NT = O::NT, KI = O::KI, XI = O::XI;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int any_mask[NG];
   cx<float>* tw = reinterpret_cast<cx<float>*>(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = warp / GW, gt = threadIdx.x - g * GT;
+  const int g = threadIdx.x / GT, gt = threadIdx.x - g * GT;
   cx<float>* b0 = tw + L + g * 2 * L;
   cx<float>* b1 = b0 + L;
-  for (int i = threadIdx.x; i < L; i += OW * 32) tw[i] = reinterpret_cast<const cx<float>*>(a.tw)[i];
+  for (int i = threadIdx.x; i < L; i += NT) tw[i] = reinterpret_cast<const cx<float>*>(a.tw)[i];
   if (gt == 0) any_mask[g] = 0;
   pdl_wait();  // the spectra, J partials and outputs belong to earlier kernels
   __syncthreads();
   const int jc = blockIdx.y, c = a.comp[jc];
   const float wc = a.w[c];
-  const int K = L / 2 + 1;
+  constexpr int K = L / 2 + 1;
   const int ra = a.row_base + (blockIdx.x * NG + g) * 2, rb = ra + 1;
   const cx<float>* in = reinterpret_cast<const cx<float>*>(a.in) + a.in_slot[jc] * a.in_cstride;
   double jacc = 0.0;
@@ -130,8 +137,8 @@ __global__ void __launch_bounds__(OW * 32) k_xobj(XInvArgs a, int L) {
         if (k > 0 && k < L - k) b0[L - k] = mk(A.x + B.y, B.x - A.y);  // conj(A) + i conj(B)
       }
     }
-    group_sync(g);
-    cx<float>* z = group_fft(b0, b1, L, tw, true, gt, g);
+    group_sync<GT>(g);
+    cx<float>* z = group_fft<L, true>(b0, b1, tw, gt, g);
     cx<float>* o = z == b0 ? b1 : b0;
     // mask and target values of the thread's cells, all loads first
     unsigned char mk2[XI][2];
@@ -170,7 +177,7 @@ __global__ void __launch_bounds__(OW * 32) k_xobj(XInvArgs a, int L) {
       }
     }
     if (mine) any_mask[g] = 1;
-    group_sync(g);
+    group_sync<GT>(g);
     cx<float>* adj = reinterpret_cast<cx<float>*>(a.adj_out) + a.in_slot[jc] * a.in_cstride;
     if (!any_mask[g]) {  // no target cell on these rows: the adjoint source vanishes
       for (int k = gt; k < a.P; k += GT) {
@@ -178,7 +185,7 @@ __global__ void __launch_bounds__(OW * 32) k_xobj(XInvArgs a, int L) {
         if (hb) adj[(long long)rb * a.P + k] = zero<float>();
       }
     } else {
-      cx<float>* Zg = group_fft(o, z, L, tw, false, gt, g);
+      cx<float>* Zg = group_fft<L, false>(o, z, tw, gt, g);
       for (int k = gt; k < a.P; k += GT) {
         cx<float> A = zero<float>(), B = zero<float>();
         if (k < K) {
@@ -193,12 +200,12 @@ __global__ void __launch_bounds__(OW * 32) k_xobj(XInvArgs a, int L) {
   }
   // J partial of the block in a fixed order, then the last block's sum
   for (int off = 16; off > 0; off >>= 1) jacc += __shfl_xor_sync(0xffffffffu, jacc, off);
-  __shared__ double red[OW];
+  __shared__ double red[NT / 32];
   if (lane == 0) red[warp] = jacc;
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int w = 0; w < OW; w++) s += red[w];
+    for (int w = 0; w < NT / 32; w++) s += red[w];
     a.Jpart[jc * gridDim.x + blockIdx.x] = s;
   }
   __shared__ unsigned int last;
@@ -210,13 +217,13 @@ __global__ void __launch_bounds__(OW * 32) k_xobj(XInvArgs a, int L) {
   __syncthreads();
   if (!last) return;
   __threadfence();
-  __shared__ double r2[OW * 32];
+  __shared__ double r2[NT];
   const int n = gridDim.x * gridDim.y;
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += OW * 32) s += __ldcg(a.Jpart + i);
+  for (int i = threadIdx.x; i < n; i += NT) s += __ldcg(a.Jpart + i);
   r2[threadIdx.x] = s;
   __syncthreads();
-  for (int w = OW * 16; w > 0; w >>= 1) {
+  for (int w = NT / 2; w > 0; w >>= 1) {
     if ((int)threadIdx.x < w) r2[threadIdx.x] += r2[threadIdx.x + w];
     __syncthreads();
   }
@@ -395,7 +402,14 @@ __global__ void __launch_bounds__(NT8) k_xobj512(XInvArgs a) {
 
 }  // namespace
 
-size_t xobj_smem(int L) { return (size_t)(L + NG * 2 * L) * sizeof(float2); }
+template <int L>
+static int run_xobj(const XInvArgs& a, int rows, cudaStream_t s) {
+  constexpr size_t sm = (size_t)(L + NG * 2 * L) * sizeof(float2);  // at most 23 KB
+  return launch_k(k_xobj<L>, dim3((rows + 2 * NG - 1) / (2 * NG), a.ncomp), dim3(ObjShape<L>::NT), sm, s, a.pdl != 0,
+                  a) == cudaSuccess
+             ? 0
+             : -1;
+}
 
 int launch_xobj(int L, const XInvArgs& a, cudaStream_t s) {
   if (L == 512) {
@@ -412,18 +426,18 @@ int launch_xobj(int L, const XInvArgs& a, cudaStream_t s) {
     if (!a.Jcount || !a.adj_out) return -1;
     return launch_k(k_xobj512, dim3(blocks, a.ncomp), dim3(NT8), sm8, s, a.pdl != 0, a) == cudaSuccess ? 0 : -1;
   }
-  const size_t sm = xobj_smem(L);
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_xobj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xobj_smem(576)) !=
-        cudaSuccess)
-      return -1;
-    init = true;
-  }
   const int rows = a.rows - a.row_base;
-  const int blocks = (rows + 2 * NG - 1) / (2 * NG);
-  if (blocks <= 0 || a.ncomp == 0 || !a.Jcount || !a.adj_out) return blocks <= 0 || a.ncomp == 0 ? 0 : -1;
-  return launch_k(k_xobj, dim3(blocks, a.ncomp), dim3(OW * 32), sm, s, a.pdl != 0, a, L) == cudaSuccess ? 0 : -1;
+  if (rows <= 0 || a.ncomp == 0) return 0;
+  if (!a.Jcount || !a.adj_out) return -1;
+  switch (L) {
+#define TM_CASE(LL) \
+  case LL:          \
+    if constexpr (LL != 512) return run_xobj<LL>(a, rows, s); \
+    break;
+    TM_FOR_EACH_L(TM_CASE)
+#undef TM_CASE
+  }
+  return -2;
 }
 
 int xobj_rows_per_block() { return 2 * (NG < NG8 ? NG : NG8); }  // the fewest rows any block holds

@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(kNT, 3) k_ypass(YArgs a) {
   cx<float>* tile = tw + L;
   load_twiddles<float, kNT>(tw, reinterpret_cast<const cx<float>*>(a.tw), L);
   pdl_wait();  // the input planes, the plane extent and the outputs belong to earlier kernels
+  if (a.zero_word && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *a.zero_word = 0u;
   const int chunk = blockIdx.x;
   int z = a.z0 + blockIdx.y;
   if (a.ext) {

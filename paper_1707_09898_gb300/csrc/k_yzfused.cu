@@ -6,12 +6,15 @@
 // tensor transformed along x and y only (see k_zdir.cu). When the target
 // occupies few planes:
 //   forward:  out(kx, ky, zo) = sum_z s(kx, ky, zo - z) Y(kx, ky, z), where Y is the
-//             y transform of the x-transformed design plane z. k_yz_fwd transforms
-//             each design plane of its chunk of z in shared memory and accumulates
-//             s Y in registers; k_yz_reduce sums the chunks in a fixed order.
-//   adjoint:  Y(kx, ky, z) = sum_p s(kx, ky, z - zp) src(kx, ky, zp) for every design
-//             plane z, followed by the inverse y transform: k_zy_adj computes Y in
-//             the loader of the inverse transform and writes the real-y rows.
+//             y transform of the x-transformed design plane z: k_yz_fwd_staged (L = 512:
+//             k_yz_fwd_ws) transforms the design planes of its chunk of z in shared memory
+//             and accumulates s Y in registers; k_yz_finish_chunks (k_yz_finish) adds the
+//             chunks in a fixed order and runs the target plane's inverse y transform.
+//   adjoint:  Y(kx, ky, z) = s(kx, ky, z - zp) src(kx, ky, zp) for every design plane z,
+//             followed by the inverse y transform: k_zy_adj (k_zy_adj_ws) runs the source
+//             plane's forward y transform, keeps the spectrum in registers, and forms and
+//             transforms the design planes of its block.
+// One spectrum, one tensor component and one plane; other cases run the separate passes.
 // Same discrete convolution as the unfused passes, without the round trip of the
 // y spectra of all design planes through HBM.
 
@@ -23,187 +26,102 @@ namespace tmk {
 
 namespace {
 
-// s = a - i b for (o, i) at offset dz of column (kx, ky); t points at Tz + kyf*P + kx
-__device__ __forceinline__ void tensor_s(const float* t, long long Tc, long long Tdz, float sy, int dz,
-                                         const float* coef, int need, float& a, float& b) {
-  const int adz = dz < 0 ? -dz : dz;
-  const float sz = dz < 0 ? -1.0f : 1.0f;
-  const float* p = t + adz * Tdz;
-  a = 0.0f;
-  b = 0.0f;
-  if (need & 1) a += coef[0] * p[0];
-  if (need & 2) a += coef[1] * p[Tc];
-  if (need & 4) a += coef[2] * p[2 * Tc];
-  if (need & 8) a += coef[3] * sy * p[3 * Tc];
-  if (need & 16) b += coef[4] * sz * p[4 * Tc];
-  if (need & 32) b += coef[5] * sy * sz * p[5 * Tc];
-}
-
-// SIMPLE: one input, one source plane, one tensor component c (its sign under y and z
-// reflection folded in), so each element is one source load and one tensor load with no
-// loop: all loads of a thread are in flight together.
-template <int L, bool SIMPLE>
-__global__ void __launch_bounds__(kNT, 2) k_zy_adj(ZYArgs a, int c) {
+// Adjoint, lengths without the warp-specialized kernel: block (chunk of kx, planes of z). The
+// source plane's rows (x spectra) are transformed along y once per block, their spectrum stays
+// in registers (unit (line, g) of the last stage: positions g R + q, frequencies k(g R) + q
+// L/R), and each plane of the block is formed and transformed back from it; the tensor row
+// of the next plane is loaded meanwhile. A launch of its own for the source's transform, and
+// one block per plane, took 3.5 + 4.5 us at 64^2 planes (L = 128), this 5.9; 3.5 + 12.4 at
+// 128^2 (L = 256), this 14.6.
+template <int L>
+__global__ void __launch_bounds__(kNT, L >= 288 ? 1 : 2) k_zy_adj(ZYArgs a, int c, int zper) {
   constexpr int S = plan_stages(L);
+  using SS = StageShape<L, S - 1>;
+  constexpr int R = SS::R, ITER = (SS::NU + kNT - 1) / kNT;
   extern __shared__ __align__(16) unsigned char smem[];
   cx<float>* tw = reinterpret_cast<cx<float>*>(smem);
   cx<float>* tile = tw + L;
   load_twiddles<float, kNT>(tw, reinterpret_cast<const cx<float>*>(a.tw), L);
   const int kx0 = blockIdx.x * TB;
-  const int z = a.zout0 + blockIdx.y;
-  const int o = blockIdx.z;
-  const cx<float>* src = reinterpret_cast<const cx<float>*>(a.src);
-  cx<float>* out = reinterpret_cast<cx<float>*>(a.out) + a.out_slot[o] * a.out_cstride + z * a.out_zstride + kx0;
-  __syncthreads();
-  if constexpr (SIMPLE) {
-    // first inverse stage (radix R, M = 1) with the direct z sum in its loads: the
-    // positions g R + q of a group hold ky = k(g R) + q L/R, so no per-element
-    // digit reversal; sign of the folded tensor and of odd dz precomputed
-    constexpr int s = S - 1;
-    using SS = StageShape<L, s>;
-    constexpr int R = SS::R, ITER = (SS::NU + kNT - 1) / kNT;
-    const int dz = z - a.zin0;
-    const int adz = dz < 0 ? -dz : dz;
-    const float cz = (c >= 4 && dz < 0) ? -a.coef[o][0][c] : a.coef[o][0][c];
-    const float* tcol = a.Tz + c * a.Tc + adz * a.Tdz + kx0;
-    const cx<float>* srow = src + a.in_slot[0] * a.src_cstride + a.zin0 * a.src_zstride + kx0;
-    cx<float> v[ITER][R];
+  const int z0 = a.zout0 + blockIdx.y * zper, z1 = min(z0 + zper, a.zout0 + a.nzout);
+  const float* tcol = a.Tz + c * a.Tc + kx0;
+  float f[ITER][R];
+  auto load_factors = [&](int z) {
+    const int dz = z - a.zin0, adz = dz < 0 ? -dz : dz;
+    const float cz = (c >= 4 && dz < 0) ? -a.coef[0][0][c] : a.coef[0][0][c];
+    const float* t = tcol + adz * a.Tdz;
 #pragma unroll
     for (int it = 0; it < ITER; it++) {
       const int u = it * kNT + threadIdx.x;
       if (SS::NU % kNT == 0 || u < SS::NU) {
-        const int line = u % TB, g = u / TB;
-        const int kb = k_of_group<L>(g);
+        const int line = u % TB, kb = k_of_group<L>(u / TB);
 #pragma unroll
         for (int q = 0; q < R; q++) {
           const int ky = kb + q * (L / R);
           const bool lo = ky <= L / 2;
-          const cx<float> vv = srow[(g * R + q) * a.P + line];
-          float f = cz * tcol[(lo ? ky : L - ky) * a.P + line];
-          if ((c == 3 || c == 5) && !lo) f = -f;
-          v[it][q] = c >= 4 ? mk(f * vv.y, -f * vv.x) : mk(f * vv.x, f * vv.y);  // (-i f) v for xz, yz
+          const float v = cz * t[(lo ? ky : L - ky) * a.P + line];
+          f[it][q] = (c == 3 || c == 5) && !lo ? -v : v;
         }
       }
     }
+  };
+  load_factors(z0);
+  pdl_wait();  // the source plane and the outputs belong to earlier kernels
+  if (a.zero_word && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *a.zero_word = 0u;
+  const cx<float>* in = reinterpret_cast<const cx<float>*>(a.gsrc) + kx0;
+  __syncthreads();
+  dif_stage0_load<float, L, kNT>(tile, tw, [&](int pos, int line) {
+    return pos < a.n_src ? in[(long long)pos * a.P + line] : zero<float>();
+  });
+  __syncthreads();
+  DifRange<float, L, kNT, 1, S - 1>::run(tile, tw);
+  cx<float> src[ITER][R];
+#pragma unroll
+  for (int it = 0; it < ITER; it++) {
+    const int u = it * kNT + threadIdx.x;
+    if (SS::NU % kNT == 0 || u < SS::NU) {
+      const int line = u % TB, g = u / TB;
+#pragma unroll
+      for (int q = 0; q < R; q++) src[it][q] = tile[tidx<false>(g * R + q, line)];
+      Dft<float, R, false>::run(src[it]);
+    }
+  }
+  for (int z = z0; z < z1; z++) {
+    // first inverse stage of plane z (its own positions of the tile; the last stage of the
+    // plane before has been read, except on the first round, where the positions are its own)
+    if (z > z0) __syncthreads();
 #pragma unroll
     for (int it = 0; it < ITER; it++) {
       const int u = it * kNT + threadIdx.x;
       if (SS::NU % kNT == 0 || u < SS::NU) {
         const int line = u % TB, g = u / TB;
-        Dft<float, R, true>::run(v[it]);
+        cx<float> v[R];
 #pragma unroll
-        for (int q = 0; q < R; q++) tile[tidx<false>(g * R + q, line)] = v[it][q];
+        for (int q = 0; q < R; q++) {
+          const cx<float> x = src[it][q];
+          v[q] = c >= 4 ? mk(f[it][q] * x.y, -f[it][q] * x.x) : mk(f[it][q] * x.x, f[it][q] * x.y);  // (-i f) v for xz, yz
+        }
+        Dft<float, R, true>::run(v);
+#pragma unroll
+        for (int q = 0; q < R; q++) tile[tidx<false>(g * R + q, line)] = v[q];
       }
     }
-  } else {
-    dit_last_load<float, L, kNT>(tile, [&](int pos, int line) {
-      const int ky = k_of_pos<L>(pos);
-      const bool lo = ky <= L / 2;
-      const int kyf = lo ? ky : L - ky;
-      const float sy = lo ? 1.0f : -1.0f;
-      const int kx = kx0 + line;
-      const float* t = a.Tz + kyf * (long long)a.P + kx;
-      const long long so = (long long)pos * a.P + kx;
-      cx<float> acc = zero<float>();
-      for (int p = 0; p < a.nzin; p++) {
-        const int zp = a.zin0 + p;
-        for (int i = 0; i < a.nin; i++) {
-          const cx<float> v = src[a.in_slot[i] * a.src_cstride + zp * a.src_zstride + so];
-          float sa, sb;
-          tensor_s(t, a.Tc, a.Tdz, sy, z - zp, a.coef[o][i], a.need[o][i], sa, sb);
-          acc = acc + mk(sa * v.x + sb * v.y, sa * v.y - sb * v.x);
-        }
-      }
-      return acc;
+    if (z + 1 < z1) load_factors(z + 1);
+    __syncthreads();
+    DitRange<float, L, kNT, 1, S - 1>::run(tile, tw);
+    cx<float>* out = reinterpret_cast<cx<float>*>(a.out) + a.out_slot[0] * a.out_cstride + z * a.out_zstride + kx0;
+    dit_stage0_store<float, L, kNT>(tile, tw, [&](int pos, int line, cx<float> v) {
+      if (pos < a.n_out) out[(long long)pos * a.P + line] = v;
     });
   }
-  __syncthreads();
-  DitRange<float, L, kNT, 1, S - 1>::run(tile, tw);
-  dit_stage0_store<float, L, kNT>(tile, tw, [&](int pos, int line, cx<float> v) {
-    if (pos < a.n_out) out[(long long)pos * a.P + line] = v;
-  });
 }
 
-// Forward: one output plane, one output; block (chunk of kx, chunk of z planes) of
-// NTF threads (twice the FFT kernels' block: half the sums per thread, twice the warps).
 constexpr int NTF = 2 * kNT;
-template <int L, bool SIMPLE>
-__global__ void __launch_bounds__(NTF, 1) k_yz_fwd(YZArgs a, int c) {
-  constexpr int S = plan_stages(L);
-  using SL = StageShape<L, S - 1>;
-  constexpr int R = SL::R, ITER = (SL::NU + NTF - 1) / NTF;
-  extern __shared__ __align__(16) unsigned char smem[];
-  cx<float>* tw = reinterpret_cast<cx<float>*>(smem);
-  cx<float>* tile = tw + L;
-  load_twiddles<float, NTF>(tw, reinterpret_cast<const cx<float>*>(a.tw), L);
-  const int kx0 = blockIdx.x * TB;
-  const int zb0 = a.zin0 + blockIdx.y * a.zchunk;
-  const int zb1 = min(zb0 + a.zchunk, a.zin0 + a.nzin);
-  cx<float> acc[ITER][R];
-#pragma unroll
-  for (int it = 0; it < ITER; it++)
-#pragma unroll
-    for (int q = 0; q < R; q++) acc[it][q] = zero<float>();
-  const cx<float>* in0 = reinterpret_cast<const cx<float>*>(a.in);
-  for (int z = zb0; z < zb1; z++) {
-    for (int i = 0; i < (SIMPLE ? 1 : a.nin); i++) {
-      const cx<float>* in = in0 + a.in_slot[i] * a.in_cstride + z * a.in_zstride + kx0;
-      __syncthreads();
-      dif_stage0_load<float, L, NTF>(tile, tw, [&](int pos, int line) {
-        return pos < a.n_in ? in[(long long)pos * a.P + line] : zero<float>();
-      });
-      __syncthreads();
-      DifRange<float, L, NTF, 1, S - 1>::run(tile, tw);
-      // last stage in registers, then s(zo - z) times the spectrum into the sums
-      const int dz = a.zout - z;
-#pragma unroll
-      for (int it = 0; it < ITER; it++) {
-        const int u = it * NTF + threadIdx.x;
-        if (SL::NU % NTF == 0 || u < SL::NU) {
-          const int line = u % TB, g = u / TB;
-          cx<float> v[R];
-#pragma unroll
-          for (int q = 0; q < R; q++) v[q] = tile[tidx<false>(g * R + q, line)];
-          Dft<float, R, false>::run(v);
-          const int kb = k_of_group<L>(g);
-          const int kx = kx0 + line;
-#pragma unroll
-          for (int q = 0; q < R; q++) {
-            const int ky = kb + q * (L / R);
-            const bool lo = ky <= L / 2;
-            const float* t = a.Tz + (lo ? ky : L - ky) * (long long)a.P + kx;
-            if constexpr (SIMPLE) {
-              const int adz = dz < 0 ? -dz : dz;
-              float f = a.coef[0][c] * t[c * a.Tc + adz * a.Tdz];
-              if ((c == 3 || c == 5) && !lo) f = -f;
-              if (c >= 4 && dz < 0) f = -f;
-              acc[it][q] = acc[it][q] + (c >= 4 ? mk(f * v[q].y, -f * v[q].x) : mk(f * v[q].x, f * v[q].y));
-            } else {
-              float sa, sb;
-              tensor_s(t, a.Tc, a.Tdz, lo ? 1.0f : -1.0f, dz, a.coef[i], a.need[i], sa, sb);
-              acc[it][q] = acc[it][q] + mk(sa * v[q].x + sb * v[q].y, sa * v[q].y - sb * v[q].x);
-            }
-          }
-        }
-      }
-    }
-  }
-  // partial of this z chunk, at the spectrum's positions
-  cx<float>* part = reinterpret_cast<cx<float>*>(a.part) + (long long)blockIdx.y * L * a.P + kx0;
-#pragma unroll
-  for (int it = 0; it < ITER; it++) {
-    const int u = it * NTF + threadIdx.x;
-    if (SL::NU % NTF == 0 || u < SL::NU) {
-      const int line = u % TB, g = u / TB;
-#pragma unroll
-      for (int q = 0; q < R; q++) part[(long long)(g * R + q) * a.P + line] = acc[it][q];
-    }
-  }
-}
 
-
-// The single-component forward with the next design plane's input rows and tensor
-// slice copied into shared memory (cp.async, two buffers) while the current plane is
+// Forward, lengths without the warp-specialized kernel: block (chunk of kx, chunk of z planes)
+// of NTF threads (twice the FFT kernels' block: half the sums per thread, twice the warps).
+// The next design plane's input rows and tensor
+// slice are copied into shared memory (cp.async, two buffers) while the current plane is
 // transformed, so the loads overlap the transform instead of following it.
 __device__ __forceinline__ void cp16(void* sdst, const void* gsrc) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(sdst);
@@ -226,6 +144,7 @@ __global__ void __launch_bounds__(NTF, 1) k_yz_fwd_staged(YZArgs a, int c) {
   cx<float>* sin0 = tile + L * TB;                               // [2][L/2][TB] input rows
   float* st0 = reinterpret_cast<float*>(sin0 + 2 * (L / 2) * TB);  // [2][KY][TB] tensor slice
   load_twiddles<float, NTF>(tw, reinterpret_cast<const cx<float>*>(a.tw), L);
+  pdl_wait();  // the x spectra and the partials belong to earlier kernels
   const int kx0 = blockIdx.x * TB;
   const int zb0 = a.zin0 + blockIdx.y * a.zchunk;
   const int zb1 = min(zb0 + a.zchunk, a.zin0 + a.nzin);
@@ -303,6 +222,57 @@ __global__ void __launch_bounds__(NTF, 1) k_yz_fwd_staged(YZArgs a, int c) {
       for (int q = 0; q < R; q++) part[(long long)(g * R + q) * a.P + line] = acc[it][q];
     }
   }
+}
+
+// The target plane after k_yz_fwd_staged: block cb adds the partials of its 16 lines over the z
+// chunks in order, straight into the first stage of their inverse y transform, and writes the
+// rows y < n_in of A (the sums and the transform were two launches, 6.3 + 2.9 us at L = 128 with
+// 22 chunks, this 6.6).
+template <int L>
+__global__ void __launch_bounds__(kNT) k_yz_finish_chunks(YZArgs a, int nch) {
+  constexpr int S = plan_stages(L);
+  using SS = StageShape<L, S - 1>;
+  constexpr int R = SS::R, ITER = (SS::NU + kNT - 1) / kNT;
+  extern __shared__ __align__(16) unsigned char smem[];
+  cx<float>* tw = reinterpret_cast<cx<float>*>(smem);
+  cx<float>* tile = tw + L;
+  load_twiddles<float, kNT>(tw, reinterpret_cast<const cx<float>*>(a.tw), L);
+  pdl_wait();  // the partials come from the forward kernel
+  const int kx0 = blockIdx.x * TB;
+  const cx<float>* part = reinterpret_cast<const cx<float>*>(a.part) + kx0;
+  const long long plane = (long long)L * a.P;
+#pragma unroll 1
+  for (int it = 0; it < ITER; it++) {
+    const int u = it * kNT + threadIdx.x;
+    if (SS::NU % kNT == 0 || u < SS::NU) {
+      const int line = u % TB, g = u / TB;
+      const cx<float>* pu = part + (long long)g * R * a.P + line;
+      cx<float> v[R];
+#pragma unroll
+      for (int q = 0; q < R; q++) v[q] = zero<float>();
+      constexpr int NC = R >= 16 ? 2 : R >= 8 ? 4 : 8;  // chunks whose loads are in flight together
+      for (int c0 = 0; c0 < nch; c0 += NC) {
+        cx<float> w[NC][R];
+#pragma unroll
+        for (int k = 0; k < NC; k++)
+#pragma unroll
+          for (int q = 0; q < R; q++) w[k][q] = c0 + k < nch ? pu[(c0 + k) * plane + q * a.P] : zero<float>();
+#pragma unroll
+        for (int k = 0; k < NC; k++)
+#pragma unroll
+          for (int q = 0; q < R; q++) v[q] = v[q] + w[k][q];
+      }
+      Dft<float, R, true>::run(v);
+#pragma unroll
+      for (int q = 0; q < R; q++) tile[tidx<false>(g * R + q, line)] = v[q];
+    }
+  }
+  __syncthreads();
+  DitRange<float, L, kNT, 1, S - 1>::run(tile, tw);
+  cx<float>* out = reinterpret_cast<cx<float>*>(a.yrows) + kx0;
+  dit_stage0_store<float, L, kNT>(tile, tw, [&](int pos, int line, cx<float> v) {
+    if (pos < a.n_in) out[(long long)pos * a.P + line] = v;
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -712,7 +682,7 @@ __global__ void __launch_bounds__(NTF, 1) k_zy_adj_ws(ZYArgs a, const __grid_con
               DftF<R1, false>::run(sv[it]);
             }
             bar_named(kBarGroup, kNT);  // the tile is free for this round's first stage
-          } else {
+          } else {  // the source given as its y spectrum
 #pragma unroll
             for (int it = 0; it < 2; it++) {
               const int u = it * kNT + t, line = u % TB, g = u / TB;
@@ -783,20 +753,6 @@ __global__ void __launch_bounds__(NTF, 1) k_zy_adj_ws(ZYArgs a, const __grid_con
   }
 }
 
-// out[pos][kx] = sum over z chunks of the partials, in chunk order
-__global__ void k_yz_reduce(const float2* part, int nchunks, long long plane, float2* out) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < plane;
-       e += (long long)gridDim.x * blockDim.x) {
-    float2 s = part[e];
-    for (int c = 1; c < nchunks; c++) {
-      const float2 v = part[(long long)c * plane + e];
-      s.x += v.x;
-      s.y += v.y;
-    }
-    out[e] = s;
-  }
-}
-
 template <int L>
 size_t fused_smem() {
   return (size_t)(L + L * TB) * sizeof(float2);
@@ -805,18 +761,25 @@ size_t fused_smem() {
 // the single tensor component of (o, i) = (0, 0), or -1
 int single_component(const int need) { return (need != 0 && (need & (need - 1)) == 0) ? __builtin_ctz(need) : -1; }
 
-template <int L, bool SIMPLE>
+int sm_count();
+
+template <int L>
 int launch_adj(const ZYArgs& a, int c, cudaStream_t s) {
   const size_t sm = fused_smem<L>();
   static bool init = false;
   if (!init) {
-    if (cudaFuncSetAttribute(k_zy_adj<L, SIMPLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-        cudaSuccess)
-      return -1;
+    if (cudaFuncSetAttribute(k_zy_adj<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) return -1;
     init = true;
   }
-  k_zy_adj<L, SIMPLE><<<dim3(a.P / TB, a.nzout, a.nout), kNT, sm, s>>>(a, c);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+  // planes per block: two blocks per SM, as many as are resident, each with the source's
+  // transform once (a 128^3 step takes 72.7 us, with one block per SM 74.7, with three 77;
+  // sixteen concurrent 64^2 x 72 optimizations gain 2.7% from one and lose 6% with three)
+  const int cols = a.P / TB, want = (2 * sm_count() + cols - 1) / cols;
+  const int zper = (a.nzout + want - 1) / want;
+  return launch_k(k_zy_adj<L>, dim3(cols, (a.nzout + zper - 1) / zper), dim3(kNT), sm, s, a.pdl != 0, a, c, zper) ==
+                 cudaSuccess
+             ? (a.zero_word ? 1 : 0)  // 1: *zero_word is cleared
+             : -1;
 }
 
 // 2-D map over a row-major array of `outer` rows of `inner` elements, row pitch `pitch`
@@ -904,25 +867,16 @@ int launch_adj_ws_c(const ZYArgs& a, int c, const CUtensorMap& ms, cudaStream_t 
 
 template <int L>
 int run_zy_adj(const ZYArgs& a, cudaStream_t s) {
-  if (a.nzout <= 0 || a.nout <= 0) return 0;
+  if (a.nzout <= 0) return 0;
   const int c = single_component(a.need[0][0]);
-  if (a.nin == 1 && a.nout == 1 && a.nzin == 1 && c >= 0) {
-    if constexpr (yz_ws_plan<L>()) {
-      CUtensorMap ms;
-      if (a.Ts && a.nzin_total > 0 && a.n_src <= L / 2 &&
-          slice_map(&ms, a.Ts, (long long)a.nzin_total * (L / 2 + 1), a.P, slice_box_rows<L>()))
-        return a.n_out == L / 2 ? launch_adj_ws_c<L, true>(a, c, ms, s) : launch_adj_ws_c<L, false>(a, c, ms, s);
-    }
-    if (a.gsrc) return -1;  // the source's y transform is only done on the warp-specialized path
-    return launch_adj<L, true>(a, c, s);
+  if (a.nin != 1 || a.nout != 1 || a.nzin != 1 || c < 0 || (!a.gsrc && !a.src)) return -1;
+  if constexpr (yz_ws_plan<L>()) {
+    CUtensorMap ms;
+    if (a.Ts && a.nzin_total > 0 && a.n_src <= L / 2 &&
+        slice_map(&ms, a.Ts, (long long)a.nzin_total * (L / 2 + 1), a.P, slice_box_rows<L>()))
+      return a.n_out == L / 2 ? launch_adj_ws_c<L, true>(a, c, ms, s) : launch_adj_ws_c<L, false>(a, c, ms, s);
   }
-  if (a.gsrc) return -1;
-  return launch_adj<L, false>(a, -1, s);
-}
-
-template <int L>
-constexpr bool ws_length() {
-  return yz_ws_plan<L>();
+  return a.gsrc ? launch_adj<L>(a, c, s) : -1;
 }
 
 template <int L>
@@ -940,22 +894,9 @@ int launch_fwd_staged(const YZArgs& a, int c, int nch, cudaStream_t s) {
       return -1;
     init = true;
   }
-  k_yz_fwd_staged<L><<<dim3(a.P / TB, nch), NTF, sm, s>>>(a, c);
-  return 0;
-}
-
-template <int L, bool SIMPLE>
-int launch_fwd(const YZArgs& a, int c, int nch, cudaStream_t s) {
-  const size_t sm = fused_smem<L>();
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_yz_fwd<L, SIMPLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-        cudaSuccess)
-      return -1;
-    init = true;
-  }
-  k_yz_fwd<L, SIMPLE><<<dim3(a.P / TB, nch), NTF, sm, s>>>(a, c);
-  return 0;
+  return launch_k(k_yz_fwd_staged<L>, dim3(a.P / TB, nch), dim3(NTF), sm, s, a.pdl != 0, a, c) == cudaSuccess
+             ? 2  // 2: partials of the z chunks written; launch_yz_finish completes the target plane
+             : -1;
 }
 
 template <int L, int C, bool FULL>
@@ -1001,15 +942,9 @@ int launch_fwd_single(const YZArgs& a, int c, int nch, cudaStream_t s) {
 
 template <int L>
 int run_yz_fwd(const YZArgs& a, cudaStream_t s) {
-  const int nch = (a.nzin + a.zchunk - 1) / a.zchunk;
   const int c = single_component(a.need[0]);
-  const int r = a.nin == 1 && c >= 0 ? launch_fwd_single<L>(a, c, nch, s) : launch_fwd<L, false>(a, -1, nch, s);
-  if (r != 0) return r;
-  const long long plane = (long long)L * a.P;
-  const long long b = (plane + 255) / 256;
-  k_yz_reduce<<<(int)(b > 2048 ? 2048 : b), 256, 0, s>>>(reinterpret_cast<const float2*>(a.part), nch, plane,
-                                                        a.out + a.out_slot * a.out_cstride + a.zout * plane);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+  if (a.nin != 1 || c < 0) return -2;
+  return launch_fwd_single<L>(a, c, (a.nzin + a.zchunk - 1) / a.zchunk, s);
 }
 
 }  // namespace
@@ -1026,7 +961,21 @@ int launch_zy_adj(int L, const ZYArgs& a, cudaStream_t s) {
 }
 
 template <int L>
-int run_yz_finish(const YZArgs& a, cudaStream_t s) {
+int run_yz_finish(const YZArgs& a, int how, cudaStream_t s) {
+  if (how == 2) {
+    const size_t sm = fused_smem<L>();
+    static bool init = false;
+    if (!init) {
+      if (cudaFuncSetAttribute(k_yz_finish_chunks<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
+          cudaSuccess)
+        return -1;
+      init = true;
+    }
+    return launch_k(k_yz_finish_chunks<L>, dim3(a.P / TB), dim3(kNT), sm, s, a.pdl != 0, a,
+                    (a.nzin + a.zchunk - 1) / a.zchunk) == cudaSuccess
+               ? 0
+               : -1;
+  }
   if constexpr (yz_ws_plan<L>()) {
     const long long items = (long long)(a.P / TB) * a.nzin;
     const int blocks = (int)(items < sm_count() ? items : sm_count());  // the forward's grid
@@ -1038,26 +987,15 @@ int run_yz_finish(const YZArgs& a, cudaStream_t s) {
   return -1;
 }
 
-int launch_yz_finish(int L, const YZArgs& a, cudaStream_t s) {
+int launch_yz_finish(int L, const YZArgs& a, int how, cudaStream_t s) {
   switch (L) {
 #define TM_CASE(LL) \
   case LL:          \
-    return run_yz_finish<LL>(a, s);
+    return run_yz_finish<LL>(a, how, s);
     TM_FOR_EACH_L(TM_CASE)
 #undef TM_CASE
   }
   return -2;
-}
-
-bool zy_adj_ws_length(int L) {
-  switch (L) {
-#define TM_CASE(LL) \
-  case LL:          \
-    return ws_length<LL>();
-    TM_FOR_EACH_L(TM_CASE)
-#undef TM_CASE
-  }
-  return false;
 }
 
 int launch_yz_fwd(int L, const YZArgs& a, cudaStream_t s) {

@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const
         add_dot(acc[MODE == ONE_IN ? k : 0], t, MODE == ONE_IN ? a.v[k] : a.u[k], x[MODE == ONE_IN ? 0 : k]);
     }
   };
+  pdl_wait();  // inputs and outputs belong to earlier kernels
   if (a.nzout <= a.nzin) {  // few outputs: stream the inputs onto NP x NO sums
     cx<float> acc[COLS][NP][NO];
 #pragma unroll

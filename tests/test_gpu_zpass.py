@@ -118,3 +118,47 @@ def test_direct_planes(n, nzd, z0, np_):
                 J, G = m.evaluate(up(rho))
                 assert abs(J - Jr) <= 1e-5 * abs(Jr)
                 assert rel(G.cpu().numpy(), Gr) <= 1e-5
+
+
+@pytest.mark.parametrize("L", [8, 12, 16, 18, 24, 32, 36, 48, 64, 72, 96, 128, 144, 192, 256, 288, 384, 512, 576])
+def test_single_product_every_length(L):
+    """One target plane and one tensor component with a full and an odd grid at every length of
+    x and y: the y transforms fused with the z sums, the plane's finish and the objective."""
+    from paper_1707_09898_gb300 import Magnet
+
+    for n, lengths in (((L // 2, 5, 5), (L, 0, 0)), ((5, L // 2, 5), (0, L, 0)), ((7, max(4, L // 2 - 3), 4), (0, L, 0))):
+        nx, ny, nz = n
+        rho, gH, _ = case(nx, ny, nz, nz - 1, L)
+        op = C.FFTOperator(C.Geometry(n, nz - 1, (1e-3,) * 3))
+        m = Magnet(n, nz - 1, (1e-3,) * 3, M0=(0.0, 0.0, W.MS), p=3.0, device=0, fft_lengths=lengths)
+        mask = (gH[0] > -0.5).astype(np.uint8)
+        mask[:nz - 1] = 0
+        Ht = (0.05 * W.MS * gH).astype(np.float32)
+        for M0, w in (((0.0, 0.0, W.MS), (0.0, 0.0, 1.0)), ((0.0, 0.0, W.MS), (0.0, 1.0, 0.0)),
+                      ((W.MS, 0.0, 0.0), (0.0, 0.5, 0.0)), ((W.MS, 0.0, 0.0), (0.0, 0.0, 2.0))):
+            m.set_M0(M0)
+            Jr, Gr, _ = O.objective_and_gradient(op, rho, np.array(M0), 3.0, mask, Ht, w)
+            m.set_target(up(mask), Ht=up(Ht), w=w)
+            J, G = m.evaluate(up(rho))
+            assert abs(J - Jr) <= 1e-5 * abs(Jr)
+            assert rel(G.cpu().numpy(), Gr) <= 1e-5
+
+
+@pytest.mark.parametrize("n,nzd", [((128, 12, 83), 82), ((144, 9, 75), 75), ((200, 24, 61), 37)])
+def test_single_product_planes_per_block(n, nzd):
+    """More design planes than blocks of a column: two and more planes per block, the last
+    block with fewer."""
+    from paper_1707_09898_gb300 import Magnet
+
+    nx, ny, nz = n
+    rho, gH, _ = case(nx, ny, nz, nzd, nx)
+    op = C.FFTOperator(C.Geometry(n, nzd, (1e-3,) * 3))
+    m = Magnet(n, nzd, (1e-3,) * 3, M0=(0.0, 0.0, W.MS), p=3.0, device=0)
+    mask = np.zeros((nz, ny, nx), np.uint8)
+    mask[nz // 2, 1:ny - 1, 1:nx - 2] = 1
+    Ht = (0.05 * W.MS * gH).astype(np.float32)
+    Jr, Gr, _ = O.objective_and_gradient(op, rho, np.array([0.0, 0.0, W.MS]), 3.0, mask, Ht, (0.0, 1.0, 0.0))
+    m.set_target(up(mask), Ht=up(Ht), w=(0.0, 1.0, 0.0))
+    J, G = m.evaluate(up(rho))
+    assert abs(J - Jr) <= 1e-5 * abs(Jr)
+    assert rel(G.cpu().numpy(), Gr) <= 1e-5
