@@ -577,12 +577,15 @@ int yz_forward(tm_ctx* ctx, const ConvSpec& cs, int zo, cudaStream_t s) {
   return TM_OK;
 }
 
-// direct z sum from the source plane zi0 (x spectra in A, transformed along y by the kernel)
-// fused with the inverse y transform of every design plane
-int zy_adjoint(tm_ctx* ctx, const ConvSpec& cs, int zi0, cudaStream_t s) {
+// direct z sum from the source plane zi0 fused with the inverse y transform of every design
+// plane; yfwd_inside: the source is given as x spectra in A and transformed along y by the kernel
+int zy_adjoint(tm_ctx* ctx, const ConvSpec& cs, int zi0, cudaStream_t s, bool yfwd_inside) {
   const int Ly = ctx->L[1];
   const long long P = ctx->P;
   ZYArgs z{};
+  z.src = ctx->B;
+  z.src_cstride = (long long)ctx->nz * Ly * P;
+  z.src_zstride = (long long)Ly * P;
   z.out = ctx->A;
   z.out_cstride = (long long)ctx->nz * ctx->ny * P;
   z.out_zstride = (long long)ctx->ny * P;
@@ -621,9 +624,10 @@ int zy_adjoint(tm_ctx* ctx, const ConvSpec& cs, int zi0, cudaStream_t s) {
     // after a rebuild it must start only once the scaling kernel has finished
     if (rebuilt) z.pdl = 0;
   }
-  // the source plane as x spectra: rows y < ny of plane zi0 of A slot ain[0]
-  z.gsrc = ctx->A + cs.ain[0] * ((long long)ctx->nz * ctx->ny * P) + (long long)zi0 * ctx->ny * P;
-  z.n_src = ctx->ny;
+  if (yfwd_inside) {  // the source plane as x spectra: rows y < ny of plane zi0 of A slot ain[0]
+    z.gsrc = ctx->A + cs.ain[0] * ((long long)ctx->nz * ctx->ny * P) + (long long)zi0 * ctx->ny * P;
+    z.n_src = ctx->ny;
+  }
   Timed t(ctx, KIND_ZYA, s);
   const int r = launch_zy_adj(Ly, z, s);
   if (r < 0) CKL(r);
@@ -1172,14 +1176,17 @@ int adjoint_planes(tm_ctx* ctx, const float* rho, float* dJdrho, const int* F, c
     }
   }
   // fused only in its single-spectrum, single-component form; with several spectra or
-  // tensor components the separate passes measured faster. The fused kernel reads the source
-  // rows from A while it writes the design planes into A, so its output goes to another slot
-  // (the target plane may be a design plane).
-  if (ctx->fuse_yz && np == 1 && single_product(ca)) {
-    ca.aout[0] = (ca.ain[0] + 1) % kSlotsA;
-    if ((r = zy_adjoint(ctx, ca, ctx->tz0, s))) return r;
+  // tensor components the separate passes measured faster
+  const bool fused = ctx->fuse_yz && np == 1 && single_product(ca);
+  // on the warp-specialized path the fused adjoint runs the source's y transform itself;
+  // it then reads the source rows from A while it writes the design planes into A, so its
+  // output goes to another slot (the target plane may be a design plane)
+  const bool yfwd_inside = fused && zy_adj_ws_length(ctx->L[1]) && ctx->ny <= ctx->L[1] / 2;
+  if (yfwd_inside) ca.aout[0] = (ca.ain[0] + 1) % kSlotsA;
+  if (!yfwd_inside && (r = ypass(ctx, false, ca.nin, ca.ain, ca.bin, ctx->tz0, np, s))) return r;
+  if (fused) {
+    if ((r = zy_adjoint(ctx, ca, ctx->tz0, s, yfwd_inside))) return r;
   } else {
-    if ((r = ypass(ctx, false, ca.nin, ca.ain, ca.bin, ctx->tz0, np, s))) return r;
     if ((r = zdirect(ctx, ca, ctx->tz0, np, 0, ctx->nzd, s))) return r;
     if ((r = ypass(ctx, true, ca.nout, ca.aout, ca.bout, 0, ctx->nzd, s, ctx->gmax))) return r;
     ctx->gmax_zeroed = true;

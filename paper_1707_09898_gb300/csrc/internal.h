@@ -169,8 +169,8 @@ struct ZDirArgs {
 int launch_zdir(const ZDirArgs& a, cudaStream_t s);
 
 // Fused y transform + direct z sum (k_yzfused.cu).
-// Adjoint: from one source plane, given as x spectra, to the real-y rows of every output
-// plane of A (one spectrum, one tensor component).
+// Adjoint: from one source plane to the real-y rows of every output plane of A (one spectrum,
+// one tensor component).
 struct ZYArgs {
   const float2* src;                        // B [slot][z][Ly][P]
   long long src_cstride, src_zstride;
@@ -187,10 +187,8 @@ struct ZYArgs {
   // warp-specialized path (one tensor component c): Ts = coef[0][0][c] * Tz[c], [nzin_total][Ly/2+1][P]
   const float* Ts;
   int nzin_total;                           // z offsets held by Ts
-  // the source plane as x spectra, rows [n_src][P]: the kernel runs its forward y transform.
-  // Null (L = 512 only): the y spectrum is read from src. No caller does so now, but without
-  // that branch the compiler spills 48 bytes instead of 28 and the kernel takes 66.6 us instead
-  // of 61.8 for 256 planes of 256^2.
+  // if set (warp-specialized path only): the source plane as x spectra, rows [n_src][P]; the
+  // kernel runs its forward y transform itself and src is not read
   const float2* gsrc;
   int n_src;
   unsigned* status;                         // device word: bit 0 set when a copy wait timed out
@@ -222,6 +220,9 @@ struct YZArgs {
   int pdl;                                  // launch with programmatic dependent launch
 };
 int launch_zy_adj(int L, const ZYArgs& a, cudaStream_t s);
+// whether launch_zy_adj takes the warp-specialized path for length L (Ts given), the path that can
+// run the source's y transform
+bool zy_adj_ws_length(int L);
 int launch_yz_fwd(int L, const YZArgs& a, cudaStream_t s);
 // after launch_yz_fwd returned how = 1 (segment partials of the warp-specialized kernel) or 2
 // (partials of z chunks): the partials added in order, and the target plane's inverse y

@@ -11,9 +11,9 @@
 //             and accumulates s Y in registers; k_yz_finish_chunks (k_yz_finish) adds the
 //             chunks in a fixed order and runs the target plane's inverse y transform.
 //   adjoint:  Y(kx, ky, z) = s(kx, ky, z - zp) src(kx, ky, zp) for every design plane z,
-//             followed by the inverse y transform: k_zy_adj (k_zy_adj_ws) runs the source
-//             plane's forward y transform, keeps the spectrum in registers, and forms and
-//             transforms the design planes of its block.
+//             followed by the inverse y transform: k_zy_adj forms Y in the loader of the
+//             inverse transform from the source's y spectrum; k_zy_adj_ws also runs the
+//             source plane's forward y transform and keeps the spectrum in registers.
 // One spectrum, one tensor component and one plane; other cases run the separate passes.
 // Same discrete convolution as the unfused passes, without the round trip of the
 // y spectra of all design planes through HBM.
@@ -26,94 +26,72 @@ namespace tmk {
 
 namespace {
 
-// Adjoint, lengths without the warp-specialized kernel: block (chunk of kx, planes of z). The
-// source plane's rows (x spectra) are transformed along y once per block, their spectrum stays
-// in registers (unit (line, g) of the last stage: positions g R + q, frequencies k(g R) + q
-// L/R), and each plane of the block is formed and transformed back from it; the tensor row
-// of the next plane is loaded meanwhile. A launch of its own for the source's transform, and
-// one block per plane, took 3.5 + 4.5 us at 64^2 planes (L = 128), this 5.9; 3.5 + 12.4 at
-// 128^2 (L = 256), this 14.6.
+// Adjoint, lengths without the warp-specialized kernel: block (chunk of kx, plane of z), from the
+// source's y spectrum in B. One source plane, one tensor component c (its sign under y and z
+// reflection folded in): each element is one source load and one tensor load with no loop, so all
+// loads of a thread are in flight together. With the source's transform inside (one launch
+// less) and several planes per block a 64^2 x 72 step took 64.9 us instead of 63.3, sixteen
+// concurrent optimizations 1640 us instead of 1521, a 128^3 step 72.8 instead of 73.2.
 template <int L>
-__global__ void __launch_bounds__(kNT, L >= 288 ? 1 : 2) k_zy_adj(ZYArgs a, int c, int zper) {
+__global__ void __launch_bounds__(kNT, 2) k_zy_adj(ZYArgs a, int c) {
   constexpr int S = plan_stages(L);
-  using SS = StageShape<L, S - 1>;
-  constexpr int R = SS::R, ITER = (SS::NU + kNT - 1) / kNT;
   extern __shared__ __align__(16) unsigned char smem[];
   cx<float>* tw = reinterpret_cast<cx<float>*>(smem);
   cx<float>* tile = tw + L;
   load_twiddles<float, kNT>(tw, reinterpret_cast<const cx<float>*>(a.tw), L);
   const int kx0 = blockIdx.x * TB;
-  const int z0 = a.zout0 + blockIdx.y * zper, z1 = min(z0 + zper, a.zout0 + a.nzout);
-  const float* tcol = a.Tz + c * a.Tc + kx0;
-  float f[ITER][R];
-  auto load_factors = [&](int z) {
-    const int dz = z - a.zin0, adz = dz < 0 ? -dz : dz;
-    const float cz = (c >= 4 && dz < 0) ? -a.coef[0][0][c] : a.coef[0][0][c];
-    const float* t = tcol + adz * a.Tdz;
-#pragma unroll
-    for (int it = 0; it < ITER; it++) {
-      const int u = it * kNT + threadIdx.x;
-      if (SS::NU % kNT == 0 || u < SS::NU) {
-        const int line = u % TB, kb = k_of_group<L>(u / TB);
-#pragma unroll
-        for (int q = 0; q < R; q++) {
-          const int ky = kb + q * (L / R);
-          const bool lo = ky <= L / 2;
-          const float v = cz * t[(lo ? ky : L - ky) * a.P + line];
-          f[it][q] = (c == 3 || c == 5) && !lo ? -v : v;
-        }
-      }
-    }
-  };
-  load_factors(z0);
+  const int z = a.zout0 + blockIdx.y;
+  const cx<float>* src = reinterpret_cast<const cx<float>*>(a.src);
+  cx<float>* out = reinterpret_cast<cx<float>*>(a.out) + a.out_slot[0] * a.out_cstride + z * a.out_zstride + kx0;
   pdl_wait();  // the source plane and the outputs belong to earlier kernels
   if (a.zero_word && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *a.zero_word = 0u;
-  const cx<float>* in = reinterpret_cast<const cx<float>*>(a.gsrc) + kx0;
   __syncthreads();
-  dif_stage0_load<float, L, kNT>(tile, tw, [&](int pos, int line) {
-    return pos < a.n_src ? in[(long long)pos * a.P + line] : zero<float>();
-  });
-  __syncthreads();
-  DifRange<float, L, kNT, 1, S - 1>::run(tile, tw);
-  cx<float> src[ITER][R];
-#pragma unroll
-  for (int it = 0; it < ITER; it++) {
-    const int u = it * kNT + threadIdx.x;
-    if (SS::NU % kNT == 0 || u < SS::NU) {
-      const int line = u % TB, g = u / TB;
-#pragma unroll
-      for (int q = 0; q < R; q++) src[it][q] = tile[tidx<false>(g * R + q, line)];
-      Dft<float, R, false>::run(src[it]);
-    }
-  }
-  for (int z = z0; z < z1; z++) {
-    // first inverse stage of plane z (its own positions of the tile; the last stage of the
-    // plane before has been read, except on the first round, where the positions are its own)
-    if (z > z0) __syncthreads();
+  {
+    // first inverse stage (radix R, M = 1) with the direct z sum in its loads: the
+    // positions g R + q of a group hold ky = k(g R) + q L/R, so no per-element
+    // digit reversal; sign of the folded tensor and of odd dz precomputed
+    constexpr int s = S - 1;
+    using SS = StageShape<L, s>;
+    constexpr int R = SS::R, ITER = (SS::NU + kNT - 1) / kNT;
+    const int dz = z - a.zin0;
+    const int adz = dz < 0 ? -dz : dz;
+    const float cz = (c >= 4 && dz < 0) ? -a.coef[0][0][c] : a.coef[0][0][c];
+    const float* tcol = a.Tz + c * a.Tc + adz * a.Tdz + kx0;
+    const cx<float>* srow = src + a.in_slot[0] * a.src_cstride + a.zin0 * a.src_zstride + kx0;
+    cx<float> v[ITER][R];
 #pragma unroll
     for (int it = 0; it < ITER; it++) {
       const int u = it * kNT + threadIdx.x;
       if (SS::NU % kNT == 0 || u < SS::NU) {
         const int line = u % TB, g = u / TB;
-        cx<float> v[R];
+        const int kb = k_of_group<L>(g);
 #pragma unroll
         for (int q = 0; q < R; q++) {
-          const cx<float> x = src[it][q];
-          v[q] = c >= 4 ? mk(f[it][q] * x.y, -f[it][q] * x.x) : mk(f[it][q] * x.x, f[it][q] * x.y);  // (-i f) v for xz, yz
+          const int ky = kb + q * (L / R);
+          const bool lo = ky <= L / 2;
+          const cx<float> vv = srow[(g * R + q) * a.P + line];
+          float f = cz * tcol[(lo ? ky : L - ky) * a.P + line];
+          if ((c == 3 || c == 5) && !lo) f = -f;
+          v[it][q] = c >= 4 ? mk(f * vv.y, -f * vv.x) : mk(f * vv.x, f * vv.y);  // (-i f) v for xz, yz
         }
-        Dft<float, R, true>::run(v);
-#pragma unroll
-        for (int q = 0; q < R; q++) tile[tidx<false>(g * R + q, line)] = v[q];
       }
     }
-    if (z + 1 < z1) load_factors(z + 1);
-    __syncthreads();
-    DitRange<float, L, kNT, 1, S - 1>::run(tile, tw);
-    cx<float>* out = reinterpret_cast<cx<float>*>(a.out) + a.out_slot[0] * a.out_cstride + z * a.out_zstride + kx0;
-    dit_stage0_store<float, L, kNT>(tile, tw, [&](int pos, int line, cx<float> v) {
-      if (pos < a.n_out) out[(long long)pos * a.P + line] = v;
-    });
+#pragma unroll
+    for (int it = 0; it < ITER; it++) {
+      const int u = it * kNT + threadIdx.x;
+      if (SS::NU % kNT == 0 || u < SS::NU) {
+        const int line = u % TB, g = u / TB;
+        Dft<float, R, true>::run(v[it]);
+#pragma unroll
+        for (int q = 0; q < R; q++) tile[tidx<false>(g * R + q, line)] = v[it][q];
+      }
+    }
   }
+  __syncthreads();
+  DitRange<float, L, kNT, 1, S - 1>::run(tile, tw);
+  dit_stage0_store<float, L, kNT>(tile, tw, [&](int pos, int line, cx<float> v) {
+    if (pos < a.n_out) out[(long long)pos * a.P + line] = v;
+  });
 }
 
 constexpr int NTF = 2 * kNT;
@@ -682,7 +660,7 @@ __global__ void __launch_bounds__(NTF, 1) k_zy_adj_ws(ZYArgs a, const __grid_con
               DftF<R1, false>::run(sv[it]);
             }
             bar_named(kBarGroup, kNT);  // the tile is free for this round's first stage
-          } else {  // the source given as its y spectrum
+          } else {
 #pragma unroll
             for (int it = 0; it < 2; it++) {
               const int u = it * kNT + t, line = u % TB, g = u / TB;
@@ -761,8 +739,6 @@ size_t fused_smem() {
 // the single tensor component of (o, i) = (0, 0), or -1
 int single_component(const int need) { return (need != 0 && (need & (need - 1)) == 0) ? __builtin_ctz(need) : -1; }
 
-int sm_count();
-
 template <int L>
 int launch_adj(const ZYArgs& a, int c, cudaStream_t s) {
   const size_t sm = fused_smem<L>();
@@ -771,12 +747,7 @@ int launch_adj(const ZYArgs& a, int c, cudaStream_t s) {
     if (cudaFuncSetAttribute(k_zy_adj<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) return -1;
     init = true;
   }
-  // planes per block: two blocks per SM, as many as are resident, each with the source's
-  // transform once (a 128^3 step takes 72.7 us, with one block per SM 74.7, with three 77;
-  // sixteen concurrent 64^2 x 72 optimizations gain 2.7% from one and lose 6% with three)
-  const int cols = a.P / TB, want = (2 * sm_count() + cols - 1) / cols;
-  const int zper = (a.nzout + want - 1) / want;
-  return launch_k(k_zy_adj<L>, dim3(cols, (a.nzout + zper - 1) / zper), dim3(kNT), sm, s, a.pdl != 0, a, c, zper) ==
+  return launch_k(k_zy_adj<L>, dim3(a.P / TB, a.nzout), dim3(kNT), sm, s, a.pdl != 0, a, c) ==
                  cudaSuccess
              ? (a.zero_word ? 1 : 0)  // 1: *zero_word is cleared
              : -1;
@@ -869,14 +840,20 @@ template <int L>
 int run_zy_adj(const ZYArgs& a, cudaStream_t s) {
   if (a.nzout <= 0) return 0;
   const int c = single_component(a.need[0][0]);
-  if (a.nin != 1 || a.nout != 1 || a.nzin != 1 || c < 0 || (!a.gsrc && !a.src)) return -1;
+  if (a.nin != 1 || a.nout != 1 || a.nzin != 1 || c < 0) return -1;
   if constexpr (yz_ws_plan<L>()) {
     CUtensorMap ms;
     if (a.Ts && a.nzin_total > 0 && a.n_src <= L / 2 &&
         slice_map(&ms, a.Ts, (long long)a.nzin_total * (L / 2 + 1), a.P, slice_box_rows<L>()))
       return a.n_out == L / 2 ? launch_adj_ws_c<L, true>(a, c, ms, s) : launch_adj_ws_c<L, false>(a, c, ms, s);
   }
-  return a.gsrc ? launch_adj<L>(a, c, s) : -1;
+  if (a.gsrc) return -1;  // the source's y transform is only done on the warp-specialized path
+  return launch_adj<L>(a, c, s);
+}
+
+template <int L>
+constexpr bool ws_length() {
+  return yz_ws_plan<L>();
 }
 
 template <int L>
@@ -996,6 +973,17 @@ int launch_yz_finish(int L, const YZArgs& a, int how, cudaStream_t s) {
 #undef TM_CASE
   }
   return -2;
+}
+
+bool zy_adj_ws_length(int L) {
+  switch (L) {
+#define TM_CASE(LL) \
+  case LL:          \
+    return ws_length<LL>();
+    TM_FOR_EACH_L(TM_CASE)
+#undef TM_CASE
+  }
+  return false;
 }
 
 int launch_yz_fwd(int L, const YZArgs& a, cudaStream_t s) {

@@ -145,9 +145,8 @@ def test_single_product_every_length(L):
 
 
 @pytest.mark.parametrize("n,nzd", [((128, 12, 83), 82), ((144, 9, 75), 75), ((200, 24, 61), 37)])
-def test_single_product_planes_per_block(n, nzd):
-    """More design planes than blocks of a column: two and more planes per block, the last
-    block with fewer."""
+def test_single_product_many_planes(n, nzd):
+    """Many design planes on a wide grid, the target inside the design or above it."""
     from paper_1707_09898_gb300 import Magnet
 
     nx, ny, nz = n
