@@ -146,7 +146,7 @@ def test_single_product_every_length(L):
 
 @pytest.mark.parametrize("n,nzd", [((128, 12, 83), 82), ((144, 9, 75), 75), ((200, 24, 61), 37)])
 def test_single_product_many_planes(n, nzd):
-    """Many design planes on a wide grid, the target inside the design or above it."""
+    """Many design planes on a wide grid, the target plane inside the design."""
     from paper_1707_09898_gb300 import Magnet
 
     nx, ny, nz = n
