@@ -179,7 +179,6 @@ __global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const
         }
       }
   } else {  // few inputs: keep them, stream the outputs
-    if (!valid) return;
     cx<float> x[COLS][NP][NI];
 #pragma unroll
     for (int c = 0; c < COLS; c++)
@@ -187,12 +186,16 @@ __global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const
       for (int p = 0; p < NP; p++)
 #pragma unroll
         for (int i = 0; i < NI; i++)
-          x[c][p][i] = p < a.nzin && (NI == 1 || i < a.nin)
+          x[c][p][i] = valid && p < a.nzin && (NI == 1 || i < a.nin)
                            ? buf[a.in_slot[i] * a.cstride + (a.zin0 + p) * a.zstride + colo[c]]
                            : zero<float>();
     const int per = (a.nzout + ZP - 1) / ZP;
     const int z0 = a.zout0 + part * per, z1 = min(z0 + per, a.zout0 + a.nzout);
-    if (z0 >= z1) return;
+    // Inputs and outputs may share a slot, and an input plane that is also an output plane (a
+    // target inside the design) belongs to one warp's z range while every warp reads it: no
+    // warp stores before all have their inputs.
+    __syncthreads();
+    if (!valid || z0 >= z1) return;
     Row r[NP];
 #pragma unroll
     for (int p = 0; p < NP - 1; p++) r[p] = row(z0 - 1 - a.zin0 - p);  // shifted into place below
