@@ -964,13 +964,18 @@ __global__ void __launch_bounds__(128) k_conv_dw_tc(const bf16* in, const bf16* 
 // output gradient (and add up the bias gradient from the float32 values they read), one thread
 // per M tile issues MMAs; the accumulators stay in tensor memory over all tiles of the block.
 // Channel chunks go in groups of 512 / (6 NO), each on its own blocks. Each block writes its
-// sums as one partial, added in block order by k_dw_finish.
+// sums as one partial, added in block order by k_dw_finish. There are as many partials as SMs
+// whatever the number of groups: the tensor core's accumulation loses about a bit per doubling
+// of the voxels that one accumulator adds up, and with the SMs divided among the groups (a
+// quarter of the partials for 64 -> 64 channels) the sums of a 64^3 x 2 layer were off by 7.5e-6
+// relative instead of 1.4e-6 (262 us; with all partials 303, k_conv_dw_halo 853).
 // What bounds it: reading the operands of the MMAs from shared memory (44 cycles for M = 128, N =
 // 48, K = 16). Measured, 64^3 x 2, 48 -> 16 channels with db: 432 -> 49 us.
-template <int W, int NO>
+// RMAX: rows of a tile at most.
+template <int W, int NO, int RMAX>
 struct DwRows {
   static constexpr int ROWB = 6 * NO * W;                     // bytes of one staged output-gradient row
-  static constexpr int MAXR = 50 * 1024 / ROWB;               // rows of a tile, two buffers of them
+  static constexpr int MAXR = 50 * 1024 / ROWB < RMAX ? 50 * 1024 / ROWB : RMAX;  // two buffers of them
   static constexpr int TZ = MAXR >= 8 ? 2 : 1, RT = MAXR >= 4 ? 4 : 2;
   static constexpr int PR = RT + 2, DROWS = TZ * RT;
   static constexpr int ABYTES = (TZ + 2) * PR * W * 32;       // one stage of input rows
@@ -983,11 +988,11 @@ struct DwRows {
   static_assert(MAXR >= 2 && GROUP >= 1 && 2 * PR + 2 <= 15 && SMEM <= 227 * 1024, "tile");
   static_assert(2 * GBYTES + 256 * 8 * 4 >= 8 * W * 32, "rows read past the stages");
 };
-template <int W, int NO>
-__global__ void __launch_bounds__(DwRows<W, NO>::THREADS, 1)
+template <int W, int NO, int RMAX>
+__global__ void __launch_bounds__(DwRows<W, NO, RMAX>::THREADS, 1)
 k_conv_dw_rows(const __grid_constant__ CUtensorMap rows, const float* dout, float* part, int Nb, int D, int H, int Cin) {
   using namespace tmk;
-  using T = DwRows<W, NO>;
+  using T = DwRows<W, NO, RMAX>;
   constexpr int TZ = T::TZ, RT = T::RT, PR = T::PR, DROWS = T::DROWS, ROWB = T::ROWB, NS = T::NS, CG = NO / 8;
   constexpr unsigned IDESC = idesc_bf16(128, 3 * NO, true);
   extern __shared__ unsigned char smem_raw[];
@@ -1180,18 +1185,17 @@ __global__ void __launch_bounds__(256) k_dw_finish(const float* part, int nblk, 
   }
 }
 
-template <int W, int NO>
-int launch_dw_rows(const bf16* in, const float* dout, float* dW, float* db, float* work, long long work_floats, int Nb,
+template <int W, int NO, int RMAX>
+int launch_dw_rows_of(const bf16* in, const float* dout, float* dW, float* db, float* work, long long work_floats, int Nb,
                    int D, int H, int Cin, cudaStream_t s) {
-  using T = DwRows<W, NO>;
+  using T = DwRows<W, NO, RMAX>;
   const long long n = 27LL * Cin * NO;
   const int skip = (int)(-(intptr_t)(reinterpret_cast<uintptr_t>(work) >> 2) & 3);  // partials from a 16-byte boundary
   work += skip;
   work_floats -= skip;
   const long long tiles = (long long)Nb * ((D + T::TZ - 1) / T::TZ) * ((H + T::RT - 1) / T::RT);
   const int groups = ((Cin >> 4) + T::GROUP - 1) / T::GROUP;
-  long long nblk = sm_count() / groups;  // one block per SM, and no more partials than work holds
-  if (nblk < 1) nblk = 1;
+  long long nblk = sm_count();  // as many partials as SMs, and no more than work holds
   if (nblk > tiles) nblk = tiles;
   if (nblk > work_floats / (n + NO)) nblk = work_floats / (n + NO);
   if (nblk < 1 || tiles > 0x7fffffffLL) return -1;
@@ -1206,14 +1210,31 @@ int launch_dw_rows(const bf16* in, const float* dout, float* dW, float* db, floa
     return -4;
   static bool init = false;
   if (!init) {
-    if (cudaFuncSetAttribute(k_conv_dw_rows<W, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM) !=
+    if (cudaFuncSetAttribute(k_conv_dw_rows<W, NO, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM) !=
         cudaSuccess)
       return -4;
     init = true;
   }
-  k_conv_dw_rows<W, NO><<<dim3((unsigned)nblk, groups), T::THREADS, T::SMEM, s>>>(rows, dout, work, Nb, D, H, Cin);
+  k_conv_dw_rows<W, NO, RMAX><<<dim3((unsigned)nblk, groups), T::THREADS, T::SMEM, s>>>(rows, dout, work, Nb, D, H, Cin);
   k_dw_finish<<<(unsigned)((n + NO + 31) / 32), 256, 0, s>>>(work, (int)nblk, n, NO, dW, db);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
+}
+
+// Tiles of at most eight rows, or of two where there are at most 16 of the large ones, or where
+// the scratch holds fewer partials than SMs: one accumulator then adds up no more voxels than it
+// has to. 8 x 8 x 64, 16 -> 16 channels: eight tiles of 512 voxels, 1.6e-7 relative error and 12.7
+// us; 32 of 128, 0.8e-7 and 10.4. 16 x 16 x 64, 96 -> 32: 64 tiles of 256, 1.2e-7 and 29 us, 128 of
+// 128, 1.1e-7 and 36 us.
+template <int W, int NO>
+int launch_dw_rows(const bf16* in, const float* dout, float* dW, float* db, float* work, long long work_floats, int Nb,
+                   int D, int H, int Cin, cudaStream_t s) {
+  using T = DwRows<W, NO, 8>;
+  if constexpr (T::DROWS > 2) {
+    const long long tiles = (long long)Nb * ((D + T::TZ - 1) / T::TZ) * ((H + T::RT - 1) / T::RT);
+    if (tiles <= 16 || work_floats / (27LL * Cin * NO + NO) < sm_count())
+      return launch_dw_rows_of<W, NO, 2>(in, dout, dW, db, work, work_floats, Nb, D, H, Cin, s);
+  }
+  return launch_dw_rows_of<W, NO, 8>(in, dout, dW, db, work, work_floats, Nb, D, H, Cin, s);
 }
 
 // Weight gradient for rows of 8 voxels (half of a K = 16 step, which k_conv_dw_rows could not
