@@ -767,13 +767,26 @@ int launch_conv_halo_tz(const void* src, const bf16* Wc, const float* bias, void
 // Two planes per tile read each staged row for more of its taps, as far as two accumulators fit
 // in tensor memory; one plane where two would leave SMs without a tile (16^3 x 2). 96 channels
 // go as two windows of 48 on their own blocks: their accumulator alone would be 288 columns
-// wide, so that no epilogue could run beside the next tile's MMAs.
+// wide, so that no epilogue could run beside the next tile's MMAs. Two planes of a window fill
+// the tensor memory in the same way, which pays where it saves more than the overlap: where each
+// stage brings its weights (more than 32 reduced channels: 64^3 x 4, 96 from 64, 850 -> 615 us),
+// and with resident weights where two planes take no more rounds of tiles than one (96 from 32,
+// 64^3 x 4 447 -> 390, 32^3 19.0 -> 18.5; 24 x 32 x 32, two rounds against three, 16.4 -> 18.5).
+// With 16 reduced channels the epilogue is most of a tile (64^3 x 4 272 with one plane, 283), and
+// so it is for rows of 8 or 16 that add to a gradient (96 from 32, 64 x 64 x 8 x 4, 55.5 and 61.5).
 template <int MODE, int W, int NO>
 int launch_conv_halo(const void* src, const bf16* Wc, const float* bias, void* dst, int Nb, int D, int H, int KC,
                      int flag, cudaStream_t s) {
   constexpr int NW = NO == 96 ? 48 : NO;
   if constexpr (NW <= 32) {
     if ((long long)Nb * ((D + 1) / 2) * ((H + 128 / W - 1) / (128 / W)) >= sm_count())
+      return launch_conv_halo_tz<MODE, W, 2, NW>(src, Wc, bias, dst, Nb, D, H, KC, NO, flag, s);
+  }
+  if constexpr (NO == 96) {
+    const int ny = (H + 128 / W - 1) / (128 / W), gx = sm_count() > 1 ? sm_count() / 2 : 1;
+    const long long t1 = (long long)Nb * D * ny, t2 = (long long)Nb * ((D + 1) / 2) * ny;
+    const bool resident = halo_smem<MODE, W, 1, NW>(3, true, KC >> 4) <= 227 * 1024;
+    if (resident ? KC > 16 && (W >= 32 || !flag) && 2 * ((t2 + gx - 1) / gx) <= (t1 + gx - 1) / gx : t2 >= gx)
       return launch_conv_halo_tz<MODE, W, 2, NW>(src, Wc, bias, dst, Nb, D, H, KC, NO, flag, s);
   }
   return launch_conv_halo_tz<MODE, W, 1, NW>(src, Wc, bias, dst, Nb, D, H, KC, NO, flag, s);
