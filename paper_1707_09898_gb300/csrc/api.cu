@@ -400,6 +400,7 @@ int conv_yz(tm_ctx* ctx, const ConvSpec& cs, int zin, int zout, cudaStream_t s) 
   z.ext = cs.ext;
   z.in_ext = cs.in_ext;
   z.out_ext = cs.out_ext;
+  z.nsm = ctx->nsm;
   z.tw = ctx->tw + Lx + Ly;
   {
     Timed t(ctx, KIND_ZPASS, s);

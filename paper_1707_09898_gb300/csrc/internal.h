@@ -145,6 +145,7 @@ struct ZArgs {
   const int2* zcol;            // launch order of columns: (ky position, ky)
   const int* ext;              // device [zlo, zhi) of the target planes
   int in_ext, out_ext;         // input / output planes restricted to ext (else 0..n_in / 0..n_out)
+  int nsm;                     // SMs of the device
   const float2* tw;
 };
 constexpr int kDirectPlanes = 4;  // at most this many planes: direct DFT instead of the z FFT

@@ -161,8 +161,9 @@ __device__ __forceinline__ float row_dot(const Signed& w, const float* n, int a)
   return n[4] * w.m[2][0] + n[5] * w.m[2][1] + n[2] * w.m[2][2];
 }
 
-// NI inputs (2 or 3: exactly so many), NO outputs (1, or 3 for two or three)
-template <int L, int NI, int NO>
+// NI inputs (2 or 3: exactly so many), NO outputs (1, or 3 for two or three). APART (NI = NO = 1):
+// the grid's third dimension is the output.
+template <int L, int NI, int NO, bool APART = false>
 __global__ void __launch_bounds__(ZPlan<L>::NT, ZPlan<L>::MINB) k_zn(const __grid_constant__ ZArgs a) {
   using Z = ZPlan<L>;
   constexpr int R0 = Z::R0, M0 = Z::M0, R = Z::R, NT = Z::NT, CH = Z::CH, TW = R0 + 2;
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(ZPlan<L>::NT, ZPlan<L>::MINB) k_zn(const __gri
     ohi = min(a.ext[1], a.n_out);
   }
   const unsigned icnt = (unsigned)max(ihi - ilo, 0), ocnt = (unsigned)max(ohi - olo, 0);
-  const int nout = NO == 1 ? 1 : a.nout;
+  const int nout = NO == 1 ? 1 : a.nout, o0 = APART ? (int)blockIdx.z : 0;
   __syncthreads();  // twiddles
 #pragma unroll
   for (int it = 0; it < (Z::NU0 + NT - 1) / NT; it++) {  // first stage: rows z = j + q M0 < L/2 in
@@ -275,8 +276,8 @@ __global__ void __launch_bounds__(ZPlan<L>::NT, ZPlan<L>::MINB) k_zn(const __gri
         const float* ne = n[e];
         const float sz = below(q) ? 1.0f : -1.0f;
         if constexpr (NI == 1 && NO == 1) {
-          const float f = ne[0] * a.coef[0][0] + ne[1] * a.coef[0][1] + ne[2] * a.coef[0][2] +
-                          ne[3] * (a.coef[0][3] * sy) + ne[4] * (a.coef[0][4] * sz) + ne[5] * (a.coef[0][5] * (sy * sz));
+          const float f = ne[0] * a.coef[o0][0] + ne[1] * a.coef[o0][1] + ne[2] * a.coef[o0][2] +
+                          ne[3] * (a.coef[o0][3] * sy) + ne[4] * (a.coef[o0][4] * sz) + ne[5] * (a.coef[o0][5] * (sy * sz));
           v[q] = scale(v[q], f);
         } else if constexpr (NI == 1) {  // outputs are components
           const Signed w = signed_by(a.u[0], sy, sz);
@@ -341,7 +342,7 @@ __global__ void __launch_bounds__(ZPlan<L>::NT, ZPlan<L>::MINB) k_zn(const __gri
 #pragma unroll
       for (int o = 0; o < NO; o++) {
         if (o < nout) {
-          cx<float>* out = reinterpret_cast<cx<float>*>(a.buf) + a.out_slot[o] * a.cstride;
+          cx<float>* out = reinterpret_cast<cx<float>*>(a.buf) + a.out_slot[o0 + o] * a.cstride;
           const cx<float>* tl = tile + o * (L * TB);
           cx<float> v[R0];
 #pragma unroll
@@ -360,25 +361,50 @@ __global__ void __launch_bounds__(ZPlan<L>::NT, ZPlan<L>::MINB) k_zn(const __gri
   }
 }
 
-template <int L, int NI, int NO>
+template <int L, int NI, int NO, bool APART = false>
 int run_zn(const ZArgs& a, cudaStream_t s) {
   using Z = ZPlan<L>;
-  const int tiles = a.nin > a.nout ? a.nin : a.nout;
+  const int tiles = APART ? 1 : a.nin > a.nout ? a.nin : a.nout;
   const size_t sm = (size_t)(ztw_size<L>() + tiles * L * TB) * sizeof(float2);
   static bool init = false;
   if (!init) {
     const size_t most = (size_t)(ztw_size<L>() + (NI > NO ? NI : NO) * L * TB) * sizeof(float2);
-    if (cudaFuncSetAttribute(k_zn<L, NI, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_zn<L, NI, NO, APART>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess)
       return -1;
     init = true;
   }
-  k_zn<L, NI, NO><<<dim3(a.P / TB, a.Ly), Z::NT, sm, s>>>(a);
+  k_zn<L, NI, NO, APART><<<dim3(a.P / TB, a.Ly, APART ? a.nout : 1), Z::NT, sm, s>>>(a);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+}
+
+// One input with several outputs: on few column tiles the outputs' inverse transforms in turn are
+// longer than the input's forward transform once more for each, on SMs that are idle otherwise.
+// The line is two blocks per SM for all outputs, three for the lengths with a factor of 9, whose
+// last stage is the longest. Field with M0 along z, outputs apart and together: 24 x 24 x 72 (96
+// tiles, L = 144) 24.6 and 28.7 us, 24 x 32 x 72 (128) 26.6 and 28.7, 16 x 16 x 64 (64, L = 128)
+// 20.8 and 22.6; 24 x 30 x 96 (128, L = 192) 26.7 and 24.6, 32 x 32 x 128 (192, L = 256) 32.8 and
+// 30.7. At L = 576 three tiles fill the shared memory of an SM and one does half of it, so rounds
+// of blocks count: 32 x 32 x 288 (192 tiles) 69.6 and 82.0, 48 x 48 x 288 (384) 159 and 180; 24 x
+// 30 x 288 (128) 55.8 and 50.4, 72 x 72 x 288 (720, tilted M0) 282 and 275.
+template <int L>
+bool outputs_apart(const ZArgs& a) {
+  if (a.nout == 1) return false;
+  for (int o = 0; o < a.nout; o++)
+    if (a.out_slot[o] == a.in_slot[0]) return false;  // another output's block may still read it
+  const long long blocks = (long long)(a.P / TB) * a.Ly;
+  if (L == 576) {
+    const long long apart = (blocks * a.nout + 2 * a.nsm - 1) / (2 * a.nsm), together = (blocks + a.nsm - 1) / a.nsm;
+    return 3 * apart <= (a.nout + 1) * together;
+  }
+  return blocks * a.nout <= (L % 9 == 0 ? 3LL : 2LL) * a.nsm;
 }
 
 template <int L>
 int run_length(const ZArgs& a, cudaStream_t s) {
-  if (a.nin == 1) return a.nout == 1 ? run_zn<L, 1, 1>(a, s) : run_zn<L, 1, 3>(a, s);
+  if (a.nin == 1) {
+    if (outputs_apart<L>(a)) return run_zn<L, 1, 1, true>(a, s);
+    return a.nout == 1 ? run_zn<L, 1, 1>(a, s) : run_zn<L, 1, 3>(a, s);
+  }
   if (a.nin == 2) return run_zn<L, 2, 1>(a, s);
   return a.nout == 1 ? run_zn<L, 3, 1>(a, s) : run_zn<L, 3, 3>(a, s);
 }
