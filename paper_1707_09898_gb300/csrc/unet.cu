@@ -709,6 +709,8 @@ k_conv_halo(const __grid_constant__ CUtensorMap rows, const __grid_constant__ CU
   }
 }
 
+// A tensor map could not be made: nothing was launched. The gather kernels need no maps.
+constexpr int kNoMap = 1;
 int sm_count() {  // of the current device
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -740,7 +742,7 @@ int launch_conv_halo_tz(const void* src, const bf16* Wc, const float* bias, void
   if (tiles <= 0) return 0;
   CUtensorMap rows = {}, wts = {};
   tmk::EncodeTiledFn fn = tmk::encoder();
-  if (!fn) return -4;
+  if (!fn) return kNoMap;
   {  // in units of 8 bytes: channel groups, dx, k half, (dz, dy), chunk
     const cuuint64_t dims[5] = {2ull * NT, 3, 2, 9, (cuuint64_t)nk};
     const cuuint64_t pitch[4] = {32ull * NT * nk, 16ull * NT, 96ull * NT * nk, 32ull * NT};
@@ -748,7 +750,7 @@ int launch_conv_halo_tz(const void* src, const bf16* Wc, const float* bias, void
     if (fn(&wts, CU_TENSOR_MAP_DATA_TYPE_UINT64, 5, const_cast<bf16*>(Wc), dims, pitch, box, step,
            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return -4;
+      return kNoMap;
   }
   if (MODE == 0) {
     const cuuint64_t dims[5] = {(cuuint64_t)KC, W, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)Nb};
@@ -757,7 +759,7 @@ int launch_conv_halo_tz(const void* src, const bf16* Wc, const float* bias, void
     if (fn(&rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(src), dims, pitch, box, step,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return -4;
+      return kNoMap;
   }
   const int windows = NT / NO, gx = sm_count() / windows;  // one block per SM
   k_conv_halo<MODE, W, TZ, NO><<<dim3((unsigned)(tiles < gx ? tiles : gx), windows), HT::THREADS, sm, s>>>(
@@ -792,15 +794,19 @@ int launch_conv_halo(const void* src, const bf16* Wc, const float* bias, void* d
   return launch_conv_halo_tz<MODE, W, 1, NW>(src, Wc, bias, dst, Nb, D, H, KC, NO, flag, s);
 }
 
-// the halo kernel for rows of 8 .. 64 voxels, else the per-voxel gather kernel
+// the halo kernel for rows of 8 .. 64 voxels, else (or without tensor maps) the per-voxel gather
+// kernel; either copies the weights in pieces of 16 bytes
 template <int MODE, int NO>
 int launch_conv(const void* src, const bf16* Wc, const float* bias, void* dst, int Nb, int D, int H, int W, int KC,
                 int flag, cudaStream_t s) {
+  if (reinterpret_cast<uintptr_t>(Wc) & 15) return -4;
   if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-    if (W == 64) return launch_conv_halo<MODE, 64, NO>(src, Wc, bias, dst, Nb, D, H, KC, flag, s);
-    if (W == 32) return launch_conv_halo<MODE, 32, NO>(src, Wc, bias, dst, Nb, D, H, KC, flag, s);
-    if (W == 16) return launch_conv_halo<MODE, 16, NO>(src, Wc, bias, dst, Nb, D, H, KC, flag, s);
-    if (W == 8) return launch_conv_halo<MODE, 8, NO>(src, Wc, bias, dst, Nb, D, H, KC, flag, s);
+    int r = kNoMap;
+    if (W == 64) r = launch_conv_halo<MODE, 64, NO>(src, Wc, bias, dst, Nb, D, H, KC, flag, s);
+    if (W == 32) r = launch_conv_halo<MODE, 32, NO>(src, Wc, bias, dst, Nb, D, H, KC, flag, s);
+    if (W == 16) r = launch_conv_halo<MODE, 16, NO>(src, Wc, bias, dst, Nb, D, H, KC, flag, s);
+    if (W == 8) r = launch_conv_halo<MODE, 8, NO>(src, Wc, bias, dst, Nb, D, H, KC, flag, s);
+    if (r != kNoMap) return r;
   }
   return launch_conv_tc<MODE, NO>(src, Wc, bias, dst, Nb, D, H, W, KC, flag, s);
 }
@@ -1220,7 +1226,7 @@ int launch_dw_rows_of(const bf16* in, const float* dout, float* dW, float* db, f
   if (!fn || fn(&rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16*>(in), dims, pitch, box, step,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return -4;
+    return kNoMap;
   static bool init = false;
   if (!init) {
     if (cudaFuncSetAttribute(k_conv_dw_rows<W, NO, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM) !=
@@ -1676,16 +1682,18 @@ int tmn_conv3d_backward_weight(const void* in, const float* dout, float* dW, flo
   const int nsm = sm_count();
   if ((reinterpret_cast<uintptr_t>(in) & 15) == 0) {
     const bf16* x = reinterpret_cast<const bf16*>(in);
-#define TMN_DW_ROWS(WW)                                                                                    \
-  if (W == WW) {                                                                                           \
-    if (Cout == 16) return launch_dw_rows<WW, 16>(x, dout, dW, db, work, work_floats, N, D, H, Cin, s);     \
-    if (Cout == 32) return launch_dw_rows<WW, 32>(x, dout, dW, db, work, work_floats, N, D, H, Cin, s);     \
-    return launch_dw_rows<WW, 64>(x, dout, dW, db, work, work_floats, N, D, H, Cin, s);                     \
+    int r = kNoMap;
+#define TMN_DW_ROWS(WW)                                                                                      \
+  if (W == WW) {                                                                                             \
+    if (Cout == 16) r = launch_dw_rows<WW, 16>(x, dout, dW, db, work, work_floats, N, D, H, Cin, s);          \
+    else if (Cout == 32) r = launch_dw_rows<WW, 32>(x, dout, dW, db, work, work_floats, N, D, H, Cin, s);     \
+    else r = launch_dw_rows<WW, 64>(x, dout, dW, db, work, work_floats, N, D, H, Cin, s);                     \
   }
     TMN_DW_ROWS(16)
     TMN_DW_ROWS(32)
     TMN_DW_ROWS(64)
 #undef TMN_DW_ROWS
+    if (r != kNoMap) return r;
   }
   if (W == 8 && (reinterpret_cast<uintptr_t>(in) & 15) == 0) {
     // halo tiles: one persistent block per SM, as many as the work buffer holds partials for
