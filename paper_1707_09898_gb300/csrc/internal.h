@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "device.cuh"
+
 namespace tmk {
 
 // Lengths the kernels are instantiated for (even 2^a 3^b, b <= 2).

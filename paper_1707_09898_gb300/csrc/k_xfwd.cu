@@ -344,21 +344,10 @@ __global__ void __launch_bounds__(2 * kNT, 1) k_xfwd_ws(XFwdArgs a) {
 template <int L, bool P3>
 int run_xfwd_ws(const XFwdArgs& a, cudaStream_t s) {
   const size_t sm = xfwd_ws_smem<L>(a.nx);
-  static size_t init = 0;
-  if (init < sm) {
-    if (cudaFuncSetAttribute(k_xfwd_ws<L, P3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-      return -1;
-    init = sm;
-  }
+  if (!allow_smem<k_xfwd_ws<L, P3>>(sm)) return -1;
   const int ntiles = (a.rows + ROWS - 1) / ROWS;
   if (ntiles <= 0) return 0;
-  static int nsm = 0;
-  if (!nsm) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (nsm <= 0) nsm = 148;
-  }
+  const int nsm = sm_count();
   const int blocks = ntiles < nsm ? ntiles : nsm;
   return launch_k(k_xfwd_ws<L, P3>, dim3(blocks), dim3(2 * kNT), sm, s, a.pdl != 0, a) == cudaSuccess ? 0 : -1;
 }
@@ -366,22 +355,10 @@ int run_xfwd_ws(const XFwdArgs& a, cudaStream_t s) {
 template <int L, int SRC, bool P3, bool UPD = false>
 int run_xfwd_src(const XFwdArgs& a, int ncomp, cudaStream_t s) {
   const size_t sm = xsmem<L>() + (UPD ? (size_t)ROWS * (L / 2 + 15) * sizeof(float) : 0);
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_xfwd<L, SRC, P3, UPD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-        cudaSuccess)
-      return -1;
-    init = true;
-  }
+  if (!allow_smem<k_xfwd<L, SRC, P3, UPD>>(sm)) return -1;
   const int tiles = (a.rows + ROWS - 1) / ROWS;
   if (tiles == 0 || ncomp == 0) return 0;
-  static int nsm = 0;
-  if (!nsm) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (nsm <= 0) nsm = 148;
-  }
+  const int nsm = sm_count();
   const int per_comp = (2 * nsm + ncomp - 1) / ncomp;  // two resident blocks per SM in total
   const int blocks = tiles < per_comp ? tiles : per_comp;
   return launch_k(k_xfwd<L, SRC, P3, UPD>, dim3(blocks, ncomp), dim3(kNT), sm, s, a.pdl != 0, a) == cudaSuccess ? 0

@@ -484,21 +484,10 @@ __global__ void __launch_bounds__(2 * kNT, 1) k_xinv_ws(XInvArgs a) {
 template <int L, bool P3>
 int run_xinv_ws(const XInvArgs& a, cudaStream_t s) {
   const size_t sm = xinv_ws_smem<L>(a.P);
-  static size_t init = 0;
-  if (init < sm) {
-    if (cudaFuncSetAttribute(k_xinv_ws<L, P3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-      return -1;
-    init = sm;
-  }
+  if (!allow_smem<k_xinv_ws<L, P3>>(sm)) return -1;
   const int ntiles = (a.rows + ROWS - 1) / ROWS;
   if (ntiles <= 0) return 0;
-  static int nsm = 0;
-  if (!nsm) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (nsm <= 0) nsm = 148;
-  }
+  const int nsm = sm_count();
   const int blocks = ntiles < nsm ? ntiles : nsm;
   return launch_k(k_xinv_ws<L, P3>, dim3(blocks), dim3(2 * kNT), sm, s, a.pdl != 0, a) == cudaSuccess ? 0 : -1;
 }
@@ -506,13 +495,7 @@ int run_xinv_ws(const XInvArgs& a, cudaStream_t s) {
 template <int L, int SINK, int MINB, bool P3, bool ONE = false>
 int run_xinv_sink(const XInvArgs& a, cudaStream_t s) {
   const size_t sm = xsmem<L>();
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_xinv<L, SINK, MINB, P3, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-        cudaSuccess)
-      return -1;
-    init = true;
-  }
+  if (!allow_smem<k_xinv<L, SINK, MINB, P3, ONE>>(sm)) return -1;
   const int blocks = (a.rows - a.row_base + ROWS - 1) / ROWS;
   if (blocks <= 0 || a.ncomp == 0) return 0;
   const int gy = SINK == SINK_CHAIN ? 1 : a.ncomp;

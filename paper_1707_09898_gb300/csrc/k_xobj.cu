@@ -414,12 +414,7 @@ static int run_xobj(const XInvArgs& a, int rows, cudaStream_t s) {
 int launch_xobj(int L, const XInvArgs& a, cudaStream_t s) {
   if (L == 512) {
     constexpr size_t sm8 = (size_t)(512 + NG8 * 2 * 512) * sizeof(float2);
-    static bool init8 = false;
-    if (!init8) {
-      if (cudaFuncSetAttribute(k_xobj512, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm8) != cudaSuccess)
-        return -1;
-      init8 = true;
-    }
+    if (!allow_smem<k_xobj512>(sm8)) return -1;
     const int rows = a.rows - a.row_base;
     const int blocks = (rows + 2 * NG8 - 1) / (2 * NG8);
     if (blocks <= 0 || a.ncomp == 0) return 0;

@@ -404,12 +404,7 @@ size_t tile_smem() {
 template <int L, bool INV>
 int run_y(const YArgs& a, int ncomp, cudaStream_t s) {
   const size_t sm = tile_smem<L>();
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_ypass<L, INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-      return -1;
-    init = true;
-  }
+  if (!allow_smem<k_ypass<L, INV>>(sm)) return -1;
   if (a.nplanes == 0 || ncomp == 0) return 0;
   dim3 grid(a.P / TB, a.nplanes, ncomp);
   return launch_k(k_ypass<L, INV>, grid, dim3(kNT), sm, s, a.pdl != 0, a) == cudaSuccess ? 0 : -1;
@@ -425,12 +420,8 @@ int run_z(const ZArgs& a, cudaStream_t s) {
       // EXT: the input or output planes come from the device range a.ext, and a few of them
       // take the direct transforms
       const bool ext = a.in_ext || a.out_ext;
+      if (!(ext ? allow_smem<k_z1m<L, true>>(sm) : allow_smem<k_z1m<L, false>>(sm))) return -1;
       auto kern = ext ? k_z1m<L, true> : k_z1m<L, false>;
-      static bool initm[2] = {false, false};
-      if (!initm[ext]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) return -1;
-        initm[ext] = true;
-      }
       kern<<<dim3(a.P / TB, a.Ly), kNT, sm, s>>>(a);
       return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
     }

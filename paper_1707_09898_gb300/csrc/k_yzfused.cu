@@ -742,11 +742,7 @@ int single_component(const int need) { return (need != 0 && (need & (need - 1)) 
 template <int L>
 int launch_adj(const ZYArgs& a, int c, cudaStream_t s) {
   const size_t sm = fused_smem<L>();
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_zy_adj<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) return -1;
-    init = true;
-  }
+  if (!allow_smem<k_zy_adj<L>>(sm)) return -1;
   return launch_k(k_zy_adj<L>, dim3(a.P / TB, a.nzout), dim3(kNT), sm, s, a.pdl != 0, a, c) ==
                  cudaSuccess
              ? (a.zero_word ? 1 : 0)  // 1: *zero_word is cleared
@@ -797,27 +793,10 @@ bool slice_map(CUtensorMap* m, const float* Ts, long long rows, int P, int box_r
   return true;
 }
 
-int sm_count() {
-  static int nsm = 0;
-  if (!nsm) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (nsm <= 0) nsm = 148;
-  }
-  return nsm;
-}
-
 template <int L, int C, bool FULL>
 int launch_adj_ws(const ZYArgs& a, const CUtensorMap& mslice, cudaStream_t s) {
   constexpr size_t sm = ws_smem<L>();
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_zy_adj_ws<L, C, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-        cudaSuccess)
-      return -1;
-    init = true;
-  }
+  if (!allow_smem<k_zy_adj_ws<L, C, FULL>>(sm)) return -1;
   const long long items = (long long)(a.P / TB) * a.nzout;
   const int blocks = (int)(items < sm_count() ? items : sm_count());  // one resident block per SM
   return launch_k(k_zy_adj_ws<L, C, FULL>, dim3(blocks), dim3(NTF), sm, s, a.pdl != 0, a, mslice) == cudaSuccess
@@ -864,13 +843,7 @@ size_t staged_smem() {
 template <int L>
 int launch_fwd_staged(const YZArgs& a, int c, int nch, cudaStream_t s) {
   const size_t sm = staged_smem<L>();
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_yz_fwd_staged<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-        cudaSuccess)
-      return -1;
-    init = true;
-  }
+  if (!allow_smem<k_yz_fwd_staged<L>>(sm)) return -1;
   return launch_k(k_yz_fwd_staged<L>, dim3(a.P / TB, nch), dim3(NTF), sm, s, a.pdl != 0, a, c) == cudaSuccess
              ? 2  // 2: partials of the z chunks written; launch_yz_finish completes the target plane
              : -1;
@@ -879,13 +852,7 @@ int launch_fwd_staged(const YZArgs& a, int c, int nch, cudaStream_t s) {
 template <int L, int C, bool FULL>
 int launch_fwd_ws(const YZArgs& a, const CUtensorMap& mslice, cudaStream_t s) {
   constexpr size_t sm = ws_smem<L>();
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_yz_fwd_ws<L, C, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-        cudaSuccess)
-      return -1;
-    init = true;
-  }
+  if (!allow_smem<k_yz_fwd_ws<L, C, FULL>>(sm)) return -1;
   const long long items = (long long)(a.P / TB) * a.nzin;
   const int blocks = (int)(items < sm_count() ? items : sm_count());  // one resident block per SM
   return launch_k(k_yz_fwd_ws<L, C, FULL>, dim3(blocks), dim3(NTF), sm, s, a.pdl != 0, a, mslice) == cudaSuccess
@@ -941,13 +908,7 @@ template <int L>
 int run_yz_finish(const YZArgs& a, int how, cudaStream_t s) {
   if (how == 2) {
     const size_t sm = fused_smem<L>();
-    static bool init = false;
-    if (!init) {
-      if (cudaFuncSetAttribute(k_yz_finish_chunks<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-          cudaSuccess)
-        return -1;
-      init = true;
-    }
+    if (!allow_smem<k_yz_finish_chunks<L>>(sm)) return -1;
     return launch_k(k_yz_finish_chunks<L>, dim3(a.P / TB), dim3(kNT), sm, s, a.pdl != 0, a,
                     (a.nzin + a.zchunk - 1) / a.zchunk) == cudaSuccess
                ? 0

@@ -366,13 +366,7 @@ int run_zn(const ZArgs& a, cudaStream_t s) {
   using Z = ZPlan<L>;
   const int tiles = APART ? 1 : a.nin > a.nout ? a.nin : a.nout;
   const size_t sm = (size_t)(ztw_size<L>() + tiles * L * TB) * sizeof(float2);
-  static bool init = false;
-  if (!init) {
-    const size_t most = (size_t)(ztw_size<L>() + (NI > NO ? NI : NO) * L * TB) * sizeof(float2);
-    if (cudaFuncSetAttribute(k_zn<L, NI, NO, APART>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess)
-      return -1;
-    init = true;
-  }
+  if (!allow_smem<k_zn<L, NI, NO, APART>>(sm)) return -1;
   k_zn<L, NI, NO, APART><<<dim3(a.P / TB, a.Ly, APART ? a.nout : 1), Z::NT, sm, s>>>(a);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }

@@ -20,9 +20,12 @@
 #include <type_traits>
 
 #include "../../include/topomag_net.h"
+#include "device.cuh"
 #include "unet_tc.cuh"
 
 namespace {
+
+using tmk::sm_count;
 
 using bf16 = __nv_bfloat16;
 
@@ -247,12 +250,7 @@ template <int MODE, int NO>
 int launch_conv_tc(const void* src, const bf16* Wc, const float* bias, void* dst, int Nb, int D, int H, int W, int KC,
                    int flag, cudaStream_t s) {
   constexpr size_t sm = conv_tc_smem<NO>();
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_conv_tc<MODE, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-      return -4;
-    init = true;
-  }
+  if (!tmk::allow_smem<k_conv_tc<MODE, NO>>(sm)) return -4;
   const long long nvox = (long long)Nb * D * H * W;
   const int blocks = (int)((nvox + 127) / 128);
   if (blocks > 0) k_conv_tc<MODE, NO><<<blocks, 128, sm, s>>>(src, Wc, bias, dst, Nb, D, H, W, KC, flag);
@@ -711,13 +709,6 @@ k_conv_halo(const __grid_constant__ CUtensorMap rows, const __grid_constant__ CU
 
 // A tensor map could not be made: nothing was launched. The gather kernels need no maps.
 constexpr int kNoMap = 1;
-int sm_count() {  // of the current device
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return 148;
-  return n > 0 ? n : 148;
-}
-
 template <int MODE, int W, int TZ, int NO>
 int launch_conv_halo_tz(const void* src, const bf16* Wc, const float* bias, void* dst, int Nb, int D, int H, int KC,
                         int NT, int flag, cudaStream_t s) {
@@ -730,13 +721,7 @@ int launch_conv_halo_tz(const void* src, const bf16* Wc, const float* bias, void
   while (ns > 2 && halo_smem<MODE, W, TZ, NO>(ns, resident, nk) > kMost) ns--;
   const size_t sm = halo_smem<MODE, W, TZ, NO>(ns, resident, nk);
   static_assert(halo_smem<MODE, W, TZ, NO>(2, false, 1) <= kMost, "shared memory of one block");
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_conv_halo<MODE, W, TZ, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost) !=
-        cudaSuccess)
-      return -4;
-    init = true;
-  }
+  if (!tmk::allow_smem<k_conv_halo<MODE, W, TZ, NO>>(kMost)) return -4;
   const long long tiles = (long long)Nb * ((D + TZ - 1) / TZ) * ((H + HT::RY - 1) / HT::RY);
   if (tiles > 0x7fffffffLL) return -1;
   if (tiles <= 0) return 0;
@@ -1227,13 +1212,7 @@ int launch_dw_rows_of(const bf16* in, const float* dout, float* dW, float* db, f
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return kNoMap;
-  static bool init = false;
-  if (!init) {
-    if (cudaFuncSetAttribute(k_conv_dw_rows<W, NO, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM) !=
-        cudaSuccess)
-      return -4;
-    init = true;
-  }
+  if (!tmk::allow_smem<k_conv_dw_rows<W, NO, RMAX>>(T::SMEM)) return -4;
   k_conv_dw_rows<W, NO, RMAX><<<dim3((unsigned)nblk, groups), T::THREADS, T::SMEM, s>>>(rows, dout, work, Nb, D, H, Cin);
   k_dw_finish<<<(unsigned)((n + NO + 31) / 32), 256, 0, s>>>(work, (int)nblk, n, NO, dW, db);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
