@@ -322,14 +322,21 @@ struct ConvSpec {
   int in_ext, out_ext;
 };
 
-// one input, one output and one tensor component between them
-bool single_product(const ConvSpec& cs) {
-  if (cs.nin != 1 || cs.nout != 1) return false;
+// one input, one output and one tensor component between them: the component (and its coefficient),
+// else -1
+int single_product(const ConvSpec& cs, float* coef = nullptr) {
+  if (cs.nin != 1 || cs.nout != 1) return -1;
   float c6[6];
   coef6(c6, cs.v[0], cs.u[0]);
-  int n = 0;
-  for (int c = 0; c < 6; c++) n += c6[c] != 0.0f;
-  return n == 1;
+  int n = 0, one = -1;
+  for (int c = 0; c < 6; c++)
+    if (c6[c] != 0.0f) {
+      n++;
+      one = c;
+    }
+  if (n != 1) return -1;
+  if (coef) *coef = c6[one];
+  return one;
 }
 
 // float copies of the vectors; returns the mask of the tensor components they use
@@ -512,8 +519,6 @@ int scaled_component(tm_ctx* ctx, int which, int c, float coef, cudaStream_t s, 
   return TM_OK;
 }
 
-int one_component(int need) { return (need != 0 && (need & (need - 1)) == 0) ? __builtin_ctz(need) : -1; }
-
 // forward y transform of the design planes fused with the direct z sum onto the single target
 // plane (one spectrum, one tensor component), and the target plane's inverse y transform into A
 int yz_forward(tm_ctx* ctx, const ConvSpec& cs, int zo, cudaStream_t s) {
@@ -524,28 +529,14 @@ int yz_forward(tm_ctx* ctx, const ConvSpec& cs, int zo, cudaStream_t s) {
   nch = nch < 1 ? 1 : (nch > ctx->nzd ? ctx->nzd : nch);
   const int zchunk = (ctx->nzd + nch - 1) / nch;
   nch = (ctx->nzd + zchunk - 1) / zchunk;
-  if (nch > ctx->yzpart_chunks) {
-    cudaFree(ctx->yzpart);
-    ctx->yzpart = nullptr;
-    ctx->yzpart_chunks = 0;
-    CK(cudaMalloc(&ctx->yzpart, (size_t)nch * Ly * P * sizeof(float2)));
-    ctx->yzpart_chunks = nch;
-  }
   YZArgs y{};
   y.in = ctx->A;
   y.in_cstride = (long long)ctx->nz * ctx->ny * P;
   y.in_zstride = (long long)ctx->ny * P;
-  y.part = ctx->yzpart;
   y.P = ctx->P;
   y.n_in = ctx->ny;
-  y.nin = cs.nin;
-  for (int i = 0; i < cs.nin; i++) {
-    y.in_slot[i] = cs.ain[i];
-    coef6(y.coef[i], cs.v[0], cs.u[i]);
-    y.need[i] = 0;
-    for (int c = 0; c < 6; c++)
-      if (y.coef[i][c] != 0.0f) y.need[i] |= 1 << c;
-  }
+  y.in_slot = cs.ain[0];
+  y.c = single_product(cs, &y.coef);
   y.Tz = ctx->Tz;
   y.Tdz = (long long)(Ly / 2 + 1) * P;
   y.Tc = (long long)ctx->nz * y.Tdz;
@@ -554,22 +545,30 @@ int yz_forward(tm_ctx* ctx, const ConvSpec& cs, int zo, cudaStream_t s) {
   y.zchunk = zchunk;
   y.zout = zo;
   y.tw = ctx->tw + ctx->L[0];
-  if (!ctx->yzseg) CK(cudaMalloc(&ctx->yzseg, (size_t)2 * ctx->nsm * Ly * TB * sizeof(float2)));
-  y.seg = ctx->yzseg;
-  {
-    const int c1 = one_component(y.need[0]);
-    int r;
+  int r;
+  if (yz_ws_length(Ly)) {
+    if (!ctx->yzseg) CK(cudaMalloc(&ctx->yzseg, (size_t)2 * ctx->nsm * Ly * TB * sizeof(float2)));
+    y.seg = ctx->yzseg;
     bool rebuilt;
-    if ((r = scaled_component(ctx, 0, c1, y.coef[0][c1], s, &y.Ts, &rebuilt))) return r;
+    if ((r = scaled_component(ctx, 0, y.c, y.coef, s, &y.Ts, &rebuilt))) return r;
     y.nz_total = ctx->nz;
   }
   y.status = ctx->dstat;
   y.yrows = ctx->A + cs.aout[0] * ((long long)ctx->nz * ctx->ny * P) + (long long)zo * ctx->ny * P;
   y.pdl = ctx->pdl;
-  int r;
+  y.part = nch <= ctx->yzpart_chunks ? ctx->yzpart : nullptr;
   {
     Timed t(ctx, KIND_YZF, s);
     r = launch_yz_fwd(Ly, y, s);
+    if (r == 3) {  // partials of z chunks
+      cudaFree(ctx->yzpart);
+      ctx->yzpart = nullptr;
+      ctx->yzpart_chunks = 0;
+      CK(cudaMalloc(&ctx->yzpart, (size_t)nch * Ly * P * sizeof(float2)));
+      ctx->yzpart_chunks = nch;
+      y.part = ctx->yzpart;
+      r = launch_yz_fwd(Ly, y, s);
+    }
     if (r < 0) CKL(r);
   }
   // the target plane: partial sums added, inverse y transform
@@ -592,34 +591,23 @@ int zy_adjoint(tm_ctx* ctx, const ConvSpec& cs, int zi0, cudaStream_t s, bool yf
   z.out_zstride = (long long)ctx->ny * P;
   z.P = ctx->P;
   z.n_out = ctx->ny;
-  z.nin = cs.nin;
-  z.nout = cs.nout;
-  for (int i = 0; i < cs.nin; i++) z.in_slot[i] = cs.bin[i];
-  for (int o = 0; o < cs.nout; o++) {
-    z.out_slot[o] = cs.aout[o];
-    for (int i = 0; i < cs.nin; i++) {
-      coef6(z.coef[o][i], cs.v[o], cs.u[i]);
-      z.need[o][i] = 0;
-      for (int c = 0; c < 6; c++)
-        if (z.coef[o][i][c] != 0.0f) z.need[o][i] |= 1 << c;
-    }
-  }
+  z.in_slot = cs.bin[0];
+  z.out_slot = cs.aout[0];
+  z.c = single_product(cs, &z.coef);
   z.Tz = ctx->Tz;
   z.Tdz = (long long)(Ly / 2 + 1) * P;
   z.Tc = (long long)ctx->nz * z.Tdz;
   z.zin0 = zi0;
-  z.nzin = 1;
   z.zout0 = 0;
   z.nzout = ctx->nzd;
   z.tw = ctx->tw + ctx->L[0];
   z.status = ctx->dstat;
   z.zero_word = ctx->gmax;  // cleared for the chain-rule pass that follows (saves a memset between kernels)
   z.pdl = ctx->pdl;
-  const int c1 = cs.nin == 1 && cs.nout == 1 ? one_component(z.need[0][0]) : -1;
-  if (c1 >= 0) {
+  if (yz_ws_length(Ly)) {
     int r;
     bool rebuilt;
-    if ((r = scaled_component(ctx, 1, c1, z.coef[0][0][c1], s, &z.Ts, &rebuilt))) return r;
+    if ((r = scaled_component(ctx, 1, z.c, z.coef, s, &z.Ts, &rebuilt))) return r;
     z.nzin_total = ctx->nz;
     // the adjoint reads its first tensor slice before it waits for the preceding kernel:
     // after a rebuild it must start only once the scaling kernel has finished
@@ -1142,7 +1130,7 @@ int forward_planes(tm_ctx* ctx, const float* rho, const int* F, int nF, cudaStre
     cs.aout[o] = o;
     cs.v[o] = kUnit[F[o]];
   }
-  if (ctx->fuse_yz && np == 1 && single_product(cs)) return yz_forward(ctx, cs, ctx->tz0, s);
+  if (ctx->fuse_yz && np == 1 && single_product(cs) >= 0) return yz_forward(ctx, cs, ctx->tz0, s);
   if ((r = ypass(ctx, false, cs.nin, cs.ain, cs.bin, 0, ctx->nzd, s))) return r;
   if ((r = zdirect(ctx, cs, 0, ctx->nzd, ctx->tz0, np, s))) return r;
   return ypass(ctx, true, cs.nout, cs.aout, cs.bout, ctx->tz0, np, s);
@@ -1178,11 +1166,11 @@ int adjoint_planes(tm_ctx* ctx, const float* rho, float* dJdrho, const int* F, c
   }
   // fused only in its single-spectrum, single-component form; with several spectra or
   // tensor components the separate passes measured faster
-  const bool fused = ctx->fuse_yz && np == 1 && single_product(ca);
+  const bool fused = ctx->fuse_yz && np == 1 && single_product(ca) >= 0;
   // on the warp-specialized path the fused adjoint runs the source's y transform itself;
   // it then reads the source rows from A while it writes the design planes into A, so its
   // output goes to another slot (the target plane may be a design plane)
-  const bool yfwd_inside = fused && zy_adj_ws_length(ctx->L[1]) && ctx->ny <= ctx->L[1] / 2;
+  const bool yfwd_inside = fused && yz_ws_length(ctx->L[1]) && ctx->ny <= ctx->L[1] / 2;
   if (yfwd_inside) ca.aout[0] = (ca.ain[0] + 1) % kSlotsA;
   if (!yfwd_inside && (r = ypass(ctx, false, ca.nin, ca.ain, ca.bin, ctx->tz0, np, s))) return r;
   if (fused) {

@@ -180,14 +180,14 @@ struct ZYArgs {
   float2* out;                              // A [slot][z][ny][P]
   long long out_cstride, out_zstride;
   int P, n_out;                             // kx columns (multiple of TB); valid y rows
-  int nin, nout, in_slot[3], out_slot[3];
-  float coef[3][3][6];
-  int need[3][3];
+  int in_slot, out_slot;
+  int c;                                    // the tensor component, and its coefficient
+  float coef;
   const float* Tz;                          // [6][nz][Ly/2+1][P]
   long long Tc, Tdz;
-  int zin0, nzin, zout0, nzout;
+  int zin0, zout0, nzout;                   // the source plane; output planes
   const float2* tw;                         // W_Ly
-  // warp-specialized path (one tensor component c): Ts = coef[0][0][c] * Tz[c], [nzin_total][Ly/2+1][P]
+  // warp-specialized path: Ts = coef * Tz[c], [nzin_total][Ly/2+1][P]
   const float* Ts;
   int nzin_total;                           // z offsets held by Ts
   // if set (warp-specialized path only): the source plane as x spectra, rows [n_src][P]; the
@@ -198,38 +198,38 @@ struct ZYArgs {
   unsigned* zero_word;                      // if set, zeroed by the kernel (launch_zy_adj returns 1)
   int pdl;                                  // launch with programmatic dependent launch
 };
-// Forward: the design planes of A onto one plane and one output of B.
+// Forward: the design planes of A onto the rows of one plane of A (one spectrum, one tensor
+// component).
 struct YZArgs {
   const float2* in;                         // A [slot][z][ny][P]
   long long in_cstride, in_zstride;
-  float2* part;                             // [z chunks][Ly][P]
+  float2* part;                             // [z chunks][Ly][P] (null: launch_yz_fwd may ask for it)
   int P, n_in;
-  int nin, in_slot[3];                      // one input
-  float coef[3][6];                         // s_i = v^T N u_i of the single output
-  int need[3];
+  int in_slot;
+  int c;                                    // the tensor component, and its coefficient
+  float coef;
   const float* Tz;
   long long Tc, Tdz;
   int zin0, nzin, zchunk, zout;
   const float2* tw;
-  // single-component path on two-stage plans (when set): per-block segment partials
-  // [2 * blocks][Ly][TB], the target plane's rows in A [ny][P], and the tensor component
-  // scaled by its coefficient, Ts = coef[0][c] * Tz[c] [nz_total][Ly/2+1][P]; launch_yz_fwd
-  // then also writes the inverse y transform of the target plane there and returns 1
+  float2* yrows;                            // the target plane's rows in A [ny][P], by launch_yz_finish
+  // warp-specialized path (when set): per-block segment partials [2 * blocks][Ly][TB], and the
+  // tensor component scaled by its coefficient, Ts = coef * Tz[c] [nz_total][Ly/2+1][P]
   float2* seg;
-  float2* yrows;
   const float* Ts;
   int nz_total;
   unsigned* status;                         // device word: bit 0 set when a copy wait timed out
   int pdl;                                  // launch with programmatic dependent launch
 };
 int launch_zy_adj(int L, const ZYArgs& a, cudaStream_t s);
-// whether launch_zy_adj takes the warp-specialized path for length L (Ts given), the path that can
-// run the source's y transform
-bool zy_adj_ws_length(int L);
+// whether the fused kernels have a warp-specialized path for length L, which reads Ts (and seg);
+// the adjoint's can run the source's y transform
+bool yz_ws_length(int L);
+// 1: segment partials written (warp-specialized); 2: partials of z chunks written; 3: nothing
+// launched, a.part is needed
 int launch_yz_fwd(int L, const YZArgs& a, cudaStream_t s);
-// after launch_yz_fwd returned how = 1 (segment partials of the warp-specialized kernel) or 2
-// (partials of z chunks): the partials added in order, and the target plane's inverse y
-// transform into a.yrows
+// after launch_yz_fwd returned how = 1 or 2: the partials added in order, and the target plane's
+// inverse y transform into a.yrows
 int launch_yz_finish(int L, const YZArgs& a, int how, cudaStream_t s);
 
 int launch_xfwd(int L, const XFwdArgs& a, int ncomp, cudaStream_t s);

@@ -33,8 +33,9 @@ namespace {
 // less) and several planes per block a 64^2 x 72 step took 64.9 us instead of 63.3, sixteen
 // concurrent optimizations 1640 us instead of 1521, a 128^3 step 72.8 instead of 73.2.
 template <int L>
-__global__ void __launch_bounds__(kNT, 2) k_zy_adj(ZYArgs a, int c) {
+__global__ void __launch_bounds__(kNT, 2) k_zy_adj(ZYArgs a) {
   constexpr int S = plan_stages(L);
+  const int c = a.c;
   extern __shared__ __align__(16) unsigned char smem[];
   cx<float>* tw = reinterpret_cast<cx<float>*>(smem);
   cx<float>* tile = tw + L;
@@ -42,7 +43,7 @@ __global__ void __launch_bounds__(kNT, 2) k_zy_adj(ZYArgs a, int c) {
   const int kx0 = blockIdx.x * TB;
   const int z = a.zout0 + blockIdx.y;
   const cx<float>* src = reinterpret_cast<const cx<float>*>(a.src);
-  cx<float>* out = reinterpret_cast<cx<float>*>(a.out) + a.out_slot[0] * a.out_cstride + z * a.out_zstride + kx0;
+  cx<float>* out = reinterpret_cast<cx<float>*>(a.out) + a.out_slot * a.out_cstride + z * a.out_zstride + kx0;
   pdl_wait();  // the source plane and the outputs belong to earlier kernels
   if (a.zero_word && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *a.zero_word = 0u;
   __syncthreads();
@@ -55,9 +56,9 @@ __global__ void __launch_bounds__(kNT, 2) k_zy_adj(ZYArgs a, int c) {
     constexpr int R = SS::R, ITER = (SS::NU + kNT - 1) / kNT;
     const int dz = z - a.zin0;
     const int adz = dz < 0 ? -dz : dz;
-    const float cz = (c >= 4 && dz < 0) ? -a.coef[0][0][c] : a.coef[0][0][c];
+    const float cz = (c >= 4 && dz < 0) ? -a.coef : a.coef;
     const float* tcol = a.Tz + c * a.Tc + adz * a.Tdz + kx0;
-    const cx<float>* srow = src + a.in_slot[0] * a.src_cstride + a.zin0 * a.src_zstride + kx0;
+    const cx<float>* srow = src + a.in_slot * a.src_cstride + a.zin0 * a.src_zstride + kx0;
     cx<float> v[ITER][R];
 #pragma unroll
     for (int it = 0; it < ITER; it++) {
@@ -111,11 +112,12 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 
 
 template <int L>
-__global__ void __launch_bounds__(NTF, 1) k_yz_fwd_staged(YZArgs a, int c) {
+__global__ void __launch_bounds__(NTF, 1) k_yz_fwd_staged(YZArgs a) {
   constexpr int S = plan_stages(L);
   using SL = StageShape<L, S - 1>;
   constexpr int R = SL::R, ITER = (SL::NU + NTF - 1) / NTF;
   constexpr int KY = L / 2 + 1;
+  const int c = a.c;
   extern __shared__ __align__(16) unsigned char smem[];
   cx<float>* tw = reinterpret_cast<cx<float>*>(smem);
   cx<float>* tile = tw + L;
@@ -126,7 +128,7 @@ __global__ void __launch_bounds__(NTF, 1) k_yz_fwd_staged(YZArgs a, int c) {
   const int kx0 = blockIdx.x * TB;
   const int zb0 = a.zin0 + blockIdx.y * a.zchunk;
   const int zb1 = min(zb0 + a.zchunk, a.zin0 + a.nzin);
-  const cx<float>* in0 = reinterpret_cast<const cx<float>*>(a.in) + a.in_slot[0] * a.in_cstride + kx0;
+  const cx<float>* in0 = reinterpret_cast<const cx<float>*>(a.in) + a.in_slot * a.in_cstride + kx0;
   const float* tc = a.Tz + c * a.Tc + kx0;
   auto issue = [&](int z, int buf) {  // 16-byte copies: 8 per input row, 4 per tensor row
     const cx<float>* src = in0 + z * a.in_zstride;
@@ -168,7 +170,7 @@ __global__ void __launch_bounds__(NTF, 1) k_yz_fwd_staged(YZArgs a, int c) {
     __syncthreads();
     DifRange<float, L, NTF, 1, S - 1>::run(tile, tw);
     const int dz = a.zout - z;
-    const float cz = (c >= 4 && dz < 0) ? -a.coef[0][c] : a.coef[0][c];
+    const float cz = (c >= 4 && dz < 0) ? -a.coef : a.coef;
 #pragma unroll
     for (int it = 0; it < ITER; it++) {
       const int u = it * NTF + threadIdx.x;
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(NTF, 1) k_yz_fwd_ws(YZArgs a, const __grid_con
     const int t = threadIdx.x;
     const int line = t % TB, j = t / TB;
     const cx<float>* in0 =
-        reinterpret_cast<const cx<float>*>(a.in) + a.in_slot[0] * a.in_cstride + (long long)j * a.P + line;
+        reinterpret_cast<const cx<float>*>(a.in) + a.in_slot * a.in_cstride + (long long)j * a.P + line;
     cx<float> pre[R0 / 2];  // rows j + q M0 (q < R0/2; n_in <= L/2) of the next item
     auto fetch = [&](Item it) {
       const cx<float>* src = in0 + it.z * a.in_zstride + it.cb * TB;
@@ -622,7 +624,7 @@ __global__ void __launch_bounds__(NTF, 1) k_zy_adj_ws(ZYArgs a, const __grid_con
   if (threadIdx.x < kNT) {
     // load warps: s times the source, first inverse stage, into tile r % 2 in round r
     const int t = threadIdx.x;
-    const cx<float>* src = reinterpret_cast<const cx<float>*>(a.src) + a.in_slot[0] * a.src_cstride +
+    const cx<float>* src = reinterpret_cast<const cx<float>*>(a.src) + a.in_slot * a.src_cstride +
                            a.zin0 * a.src_zstride;
     // the source spectrum does not depend on the design plane: a thread keeps its 2 R1
     // values (positions g R1 + q of its two units) for as long as the column block stays
@@ -696,7 +698,7 @@ __global__ void __launch_bounds__(NTF, 1) k_zy_adj_ws(ZYArgs a, const __grid_con
     // store warps: last inverse stage of the item of round r - 1, rows y < n_out out
     const int t = threadIdx.x - kNT;
     const int line = t % TB, j = t / TB;
-    cx<float>* out0 = reinterpret_cast<cx<float>*>(a.out) + a.out_slot[0] * a.out_cstride;
+    cx<float>* out0 = reinterpret_cast<cx<float>*>(a.out) + a.out_slot * a.out_cstride;
     Item cur = first;                                   // the item of round r - 1
     Item ahead = next_item(first, a.zout0, a.nzout);    // the item whose slice is issued in round r
     for (int r = 0; r <= n; r++) {
@@ -736,14 +738,11 @@ size_t fused_smem() {
   return (size_t)(L + L * TB) * sizeof(float2);
 }
 
-// the single tensor component of (o, i) = (0, 0), or -1
-int single_component(const int need) { return (need != 0 && (need & (need - 1)) == 0) ? __builtin_ctz(need) : -1; }
-
 template <int L>
-int launch_adj(const ZYArgs& a, int c, cudaStream_t s) {
+int launch_adj(const ZYArgs& a, cudaStream_t s) {
   const size_t sm = fused_smem<L>();
   if (!allow_smem<k_zy_adj<L>>(sm)) return -1;
-  return launch_k(k_zy_adj<L>, dim3(a.P / TB, a.nzout), dim3(kNT), sm, s, a.pdl != 0, a, c) ==
+  return launch_k(k_zy_adj<L>, dim3(a.P / TB, a.nzout), dim3(kNT), sm, s, a.pdl != 0, a) ==
                  cudaSuccess
              ? (a.zero_word ? 1 : 0)  // 1: *zero_word is cleared
              : -1;
@@ -804,8 +803,8 @@ int launch_adj_ws(const ZYArgs& a, const CUtensorMap& mslice, cudaStream_t s) {
              : -1;
 }
 template <int L, bool FULL>
-int launch_adj_ws_c(const ZYArgs& a, int c, const CUtensorMap& ms, cudaStream_t s) {
-  switch (c) {
+int launch_adj_ws_c(const ZYArgs& a, const CUtensorMap& ms, cudaStream_t s) {
+  switch (a.c) {
     case 0: return launch_adj_ws<L, 0, FULL>(a, ms, s);
     case 1: return launch_adj_ws<L, 1, FULL>(a, ms, s);
     case 2: return launch_adj_ws<L, 2, FULL>(a, ms, s);
@@ -818,21 +817,14 @@ int launch_adj_ws_c(const ZYArgs& a, int c, const CUtensorMap& ms, cudaStream_t 
 template <int L>
 int run_zy_adj(const ZYArgs& a, cudaStream_t s) {
   if (a.nzout <= 0) return 0;
-  const int c = single_component(a.need[0][0]);
-  if (a.nin != 1 || a.nout != 1 || a.nzin != 1 || c < 0) return -1;
   if constexpr (yz_ws_plan<L>()) {
     CUtensorMap ms;
     if (a.Ts && a.nzin_total > 0 && a.n_src <= L / 2 &&
         slice_map(&ms, a.Ts, (long long)a.nzin_total * (L / 2 + 1), a.P, slice_box_rows<L>()))
-      return a.n_out == L / 2 ? launch_adj_ws_c<L, true>(a, c, ms, s) : launch_adj_ws_c<L, false>(a, c, ms, s);
+      return a.n_out == L / 2 ? launch_adj_ws_c<L, true>(a, ms, s) : launch_adj_ws_c<L, false>(a, ms, s);
   }
   if (a.gsrc) return -1;  // the source's y transform is only done on the warp-specialized path
-  return launch_adj<L>(a, c, s);
-}
-
-template <int L>
-constexpr bool ws_length() {
-  return yz_ws_plan<L>();
+  return launch_adj<L>(a, s);
 }
 
 template <int L>
@@ -841,10 +833,11 @@ size_t staged_smem() {
 }
 
 template <int L>
-int launch_fwd_staged(const YZArgs& a, int c, int nch, cudaStream_t s) {
+int launch_fwd_staged(const YZArgs& a, int nch, cudaStream_t s) {
+  if (!a.part) return 3;
   const size_t sm = staged_smem<L>();
   if (!allow_smem<k_yz_fwd_staged<L>>(sm)) return -1;
-  return launch_k(k_yz_fwd_staged<L>, dim3(a.P / TB, nch), dim3(NTF), sm, s, a.pdl != 0, a, c) == cudaSuccess
+  return launch_k(k_yz_fwd_staged<L>, dim3(a.P / TB, nch), dim3(NTF), sm, s, a.pdl != 0, a) == cudaSuccess
              ? 2  // 2: partials of the z chunks written; launch_yz_finish completes the target plane
              : -1;
 }
@@ -860,8 +853,8 @@ int launch_fwd_ws(const YZArgs& a, const CUtensorMap& mslice, cudaStream_t s) {
              : -1;
 }
 template <int L, bool FULL>
-int launch_fwd_ws_c(const YZArgs& a, int c, const CUtensorMap& ms, cudaStream_t s) {
-  switch (c) {
+int launch_fwd_ws_c(const YZArgs& a, const CUtensorMap& ms, cudaStream_t s) {
+  switch (a.c) {
     case 0: return launch_fwd_ws<L, 0, FULL>(a, ms, s);
     case 1: return launch_fwd_ws<L, 1, FULL>(a, ms, s);
     case 2: return launch_fwd_ws<L, 2, FULL>(a, ms, s);
@@ -872,23 +865,21 @@ int launch_fwd_ws_c(const YZArgs& a, int c, const CUtensorMap& ms, cudaStream_t 
 }
 
 template <int L>
-int launch_fwd_single(const YZArgs& a, int c, int nch, cudaStream_t s) {
+int launch_fwd(const YZArgs& a, int nch, cudaStream_t s) {
   if constexpr (yz_ws_plan<L>()) {
     // needs the segment buffers, the scaled tensor component, and at most two column
     // blocks per block (blocks >= P / TB)
     CUtensorMap ms;
     if (a.n_in <= L / 2 && a.seg && a.yrows && a.Ts && a.P / TB <= sm_count() && sm_count() <= kFinishMaxBlocks &&
         slice_map(&ms, a.Ts, (long long)a.nz_total * (L / 2 + 1), a.P, slice_box_rows<L>()))
-      return a.n_in == L / 2 ? launch_fwd_ws_c<L, true>(a, c, ms, s) : launch_fwd_ws_c<L, false>(a, c, ms, s);
+      return a.n_in == L / 2 ? launch_fwd_ws_c<L, true>(a, ms, s) : launch_fwd_ws_c<L, false>(a, ms, s);
   }
-  return launch_fwd_staged<L>(a, c, nch, s);
+  return launch_fwd_staged<L>(a, nch, s);
 }
 
 template <int L>
 int run_yz_fwd(const YZArgs& a, cudaStream_t s) {
-  const int c = single_component(a.need[0]);
-  if (a.nin != 1 || c < 0) return -2;
-  return launch_fwd_single<L>(a, c, (a.nzin + a.zchunk - 1) / a.zchunk, s);
+  return launch_fwd<L>(a, (a.nzin + a.zchunk - 1) / a.zchunk, s);
 }
 
 }  // namespace
@@ -936,11 +927,11 @@ int launch_yz_finish(int L, const YZArgs& a, int how, cudaStream_t s) {
   return -2;
 }
 
-bool zy_adj_ws_length(int L) {
+bool yz_ws_length(int L) {
   switch (L) {
 #define TM_CASE(LL) \
   case LL:          \
-    return ws_length<LL>();
+    return yz_ws_plan<LL>();
     TM_FOR_EACH_L(TM_CASE)
 #undef TM_CASE
   }

@@ -396,8 +396,9 @@ bool outputs_apart(const ZArgs& a) {
 template <int L>
 int run_length(const ZArgs& a, cudaStream_t s) {
   if (a.nin == 1) {
-    if (outputs_apart<L>(a)) return run_zn<L, 1, 1, true>(a, s);
-    return a.nout == 1 ? run_zn<L, 1, 1>(a, s) : run_zn<L, 1, 3>(a, s);
+    if constexpr (L == 512) return -2;  // k_z1m's
+    else if (outputs_apart<L>(a)) return run_zn<L, 1, 1, true>(a, s);
+    else return a.nout == 1 ? run_zn<L, 1, 1>(a, s) : run_zn<L, 1, 3>(a, s);
   }
   if (a.nin == 2) return run_zn<L, 2, 1>(a, s);
   return a.nout == 1 ? run_zn<L, 3, 1>(a, s) : run_zn<L, 3, 3>(a, s);
