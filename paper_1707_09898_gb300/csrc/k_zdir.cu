@@ -70,7 +70,11 @@ constexpr int ZP = 8;  // z parts per block, one warp each
 
 // Blocks per SM: more warps against more registers, hence loads, per thread. One plane at
 // 256^3, both directions: three and three 4 blocks 452 us, 5 470, 6 494, no bound 543; one to
-// one with tilted M0 no bound 119, 6 blocks 103.
+// one with tilted M0 no bound 119, 6 blocks 103. The variants with three inputs or outputs spill
+// (72 to 212 bytes with one plane at 6 blocks, 28 to 108 with two at 4); fewer blocks were better
+// on middle grids and worse on large ones. Evaluation with tilted M0 and three weights, us, one
+// plane with 6, 5 and 4 blocks: 128^3 104, 99, 113, 256^3 568, 578, 569; two planes with 4, 3 and 2:
+// 128^3 126, 117, 132, 256^3 619, 638, 698 (before this kernel 512 and 1305, 709 and 3000).
 __host__ __device__ constexpr int blocks_per_sm(int np, int mode) {
   return np == 1 ? (mode == FULL ? 4 : 6) : np == 2 ? 4 : np == 4 ? 2 : 1;
 }
@@ -83,8 +87,10 @@ __global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const
   constexpr int UNR = MODE == FULL ? 1 : 2;  // z per round of loads; the others measured slower
   __shared__ cx<float> red[ZP][NP][32];
   const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
-  const int kx = blockIdx.x * 32 + lane;
-  const bool valid = kx < a.P;
+  const bool valid = blockIdx.x * 32 + lane < a.P;
+  // Lanes past P load the last column and store nothing: with a test on every load of the inputs
+  // instead, one plane of three and three took 102 us at 128^3 (88 so), 473 at 256^3 (450).
+  const int kx = min(blockIdx.x * 32 + lane, a.P - 1);
   // zcol holds ky = 0, then the pairs (ky, Ly - ky), then Ly / 2
   const int c0 = COLS == 1 ? blockIdx.y : (blockIdx.y == 0 ? 0 : 2 * blockIdx.y - 1);
   const int nc = COLS == 1 || blockIdx.y == 0 || c0 == a.Ly - 1 ? 1 : 2;
@@ -186,7 +192,7 @@ __global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const
       for (int p = 0; p < NP; p++)
 #pragma unroll
         for (int i = 0; i < NI; i++)
-          x[c][p][i] = valid && p < a.nzin && (NI == 1 || i < a.nin)
+          x[c][p][i] = p < a.nzin && (NI == 1 || i < a.nin)
                            ? buf[a.in_slot[i] * a.cstride + (a.zin0 + p) * a.zstride + colo[c]]
                            : zero<float>();
     const int per = (a.nzout + ZP - 1) / ZP;
