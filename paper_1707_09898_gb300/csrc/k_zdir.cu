@@ -71,7 +71,7 @@ constexpr int ZP = 8;  // z parts per block, one warp each
 // Blocks per SM: more warps against more registers, hence loads, per thread. One plane at
 // 256^3, both directions: three and three 4 blocks 452 us, 5 470, 6 494, no bound 543; one to
 // one with tilted M0 no bound 119, 6 blocks 103. The variants with three inputs or outputs spill
-// (72 to 212 bytes with one plane at 6 blocks, 28 to 108 with two at 4); fewer blocks were better
+// (72 to 212 bytes with one plane at 6 blocks, 28 to 120 with two at 4); fewer blocks were better
 // on middle grids and worse on large ones. Evaluation with tilted M0 and three weights, us, one
 // plane with 6, 5 and 4 blocks: 128^3 104, 99, 113, 256^3 568, 578, 569; two planes with 4, 3 and 2:
 // 128^3 126, 117, 132, 256^3 619, 638, 698 (before this kernel 512 and 1305, 709 and 3000).
@@ -80,17 +80,21 @@ __host__ __device__ constexpr int blocks_per_sm(int np, int mode) {
 }
 
 // NP: planes on the short side (at most). COLS: columns per thread (ky, Ly - ky).
-// NK: inputs (ONE_OUT), outputs (ONE_IN) held: 1 or 3.
-template <int NP, int COLS, int MODE, int NK>
+// NK: inputs (ONE_OUT), outputs (ONE_IN) held: 1 or 3. SHARED: few inputs, some of whose planes are
+// also output planes (a target inside the design). Inputs and outputs share a slot, and such a
+// plane belongs to one warp's z range while every warp reads it, so no warp may store before all
+// have their inputs. (Few outputs are stored behind a barrier anyway.) An instantiation of its own:
+// in one kernel for both, the barrier made the compiler order the other direction's loads
+// differently, and one plane of three and three took 100 us both ways at 128^3 (88 so), 467 at
+// 256^3 (449).
+template <int NP, int COLS, int MODE, int NK, bool SHARED>
 __global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const __grid_constant__ ZDirArgs a) {
   constexpr int NI = MODE == ONE_IN ? 1 : NK, NO = MODE == ONE_OUT ? 1 : NK;
   constexpr int UNR = MODE == FULL ? 1 : 2;  // z per round of loads; the others measured slower
   __shared__ cx<float> red[ZP][NP][32];
   const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
   const bool valid = blockIdx.x * 32 + lane < a.P;
-  // Lanes past P load the last column and store nothing: with a test on every load of the inputs
-  // instead, one plane of three and three took 102 us at 128^3 (88 so), 473 at 256^3 (450).
-  const int kx = min(blockIdx.x * 32 + lane, a.P - 1);
+  const int kx = SHARED ? min(blockIdx.x * 32 + lane, a.P - 1) : blockIdx.x * 32 + lane;  // SHARED: lanes past P load it
   // zcol holds ky = 0, then the pairs (ky, Ly - ky), then Ly / 2
   const int c0 = COLS == 1 ? blockIdx.y : (blockIdx.y == 0 ? 0 : 2 * blockIdx.y - 1);
   const int nc = COLS == 1 || blockIdx.y == 0 || c0 == a.Ly - 1 ? 1 : 2;
@@ -185,6 +189,7 @@ __global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const
         }
       }
   } else {  // few inputs: keep them, stream the outputs
+    if (!SHARED && !valid) return;
     cx<float> x[COLS][NP][NI];
 #pragma unroll
     for (int c = 0; c < COLS; c++)
@@ -197,10 +202,7 @@ __global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const
                            : zero<float>();
     const int per = (a.nzout + ZP - 1) / ZP;
     const int z0 = a.zout0 + part * per, z1 = min(z0 + per, a.zout0 + a.nzout);
-    // Inputs and outputs may share a slot, and an input plane that is also an output plane (a
-    // target inside the design) belongs to one warp's z range while every warp reads it: no
-    // warp stores before all have their inputs.
-    __syncthreads();
+    if (SHARED) __syncthreads();
     if (!valid || z0 >= z1) return;
     Row r[NP];
 #pragma unroll
@@ -230,7 +232,9 @@ __global__ void __launch_bounds__(32 * ZP, blocks_per_sm(NP, MODE)) k_zdir(const
 template <int NP, int COLS, int MODE, int NK>
 int run_zdir(const ZDirArgs& a, cudaStream_t s) {
   const dim3 grid((a.P + 31) / 32, COLS == 1 ? a.Ly : a.Ly / 2 + 1);
-  return launch_k(k_zdir<NP, COLS, MODE, NK>, grid, dim3(32 * ZP), 0, s, a.pdl != 0, a) == cudaSuccess ? 0 : -1;
+  const bool shared = a.nzout > a.nzin && a.zin0 < a.zout0 + a.nzout && a.zout0 < a.zin0 + a.nzin;
+  auto kernel = shared ? k_zdir<NP, COLS, MODE, NK, true> : k_zdir<NP, COLS, MODE, NK, false>;
+  return launch_k(kernel, grid, dim3(32 * ZP), 0, s, a.pdl != 0, a) == cudaSuccess ? 0 : -1;
 }
 
 template <int NP, int COLS>
