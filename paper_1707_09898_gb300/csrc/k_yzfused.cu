@@ -207,7 +207,8 @@ __global__ void __launch_bounds__(NTF, 1) k_yz_fwd_staged(YZArgs a) {
 // The target plane after k_yz_fwd_staged: block cb adds the partials of its 16 lines over the z
 // chunks in order, straight into the first stage of their inverse y transform, and writes the
 // rows y < n_in of A (the sums and the transform were two launches, 6.3 + 2.9 us at L = 128 with
-// 22 chunks, this 6.6).
+// 22 chunks, this 6.6; at L = 256, P / 16 = 9 blocks and 16 chunks, 4.4 + 3.5 and 8.5, which the
+// launch less makes up for).
 template <int L>
 __global__ void __launch_bounds__(kNT) k_yz_finish_chunks(YZArgs a, int nch) {
   constexpr int S = plan_stages(L);

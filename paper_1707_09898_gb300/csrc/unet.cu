@@ -257,32 +257,6 @@ int launch_conv_tc(const void* src, const bf16* Wc, const float* bias, void* dst
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -4;
 }
 
-// Halo-tile implicit GEMM for grids whose rows hold W = 8, 16, 32 or 64 voxels (128 % W ==
-// 0). A tile is TZ planes of RY = 128 / W rows of one batch item: TZ MMA tiles of M = 128, the
-// RY rows of plane z0 + m in (y, x) order, one tensor-memory lane per voxel. A stage holds the
-// (TZ + 2) x (RY + 2) rows around a tile for 16 channels of the reduced dimension: MODE 0 as one
-// box copy brings them (32-byte rows, 32-byte swizzle, zero outside the grid), MODE 1 in the
-// K-major core-matrix layout [channel half][z][y][x][8 channels], the float32 output gradient
-// rounded to bfloat16 by the staging warps.
-// The three taps of a row, dx = -1, 0, +1, are columns of one MMA (N = 3 NO): the A operand of
-// a (dz, dy) pair is the staged rows from (m + dz + 1, dy + 1) on, unshifted, and the product
-// with W(dz, dy, dx) is accumulated per dx; the epilogue adds the three, each taken from the
-// lane one voxel to its side (warp shuffles, and shared memory between the two warps of a
-// 64-voxel row; a voxel past the row's end is the zero padding). So 9 MMAs per stage and M
-// tile instead of 27, and no dx-shifted copies of the rows: an MMA of so few columns is bound
-// by reading A from shared memory (4 KB for M = 128, K = 16), and the copies were two thirds
-// of the staging.
-// One persistent block per SM, its warps specialized: staging (one thread for the box copies,
-// or four groups of two warps, a buffer each), one thread per M tile that issues the MMAs, one
-// that copies weights, and groups of four warps that read alternate accumulators (a ring in
-// tensor memory) and write the output, which for MODE 1 is one bulk copy per M tile; mbarriers
-// between them. The packed weights stay in shared memory where they fit, otherwise each stage
-// brings its chunk's.
-// Measured, 64^3 x 2: forward 48 -> 16 channels 139 -> 33 us, of which the MMAs' operand reads
-// are 16 (44 cycles for M = 128, N = 48); data gradient 16 -> 48 113 -> 56 us, most of it the
-// epilogue's instructions (shuffles and sums of three arrays). Before: one block per two tiles, three shifted copies, 27 MMAs a chunk
-// and nothing overlapped inside a block. On the way: 9 MMAs without the pipeline 88 and 139,
-// rows staged by threads in MODE 0 59, 54 weight copies a chunk instead of one box 39.
 // compile-time loop: f(std::integral_constant<int, i>) for i in [B, E)
 template <int B, int E, class F>
 __device__ __forceinline__ void static_for(F&& f) {
@@ -330,6 +304,37 @@ __device__ __forceinline__ void stage_halo_finish(unsigned char* As) {
   }
 }
 
+// Halo-tile implicit GEMM for grids whose rows hold W = 8, 16, 32 or 64 voxels (128 % W ==
+// 0). A tile is TZ planes of RY = 128 / W rows of one batch item: TZ MMA tiles of M = 128, the
+// RY rows of plane z0 + m in (y, x) order, one tensor-memory lane per voxel. A stage holds the
+// (TZ + 2) x (RY + 2) rows around a tile for 16 channels of the reduced dimension: MODE 0 as one
+// box copy brings them (32-byte rows, 32-byte swizzle, zero outside the grid), MODE 1 in the
+// K-major core-matrix layout [channel half][z][y][x][8 channels], the float32 output gradient
+// rounded to bfloat16 by the staging warps.
+// The three taps of a row, dx = -1, 0, +1, are columns of one MMA (N = 3 NO): the A operand of
+// a (dz, dy) pair is the staged rows from (m + dz + 1, dy + 1) on, unshifted, and the product
+// with W(dz, dy, dx) is accumulated per dx; the epilogue adds the three, each taken from the
+// lane one voxel to its side (warp shuffles, and shared memory between the two warps of a
+// 64-voxel row; a voxel past the row's end is the zero padding). So 9 MMAs per stage and M
+// tile instead of 27, and no dx-shifted copies of the rows: an MMA of so few columns is bound
+// by reading A from shared memory (4 KB for M = 128, K = 16), and the copies were two thirds
+// of the staging.
+// One persistent block per SM, its warps specialized: staging (one thread for the box copies,
+// or four groups of two warps, a buffer each), one thread per M tile that issues the MMAs, one
+// that copies weights, and groups of four warps that read alternate accumulators (a ring in
+// tensor memory) and write the output, which for MODE 1 is one bulk copy per M tile; mbarriers
+// between them. The packed weights stay in shared memory where they fit, otherwise each stage
+// brings its chunk's.
+// Measured, 64^3 x 2: forward 48 -> 16 channels 139 -> 33 us, of which the MMAs' operand reads
+// are 16 (44 cycles for M = 128, N = 48); data gradient 16 -> 48 113 -> 56 us. What bounds the
+// latter is the path through L1 and shared memory, 78% busy while it runs (ncu; issue 36%, tensor
+// pipe 18%, DRAM 74 MB): the float32 rows read and rounded, the operands of the MMAs and the
+// output's staging all take it. Before: one block per two tiles, three shifted copies, 27 MMAs a
+// chunk and nothing overlapped inside a block. On the way: 9 MMAs without the pipeline 88 and 139,
+// rows staged by threads in MODE 0 59, 54 weight copies a chunk instead of one box 39.
+// Two planes to a tile of 32-voxel rows in MODE 1 spill 328 bytes a thread; the layers that take
+// the form are still ahead of the kernel before (32^3 x 4, 16 -> 16 channels 18.4 -> 14.4 us, 32 -> 32
+// 36.9 -> 26.7).
 template <int MODE, int W, int TZ, int NO>
 struct Halo {
   static constexpr int RY = 128 / W, ROWS = (TZ + 2) * (RY + 2);
@@ -348,15 +353,17 @@ struct Halo {
 };
 constexpr int kHaloStages = 4;
 constexpr size_t kHaloTail = 8 * 64 * 4 + 64 * 4 + (2 * kHaloStages + 2 * 4 + 1) * 8 + 16;
-// shared memory with ns stages: 256 bytes of slack to align the staged rows
+// whether the output goes through shared memory (where a tile's rows are whole, see OBYTES)
 template <int MODE, int NO>
 __host__ __device__ constexpr bool halo_staged_out() {
   return MODE == 1;
 }
+// shared memory with ns stages: 256 bytes of slack to align the staged rows
 template <int MODE, int W, int TZ, int NO>
 constexpr size_t halo_smem(int ns, bool resident, int nk) {
   using HT = Halo<MODE, W, TZ, NO>;
-  return 256 + (halo_staged_out<MODE, NO>() ? (size_t)HT::EG * HT::OBYTES : 0) + (size_t)ns * (HT::ABYTES + (resident ? 0 : HT::BB)) + (resident ? (size_t)nk * HT::BB : 0) + kHaloTail;
+  return 256 + (halo_staged_out<MODE, NO>() ? (size_t)HT::EG * HT::OBYTES : 0) +
+         (size_t)ns * (HT::ABYTES + (resident ? 0 : HT::BB)) + (resident ? (size_t)nk * HT::BB : 0) + kHaloTail;
 }
 // contiguous bulk copy shared -> global (16-byte aligned, size a multiple of 16), and the wait
 // until this thread's copies have read shared memory
@@ -1406,7 +1413,6 @@ __global__ void k_to_bf16(const float* x, bf16* y, long long n) {
   }
 }
 
-// the bias gradient: float32 sum over the voxels of the unrounded output gradient
 // The bias gradient db[c] = sum over the voxels of dout[v][c] (float32, unrounded), in a
 // fixed order: block b sums its range of voxels for every channel (consecutive threads on
 // consecutive channels, then voxels), k_db_final adds the block partials in block order.
